@@ -67,7 +67,10 @@ struct dsdna_ctx {
   GridBar* bar = nullptr; unsigned* err = nullptr; int64_t* step_d = nullptr; int* rebuild = nullptr;
   unsigned long long* nrebuild = nullptr;
   double* fout = nullptr; double* eout = nullptr; double* stage = nullptr;
-  double* obs_scratch = nullptr; double* obs_out = nullptr;
+  double* obs_scratch = nullptr; double* obs_part = nullptr; unsigned* obs_counter = nullptr;
+  double* obs_host = nullptr;    // results of the observable kernels, pinned host memory they write directly
+  double* obs_out = nullptr;     // its device address
+  int nsm = 0;
   int64_t* steps_left = nullptr; unsigned* iters = nullptr;
   unsigned long long* nlaunch = nullptr;   // engine launches made by step graphs
   int64_t host_launches = 0;               // engine launches queued directly by the host
@@ -139,6 +142,7 @@ static void free_all(dsdna_ctx* c) {
     else cudaFree(p);
   }
   c->bufs.clear();
+  if (c->obs_host) { cudaFreeHost(c->obs_host); c->obs_host = nullptr; }
 }
 
 // Philox4x32-10 (Salmon et al., SC'11) for the host-side initial velocities.
@@ -577,7 +581,11 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   ALLOC(fout, double, 6 * nn); ALLOC(eout, double, (size_t)c->n_mol * EOUT_STRIDE);
   ALLOC(stage, double, 12 * nn);
   ALLOC(obs_scratch, double, 3 * (size_t)(3 * (c->maxN + 4)) + (size_t)c->maxN + 4);   // curves + twist increments
-  ALLOC(obs_out, double, 8);
+  ALLOC(obs_part, double, obs_partials(c->maxN));
+  ALLOC(obs_counter, unsigned, 1);
+  if (cudaHostAlloc((void**)&c->obs_host, 8 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer((void**)&c->obs_out, c->obs_host, 0) != cudaSuccess)
+    return bad(fail(c, DSDNA_ENOMEM, "host allocation failed: observables"));
   ALLOC(steps_left, int64_t, 1);
   ALLOC(iters, unsigned, 4);
   ALLOC(nlaunch, unsigned long long, 1);
@@ -585,6 +593,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   // launch shape per mode (cooperative: every CTA resident)
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
+  c->nsm = nsm;
   for (int mode = 0; mode < 3; ++mode) {
     int bps = 0;
     const int m = mode | c->kernel_flags(mode);
@@ -656,7 +665,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
     return bad(fail(c, DSDNA_ECUDA, "topology upload"));
   if (cudaMemset(c->cnt, 0, sizeof(unsigned) * c->H_alloc) != cudaSuccess || cudaMemset(c->err, 0, 16) != cudaSuccess ||
       cudaMemset(c->step_d, 0, 8) != cudaSuccess || cudaMemset(c->nrebuild, 0, 8) != cudaSuccess ||
-      cudaMemset(c->nlaunch, 0, 8) != cudaSuccess ||
+      cudaMemset(c->nlaunch, 0, 8) != cudaSuccess || cudaMemset(c->obs_counter, 0, 4) != cudaSuccess ||
       cudaMemset(c->bar, 0, sizeof(GridBar)) != cudaSuccess || cudaMemset(c->ncnt, 0, sizeof(int) * ns) != cudaSuccess ||
       cudaMemset(c->Om, 0, (f64 ? 8 : 4) * 3 * ns) != cudaSuccess || cudaMemset(c->V, 0, 24 * ns) != cudaSuccess ||
       cudaMemset(c->X, 0, (f64 ? 48 : 24) * ns) != cudaSuccess || cudaMemset(c->kref, 0, 12 * ns) != cudaSuccess ||
@@ -974,12 +983,8 @@ extern "C" int dsdna_energy_virial(dsdna_ctx* c, int mol, double energy[DSDNA_NT
   return DSDNA_OK;
 }
 
-extern "C" int dsdna_observables(dsdna_ctx* c, int mol, unsigned flags, dsdna_obs* out) {
-  if (!c || !out) return DSDNA_EINVAL;
-  if (c->poisoned) return fail(c, DSDNA_ESTATE, "context poisoned by an earlier error");
-  if (mol < 0 || mol >= c->n_mol) return fail(c, DSDNA_EINVAL, "molecule index out of range");
-  int rc = sync_check(c);
-  if (rc) return rc;
+// Arguments of the observable reductions of molecule mol.
+static ObsArgs obs_args(dsdna_ctx* c, int mol) {
   const int cur = (int)(c->step & 1);
   ObsArgs a{};
   a.n = c->ns;   // row stride of the [3][n] arrays
@@ -995,10 +1000,24 @@ extern "C" int dsdna_observables(dsdna_ctx* c, int mol, unsigned flags, dsdna_ob
   a.ca = a.mid + 3 * (size_t)(c->maxN + 4);
   a.cb = a.ca + 3 * (size_t)(c->maxN + 4);
   a.out = c->obs_out;
-  CK(obs_launch(a, flags, c->st), "observables");
-  double o[8];
-  CK(cudaMemcpyAsync(o, c->obs_out, sizeof(o), cudaMemcpyDeviceToHost, c->st), "read observables");
+  a.part = c->obs_part;
+  a.counter = c->obs_counter;
+  a.err = c->err;
+  return a;
+}
+
+// The kernels write the results and the engine's error word straight to
+// pinned host memory, so one wait completes the call.
+extern "C" int dsdna_observables(dsdna_ctx* c, int mol, unsigned flags, dsdna_obs* out) {
+  if (!c || !out) return DSDNA_EINVAL;
+  if (c->poisoned) return fail(c, DSDNA_ESTATE, "context poisoned by an earlier error");
+  if (mol < 0 || mol >= c->n_mol) return fail(c, DSDNA_EINVAL, "molecule index out of range");
+  const ObsArgs a = obs_args(c, mol);
+  CK(obs_launch(a, flags, c->nsm, c->st), "observables");
   CK(cudaStreamSynchronize(c->st), "observables sync");
+  const double* o = c->obs_host;
+  const int rc = map_err(c, (unsigned)o[7]);
+  if (rc) return rc;
   out->rz = o[0];
   out->denat = o[1] / (double)a.N;
   out->tw = o[2];
@@ -1021,23 +1040,9 @@ extern "C" int dsdna_profiles(dsdna_ctx* c, int mol, double* centre, double* twi
   if (rc) return rc;
   const int N = c->n_bp[mol];
   const int ninc = c->circular[mol] ? N : std::max(0, N - 2);
-  const int cur = (int)(c->step & 1);
-  ObsArgs a{};
-  a.n = c->ns;
-  a.X = c->fp64() ? c->X + (size_t)cur * 3 * c->ns : c->X;
-  a.uf = c->fp64() ? nullptr : c->U + (size_t)cur * c->ns;
-  a.ud = c->fp64() ? c->ud + (size_t)cur * 3 * c->ns : nullptr;
-  a.g0 = 2 * c->off[mol];
-  a.N = N;
-  a.ring = c->circular[mol];
-  a.h = 0.5 * c->p.ell;
-  a.rc2 = c->p.rc_hb * c->p.rc_hb;
-  a.mid = c->obs_scratch;
-  a.ca = a.mid + 3 * (size_t)(c->maxN + 4);
-  a.cb = a.ca + 3 * (size_t)(c->maxN + 4);
-  a.out = c->obs_out;
+  ObsArgs a = obs_args(c, mol);
   a.inc = c->obs_scratch + 9 * (size_t)(c->maxN + 4);   // beyond the three curves
-  CK(obs_launch(a, DSDNA_OBS_TW, c->st), "profiles");
+  CK(obs_launch(a, DSDNA_OBS_TW, c->nsm, c->st), "profiles");
   if (centre) CK(cudaMemcpyAsync(centre, a.mid, sizeof(double) * 3 * (size_t)N, cudaMemcpyDeviceToHost, c->st), "read centre");
   if (twist && ninc) CK(cudaMemcpyAsync(twist, a.inc, sizeof(double) * (size_t)ninc, cudaMemcpyDeviceToHost, c->st), "read twist");
   CK(cudaStreamSynchronize(c->st), "profiles sync");

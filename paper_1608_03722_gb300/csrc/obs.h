@@ -18,10 +18,17 @@ struct ObsArgs {
   double* mid;        // [3*N] scratch
   double* ca;         // [3*(N+4)] scratch: closed curve of strand A
   double* cb;         // [3*(N+4)] scratch: closed curve of strand B
-  double* out;        // [8]: rz, broken count, tw, -, lk
+  double* out;        // [8]: rz, broken count, tw, -, lk, -, -, error word of the engine (host memory, mapped)
+  double* part;       // [obs_partials(N)] sums of the blocks
+  unsigned* counter;  // blocks done (zero between launches)
+  const unsigned* err;   // the engine's error word
   double* inc;        // [N-2] (ring: [N]) twist increments in turns, or nullptr
 };
 
-cudaError_t obs_launch(const ObsArgs& a, unsigned flags, cudaStream_t st);
+constexpr int OBS_MAX_GRID = 1024;   // blocks of the linking-number kernel
+
+// Doubles of block sums that a molecule of at most maxN base pairs needs.
+int64_t obs_partials(int maxN);
+cudaError_t obs_launch(const ObsArgs& a, unsigned flags, int nsm, cudaStream_t st);
 
 }  // namespace dsdna
