@@ -4,11 +4,11 @@
 //
 // Weights are kept as FP32 masters and BF16 copies.  The contractions run on
 // the fifth-generation tensor cores: tcgen05.mma (kind::f16, BF16 operands in
-// shared memory, FP32 accumulators in tensor memory), one 128-row batch tile
+// shared memory, FP32 accumulators in tensor memory), one 32-row batch tile
 // per CTA, issued by one thread and completed through an mbarrier; epilogues
 // read the accumulators with tcgen05.ld.  Small dimensions (4 inputs, 3
 // outputs) are zero-padded to the MMA shape; the 3- and 4-wide weight
-// gradients are FP32 warp reductions.  The forward pass keeps the
+// gradients are FP32 sums over the tile's rows.  The forward pass keeps the
 // pre-activations for the backward pass; the backward pass forms the mean
 // squared error on normalised targets and accumulates the weight gradients in
 // FP32; Adam updates the masters and refreshes the BF16 copies.
@@ -114,11 +114,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 4 FP32 accumulator columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 constexpr int TC_COLS = 128;   // TMEM columns per CTA (two 64-column accumulators)
 
 // Warp 0 allocates TC_COLS TMEM columns; the base address lands in *slot.
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot) {
   if ((threadIdx.x >> 5) == 0) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
                  "r"(TC_COLS)
                  : "memory");
@@ -132,6 +143,13 @@ __device__ __forceinline__ void tmem_free(uint32_t taddr) {
 
 __device__ __forceinline__ void put_bf16(unsigned char* base, uint32_t off, float v) {
   *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(v);
+}
+__device__ __forceinline__ uint2 pack4_bf16(const float* v) {
+  uint2 p;
+  __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+  p.x = *reinterpret_cast<unsigned*>(&a);
+  p.y = *reinterpret_cast<unsigned*>(&b);
+  return p;
 }
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
@@ -155,18 +173,23 @@ struct MlpDev {
 };
 
 // ---------------------------------------------------------------- forward
-// One CTA of 128 threads per 128-row batch tile; thread t owns row t, which
-// is also TMEM lane t of every accumulator (M = 128, warp w reads lanes
-// 32w..32w+31).  Every contraction is a tcgen05.mma (BF16 operands from shared
-// memory, FP32 accumulator in TMEM) issued by thread 0 and completed through
-// an mbarrier; epilogues read the accumulators with tcgen05.ld.
-constexpr int TC_ROWS = 128;
+// One CTA of 16 warps per tile of 32 batch rows.  Every contraction is a
+// tcgen05.mma (BF16 operands from shared memory, FP32 accumulator in TMEM, M =
+// 128) issued by thread 0 and completed through an mbarrier.  The network is
+// small, so a pass is a chain of latencies -- operand loads, three MMAs, an
+// epilogue of biases and GELUs after each -- and what it can be cut by is the
+// epilogue's serial work: each of the 32 rows stands in the A operand four
+// times, at rows r + 32 p, so that the warps of every TMEM sub-partition (warp
+// w reads lanes 32 (w mod 4) ...) find all rows, and a thread takes 4 of the 64
+// columns of one row.  32-row tiles also spread a minibatch of 256 over eight
+// SMs.  256 or 2000 rows: 25 us with 128-row tiles of 128 threads (64 columns
+// per thread, weights staged two bytes at a time), 5.0 us now.
+constexpr int TC_ROWS = 32, TC_REP = 4, TC_THREADS = 512;
 constexpr size_t F_AX = 0;                          // A  Xn  [128 x 16] (K = 4 padded)
 constexpr size_t F_BW1 = F_AX + 128 * 16 * 2;       // B  W1  [64 x 16]
-constexpr size_t F_AH1 = F_BW1 + 64 * 16 * 2;       // A  H1  [128 x 64]
-constexpr size_t F_BW2 = F_AH1 + 128 * 64 * 2;      // B  W2  [64 x 64]
-constexpr size_t F_AH2 = F_BW2 + 64 * 64 * 2;       // A  H2  [128 x 64]
-constexpr size_t F_BW3 = F_AH2 + 128 * 64 * 2;      // B  W3  [16 x 64] (rows 3..15 zero)
+constexpr size_t F_AH = F_BW1 + 64 * 16 * 2;        // A  H1, then H2  [128 x 64]
+constexpr size_t F_BW2 = F_AH + 128 * 64 * 2;       // B  W2  [64 x 64]
+constexpr size_t F_BW3 = F_BW2 + 64 * 64 * 2;       // B  W3  [16 x 64] (rows 3..15 zero)
 constexpr size_t F_BYTES = F_BW3 + 16 * 64 * 2;
 
 // Issue (thread 0) and complete (every thread) one batch of MMAs; ok turns
@@ -189,83 +212,98 @@ struct TcSync {
   }
 };
 
-__global__ void __launch_bounds__(TC_ROWS) k_mlp_forward(MlpDev m, const float* X, int B, float* Y) {
+// This thread's share of an accumulator: batch row `lane` of the tile, columns
+// c0 .. c0 + 3 (TMEM lane 32 (warp mod 4) + lane holds that row's copy).
+struct Share {
+  int lane, c0;
+  uint32_t tlane;
+  __device__ Share() {
+    const int w = threadIdx.x >> 5;
+    lane = threadIdx.x & 31;
+    c0 = 4 * (4 * (w & 3) + (w >> 2));
+    tlane = (uint32_t)(32 * (w & 3)) << 16;
+  }
+  // four BF16 values of this row and columns into every copy of the row of a
+  // 64-column A operand
+  __device__ void put_a64(unsigned char* base, const float* v) const {
+    const uint2 q = pack4_bf16(v);
+#pragma unroll
+    for (int p = 0; p < TC_REP; ++p) *reinterpret_cast<uint2*>(base + cm_off(lane + 32 * p, c0, 64)) = q;
+  }
+};
+
+__global__ void __launch_bounds__(TC_THREADS) k_mlp_forward(MlpDev m, const float* X, int B, float* Y) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tslot;
-  const int t = threadIdx.x, warp = t >> 5;
-  const int row = blockIdx.x * TC_ROWS + t;
+  const int t = threadIdx.x;
+  const Share sh;
+  const int row = blockIdx.x * TC_ROWS + sh.lane;
   const bool live = row < B;
-  const __nv_bfloat16 zero = __float2bfloat16_rn(0.0f);
-  for (int i = t; i < 64 * 16; i += TC_ROWS) {
-    const int n = i / 16, k = i % 16;
-    *reinterpret_cast<__nv_bfloat16*>(sm + F_BW1 + cm_off(n, k, 16)) = k < NI ? m.Pb[OW1 + n * NI + k] : zero;
-  }
-  for (int i = t; i < 64 * 64; i += TC_ROWS) {
-    const int n = i / 64, k = i % 64;
-    *reinterpret_cast<__nv_bfloat16*>(sm + F_BW2 + cm_off(n, k, 64)) = m.Pb[OW2 + n * NH + k];
-  }
-  for (int i = t; i < 16 * 64; i += TC_ROWS) {
-    const int n = i / 64, k = i % 64;
-    *reinterpret_cast<__nv_bfloat16*>(sm + F_BW3 + cm_off(n, k, 64)) = n < NO ? m.Pb[OW3 + n * NH + k] : zero;
-  }
-  for (int k = 0; k < 16; ++k) {
-    float v = 0.0f;
-    if (live && k < NI) {
-      v = (X[(size_t)row * NI + k] - m.norm.in_mean[k]) / m.norm.in_scale[k];
-      m.Xn[(size_t)row * NI + k] = v;
-    }
-    put_bf16(sm + F_AX, cm_off(t, k, 16), v);
-  }
+  const uint4 none = make_uint4(0u, 0u, 0u, 0u);
   if (t == 0) mbar_init(smem_u32(&mbar), 1);
   tmem_alloc(&tslot);
+  {   // weights, eight BF16 values at a time (rows of Pb start on 16-byte boundaries)
+    const int n = t >> 3, kc = (t & 7) * 8;
+    *reinterpret_cast<uint4*>(sm + F_BW2 + cm_off(n, kc, 64)) = *reinterpret_cast<const uint4*>(m.Pb + OW2 + n * NH + kc);
+  }
+  if (t < 128) {   // inputs: row t mod 32, copy t / 32
+    float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (live) {
+      for (int k = 0; k < NI; ++k) v[k] = (X[(size_t)row * NI + k] - m.norm.in_mean[k]) / m.norm.in_scale[k];
+      if (t < 32) *reinterpret_cast<float4*>(m.Xn + (size_t)row * NI) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    const uint2 q = pack4_bf16(v);
+    *reinterpret_cast<uint4*>(sm + F_AX + cm_off(t, 0, 16)) = make_uint4(q.x, q.y, 0u, 0u);
+    *reinterpret_cast<uint4*>(sm + F_AX + cm_off(t, 8, 16)) = none;
+  } else if (t < 192) {
+    const int n = t - 128;
+    const uint2 q = *reinterpret_cast<const uint2*>(m.Pb + OW1 + n * NI);
+    *reinterpret_cast<uint4*>(sm + F_BW1 + cm_off(n, 0, 16)) = make_uint4(q.x, q.y, 0u, 0u);
+    *reinterpret_cast<uint4*>(sm + F_BW1 + cm_off(n, 8, 16)) = none;
+  } else if (t < 320) {
+    const int n = (t - 192) >> 3, kc = (t & 7) * 8;
+    *reinterpret_cast<uint4*>(sm + F_BW3 + cm_off(n, kc, 64)) =
+        n < NO ? *reinterpret_cast<const uint4*>(m.Pb + OW3 + n * NH + kc) : none;
+  }
+  const float4 b1 = *reinterpret_cast<const float4*>(m.P + OB1 + sh.c0), b2 = *reinterpret_cast<const float4*>(m.P + OB2 + sh.c0);
   TcSync sy{smem_u32(&mbar), 0u, true};
   sy.start();
   const uint32_t tmem = tslot;
-  const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+  // GELU of this thread's accumulator columns plus bias -> Z and the next A operand
+  auto epilogue = [&](uint32_t col, float4 b, float* Z) {
+    float v[4], h[4];
+    tmem_ld4(tmem + sh.tlane + col + sh.c0, v);
+    v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
+    if (live) *reinterpret_cast<float4*>(Z + (size_t)row * NH + sh.c0) = make_float4(v[0], v[1], v[2], v[3]);
+    for (int j = 0; j < 4; ++j) h[j] = gelu(v[j]);
+    sh.put_a64(sm + F_AH, h);
+  };
   // layer 1: Z1 = Xn W1^T + b1 -> TMEM columns 0..63
   if (t == 0) {
     umma_128xN(tmem, smem_u32(sm + F_AX), smem_u32(sm + F_BW1), 16, 64, false);
     umma_commit(sy.mbar);
   }
   sy.finish();
-  if (sy.ok)
-    for (int c0 = 0; c0 < NH; c0 += 16) {
-      float v[16];
-      tmem_ld16(lanes + c0, v);
-      for (int j = 0; j < 16; ++j) {
-        const float z = v[j] + m.P[OB1 + c0 + j];
-        if (live) m.Z1[(size_t)row * NH + c0 + j] = z;
-        put_bf16(sm + F_AH1, cm_off(t, c0 + j, 64), gelu(z));
-      }
-    }
+  if (sy.ok) epilogue(0, b1, m.Z1);
   // layer 2: Z2 = H1 W2^T + b2 -> columns 64..127
   sy.start();
   if (t == 0 && sy.ok) {
-    umma_128xN(tmem + 64, smem_u32(sm + F_AH1), smem_u32(sm + F_BW2), 64, 64, false);
+    umma_128xN(tmem + 64, smem_u32(sm + F_AH), smem_u32(sm + F_BW2), 64, 64, false);
     umma_commit(sy.mbar);
   }
   sy.finish();
-  if (sy.ok)
-    for (int c0 = 0; c0 < NH; c0 += 16) {
-      float v[16];
-      tmem_ld16(lanes + 64 + c0, v);
-      for (int j = 0; j < 16; ++j) {
-        const float z = v[j] + m.P[OB2 + c0 + j];
-        if (live) m.Z2[(size_t)row * NH + c0 + j] = z;
-        put_bf16(sm + F_AH2, cm_off(t, c0 + j, 64), gelu(z));
-      }
-    }
-  // layer 3: Y = H2 W3^T + b3 -> columns 0..15 (N = 3 padded to 16)
+  if (sy.ok) epilogue(64, b2, m.Z2);
+  // layer 3: Y = H2 W3^T + b3 -> columns 0..15 (N = 3 padded to 16), read by one warp
   sy.start();
   if (t == 0 && sy.ok) {
-    umma_128xN(tmem, smem_u32(sm + F_AH2), smem_u32(sm + F_BW3), 64, 16, false);
+    umma_128xN(tmem, smem_u32(sm + F_AH), smem_u32(sm + F_BW3), 64, 16, false);
     umma_commit(sy.mbar);
   }
   sy.finish();
-  if (sy.ok) {
-    float v[16];
-    tmem_ld16(lanes, v);
+  if (sy.ok && t < 32) {
+    float v[4];
+    tmem_ld4(tmem, v);
     if (live)
       for (int c = 0; c < NO; ++c) {
         const float yn = v[c] + m.P[OB3 + c];
@@ -282,128 +320,151 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_forward(MlpDev m, const float* 
 
 // ---------------------------------------------------------------- backward
 // Mean squared error over the B x 3 normalised outputs and its gradient, one
-// 128-row tile per CTA.  dH2 = dY W3, dH1 = dZ2 W2 and dW2 = dZ2^T H1 (K = the
-// tile's 128 rows; M = 64 output rows padded to 128) run on the tensor cores;
-// the 3- and 4-wide gradients dW3 = dY^T H2, dW1 = dZ1^T Xn and the biases are
-// FP32 warp reductions.  Weight gradients are added to G with atomics.
-constexpr size_t B_ADY = 0;                          // A  dY    [128 x 16] (K = 3 padded)
-constexpr size_t B_BW3T = B_ADY + 128 * 16 * 2;      // B  W3^T  [64 x 16]: (f, o) = W3[o][f]
-constexpr size_t B_ADZ2 = B_BW3T + 64 * 16 * 2;      // A  dZ2   [128 x 64]
-constexpr size_t B_BW2T = B_ADZ2 + 128 * 64 * 2;     // B  W2^T  [64 x 64]: (i, o) = W2[o][i]
-constexpr size_t B_ADZ2T = B_BW2T + 64 * 64 * 2;     // A  dZ2^T [128 x 128]: (o, b) = dZ2[b][o]; rows 64.. zero
-constexpr size_t B_BH1T = B_ADZ2T + 128 * 128 * 2;   // B  H1^T  [64 x 128]: (i, b) = H1[b][i]
-constexpr size_t B_BYTES = B_BH1T + 64 * 128 * 2;
+// 32-row tile per CTA, rows and columns shared out as in the forward pass.
+// dH2 = dY W3, dH1 = dZ2 W2 and dW2 = dZ2^T H1 (K = the tile's 32 rows; M = 64
+// output rows of 128, the rest unread) run on the tensor cores; the 3- and
+// 4-wide gradients dW3 = dY^T H2, dW1 = dZ1^T Xn and the biases are FP32 sums
+// over the tile's rows, one thread per gradient reading columns of FP32 tiles
+// in shared memory, in the shadow of the MMAs where it can be.  (As warp sums,
+// 580 of them one after the other in each of four warps, they made a pass over
+// 256 rows 95 us; now 7.4 us.)  Weight gradients are added to G with atomics.
+constexpr int SROW = NH + 1;                          // padded row of an FP32 tile
+constexpr size_t B_ADY = 0;                           // A  dY    [128 x 16] (K = 3 padded)
+constexpr size_t B_BW3T = B_ADY + 128 * 16 * 2;       // B  W3^T  [64 x 16]: (f, o) = W3[o][f]
+constexpr size_t B_ADZ2 = B_BW3T + 64 * 16 * 2;       // A  dZ2   [128 x 64]
+constexpr size_t B_BW2T = B_ADZ2 + 128 * 64 * 2;      // B  W2^T  [64 x 64]: (i, o) = W2[o][i]
+constexpr size_t B_ADZ2T = B_BW2T + 64 * 64 * 2;      // A  dZ2^T [128 x 32]: (o, b) = dZ2[b][o]; rows 64.. not set
+constexpr size_t B_BH1T = B_ADZ2T + 128 * 32 * 2;     // B  H1^T  [64 x 32]: (i, b) = H1[b][i]
+constexpr size_t B_S2 = B_BH1T + 64 * 32 * 2;         // FP32 [32][SROW]  dZ2
+constexpr size_t B_S1 = B_S2 + 32 * SROW * 4;         // FP32 [32][SROW]  H2, then dZ1
+constexpr size_t B_BYTES = B_S1 + 32 * SROW * 4;
 
 __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-__global__ void __launch_bounds__(TC_ROWS) k_mlp_backward(MlpDev m, const float* T, int B) {
+// Sum over the tile's rows of x[row * sx] * y[row * sy] (y null: of x alone).
+__device__ __forceinline__ float row_sum(const float* x, int sx, const float* y, int sy) {
+  float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int r = 0; r < TC_ROWS; ++r) a[r & 3] += y ? x[r * sx] * y[r * sy] : x[r * sx];
+  return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+__device__ __forceinline__ void red4(float* p, const float* v) {   // p on a 16-byte boundary
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+               : "memory");
+}
+
+__global__ void __launch_bounds__(TC_THREADS) k_mlp_backward(MlpDev m, const float* T, int B) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tslot;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int row = blockIdx.x * TC_ROWS + t;
+  __shared__ float s_dy[TC_ROWS][NO], s_xn[TC_ROWS][NI];
+  const int t = threadIdx.x;
+  const Share sh;
+  const int lane = sh.lane, c0 = sh.c0;
+  const int row = blockIdx.x * TC_ROWS + lane;
   const bool live = row < B;
   const float inv = 1.0f / (float)(B * NO);
-  const __nv_bfloat16 zero = __float2bfloat16_rn(0.0f);
-  for (int i = t; i < 64 * 16; i += TC_ROWS) {
-    const int n = i / 16, k = i % 16;
-    *reinterpret_cast<__nv_bfloat16*>(sm + B_BW3T + cm_off(n, k, 16)) = k < NO ? m.Pb[OW3 + k * NH + n] : zero;
-  }
-  for (int i = t; i < 64 * 64; i += TC_ROWS) {
-    const int n = i / 64, k = i % 64;
-    *reinterpret_cast<__nv_bfloat16*>(sm + B_BW2T + cm_off(n, k, 64)) = m.Pb[OW2 + k * NH + n];
-  }
-  for (int i = t; i < 64 * 128 * 2 / 16; i += TC_ROWS)   // rows 64..127 of dZ2^T: the second half of the buffer
-    reinterpret_cast<uint4*>(sm + B_ADZ2T + 64 * 128 * 2)[i] = make_uint4(0u, 0u, 0u, 0u);
-  // dY of this row and the loss
-  float dy[NO], lsum = 0.0f;
-  for (int c = 0; c < NO; ++c) {
-    dy[c] = 0.0f;
-    if (live) {
-      const float tn = (T[(size_t)row * NO + c] - m.norm.out_mean[c]) / m.norm.out_scale[c];
-      const float e = m.Yn[(size_t)row * NO + c] - tn;
-      lsum += e * e;
-      dy[c] = 2.0f * e * inv;
-    }
-  }
-  for (int k = 0; k < 16; ++k) put_bf16(sm + B_ADY, cm_off(t, k, 16), k < NO ? dy[k] : 0.0f);
-  lsum = warp_sum(lsum);
-  if (lane == 0) atomicAdd(m.loss, lsum * inv);
-  // dW3 = dY^T H2 and db3 (CUDA cores); H1^T operand
-  for (int f = 0; f < NH; ++f) {
-    const float h2 = live ? gelu(m.Z2[(size_t)row * NH + f]) : 0.0f;
-    const float h1 = live ? gelu(m.Z1[(size_t)row * NH + f]) : 0.0f;
-    put_bf16(sm + B_BH1T, cm_off(f, t, 128), h1);
-    for (int o = 0; o < NO; ++o) {
-      const float g = warp_sum(dy[o] * h2);
-      if (lane == 0) atomicAdd(&m.G[OW3 + o * NH + f], g);
-    }
-  }
-  for (int o = 0; o < NO; ++o) {
-    const float g = warp_sum(dy[o]);
-    if (lane == 0) atomicAdd(&m.G[OB3 + o], g);
-  }
+  const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+  float* s1 = reinterpret_cast<float*>(sm + B_S1);
+  float* s2 = reinterpret_cast<float*>(sm + B_S2);
   if (t == 0) mbar_init(smem_u32(&mbar), 1);
   tmem_alloc(&tslot);
+  // this thread's pre-activations
+  const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const float4 q1 = live ? *reinterpret_cast<const float4*>(m.Z1 + (size_t)row * NH + c0) : zero4;
+  const float4 q2 = live ? *reinterpret_cast<const float4*>(m.Z2 + (size_t)row * NH + c0) : zero4;
+  const float z1[4] = {q1.x, q1.y, q1.z, q1.w}, z2[4] = {q2.x, q2.y, q2.z, q2.w};
+  {   // W2^T: eight rows o of one column i per thread
+    const int n = t & 63, kc = (t >> 6) * 8;
+    __align__(16) __nv_bfloat16 w[8];
+    for (int q = 0; q < 8; ++q) w[q] = m.Pb[OW2 + (kc + q) * NH + n];
+    *reinterpret_cast<uint4*>(sm + B_BW2T + cm_off(n, kc, 64)) = *reinterpret_cast<const uint4*>(w);
+  }
+  if (t < 128) {   // dY of row t mod 32 (copy t / 32) and, from the first copy, the loss
+    float dy[4] = {0.0f, 0.0f, 0.0f, 0.0f}, lsum = 0.0f;
+    for (int c = 0; c < NO; ++c) {
+      if (live) {
+        const float tn = (T[(size_t)row * NO + c] - m.norm.out_mean[c]) / m.norm.out_scale[c];
+        const float e = m.Yn[(size_t)row * NO + c] - tn;
+        lsum += e * e;
+        dy[c] = 2.0f * e * inv;
+      }
+    }
+    const uint2 q = pack4_bf16(dy);
+    *reinterpret_cast<uint4*>(sm + B_ADY + cm_off(t, 0, 16)) = make_uint4(q.x, q.y, 0u, 0u);
+    *reinterpret_cast<uint4*>(sm + B_ADY + cm_off(t, 8, 16)) = none;
+    if (t < 32) {
+      for (int c = 0; c < NO; ++c) s_dy[t][c] = dy[c];
+      for (int i = 0; i < NI; ++i) s_xn[t][i] = live ? m.Xn[(size_t)row * NI + i] : 0.0f;
+      lsum = warp_sum(lsum);
+      if (t == 0) atomicAdd(m.loss, lsum * inv);
+    }
+  } else if (t < 192) {   // W3^T
+    const int n = t - 128;
+    __align__(16) __nv_bfloat16 w[8];
+    for (int k = 0; k < 8; ++k) w[k] = k < NO ? m.Pb[OW3 + k * NH + n] : __float2bfloat16_rn(0.0f);
+    *reinterpret_cast<uint4*>(sm + B_BW3T + cm_off(n, 0, 16)) = *reinterpret_cast<const uint4*>(w);
+    *reinterpret_cast<uint4*>(sm + B_BW3T + cm_off(n, 8, 16)) = none;
+  }
+  for (int j = 0; j < 4; ++j) {
+    s1[lane * SROW + c0 + j] = live ? gelu(z2[j]) : 0.0f;
+    put_bf16(sm + B_BH1T, cm_off(c0 + j, lane, 32), live ? gelu(z1[j]) : 0.0f);
+  }
   TcSync sy{smem_u32(&mbar), 0u, true};
   sy.start();
   const uint32_t tmem = tslot;
-  const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
-  // dH2 = dY W3 -> columns 0..63
+  // dH2 = dY W3 -> columns 0..63; meanwhile dW3 = dY^T H2 and db3
   if (t == 0) {
     umma_128xN(tmem, smem_u32(sm + B_ADY), smem_u32(sm + B_BW3T), 16, 64, false);
     umma_commit(sy.mbar);
   }
+  if (t >= 32 && t < 32 + NO * NH) {
+    const int o = (t - 32) / NH, f = (t - 32) % NH;
+    atomicAdd(&m.G[OW3 + o * NH + f], row_sum(s1 + f, SROW, &s_dy[0][o], NO));
+  } else if (t >= 256 && t < 256 + NO) {
+    atomicAdd(&m.G[OB3 + t - 256], row_sum(&s_dy[0][t - 256], NO, nullptr, 0));
+  }
   sy.finish();
-  // dZ2 = dH2 gelu'(Z2): A operand, its transpose, db2
-  if (sy.ok)
-    for (int c0 = 0; c0 < NH; c0 += 16) {
-      float v[16];
-      tmem_ld16(lanes + c0, v);
-      for (int j = 0; j < 16; ++j) {
-        const int c = c0 + j;
-        const float dz = live ? v[j] * gelu_d(m.Z2[(size_t)row * NH + c]) : 0.0f;
-        put_bf16(sm + B_ADZ2, cm_off(t, c, 64), dz);
-        put_bf16(sm + B_ADZ2T, cm_off(c, t, 128), dz);
-        const float g = warp_sum(dz);
-        if (lane == 0) atomicAdd(&m.G[OB2 + c], g);
-      }
+  // dZ2 = dH2 gelu'(Z2): A operand, its transpose, FP32 tile
+  if (sy.ok) {
+    float v[4];
+    tmem_ld4(tmem + sh.tlane + c0, v);
+    for (int j = 0; j < 4; ++j) {
+      v[j] = live ? v[j] * gelu_d(z2[j]) : 0.0f;
+      put_bf16(sm + B_ADZ2T, cm_off(c0 + j, lane, 32), v[j]);
+      s2[lane * SROW + c0 + j] = v[j];
     }
-  // dH1 = dZ2 W2 -> columns 64..127; dW2 = dZ2^T H1 -> columns 0..63 (lanes 0..63)
+    sh.put_a64(sm + B_ADZ2, v);
+  }
+  // dH1 = dZ2 W2 -> columns 64..127; dW2 = dZ2^T H1 -> columns 0..63 (lanes 0..63); meanwhile db2
   sy.start();
   if (t == 0 && sy.ok) {
     umma_128xN(tmem + 64, smem_u32(sm + B_ADZ2), smem_u32(sm + B_BW2T), 64, 64, false);
-    umma_128xN(tmem, smem_u32(sm + B_ADZ2T), smem_u32(sm + B_BH1T), 128, 64, false);
+    umma_128xN(tmem, smem_u32(sm + B_ADZ2T), smem_u32(sm + B_BH1T), 32, 64, false);
     umma_commit(sy.mbar);
   }
+  if (sy.ok && t >= 64 && t < 64 + NH) atomicAdd(&m.G[OB2 + t - 64], row_sum(s2 + t - 64, SROW, nullptr, 0));
   sy.finish();
   if (sy.ok) {
-    if (warp < 2)   // output rows o = t < 64 of dW2
-      for (int c0 = 0; c0 < NH; c0 += 16) {
-        float v[16];
-        tmem_ld16(lanes + c0, v);
-        for (int j = 0; j < 16; ++j) atomicAdd(&m.G[OW2 + t * NH + c0 + j], v[j]);
-      }
     // dZ1 = dH1 gelu'(Z1); dW1 = dZ1^T Xn and db1 (CUDA cores)
-    float xn[NI];
-    for (int i = 0; i < NI; ++i) xn[i] = live ? m.Xn[(size_t)row * NI + i] : 0.0f;
-    for (int c0 = 0; c0 < NH; c0 += 16) {
-      float v[16];
-      tmem_ld16(lanes + 64 + c0, v);
-      for (int j = 0; j < 16; ++j) {
-        const int c = c0 + j;
-        const float dz = live ? v[j] * gelu_d(m.Z1[(size_t)row * NH + c]) : 0.0f;
-        const float gb = warp_sum(dz);
-        if (lane == 0) atomicAdd(&m.G[OB1 + c], gb);
-        for (int i = 0; i < NI; ++i) {
-          const float g = warp_sum(dz * xn[i]);
-          if (lane == 0) atomicAdd(&m.G[OW1 + c * NI + i], g);
-        }
-      }
+    float v[4];
+    tmem_ld4(tmem + sh.tlane + 64 + c0, v);
+    for (int j = 0; j < 4; ++j) s1[lane * SROW + c0 + j] = live ? v[j] * gelu_d(z1[j]) : 0.0f;
+    if ((t >> 5 & 3) < 2) {   // TMEM lanes 0..63: output rows o of dW2, 16 columns per warp
+      const int o = 32 * (t >> 5 & 3) + lane, cc = 16 * (t >> 7);
+      float w[16];
+      tmem_ld16(tmem + sh.tlane + cc, w);
+      for (int j = 0; j < 16; j += 4) red4(&m.G[OW2 + o * NH + cc + j], w + j);
     }
+  }
+  __syncthreads();
+  if (sy.ok) {
+    if (t < NH * NI) atomicAdd(&m.G[OW1 + t], row_sum(s1 + t / NI, SROW, &s_xn[0][t % NI], NI));
+    else if (t < NH * NI + NH) atomicAdd(&m.G[OB1 + t - NH * NI], row_sum(s1 + t - NH * NI, SROW, nullptr, 0));
   }
   tc_fence_before();
   __syncthreads();
@@ -476,19 +537,19 @@ extern "C" int dsdna_mlp_create(int max_batch, const dsdna_allocator* alloc, voi
   MlpDev& d = m->d;
   d.P = (float*)mlp_alloc(m, sizeof(float) * NP);
   d.Pb = (__nv_bfloat16*)mlp_alloc(m, sizeof(__nv_bfloat16) * NP);
-  d.G = (float*)mlp_alloc(m, sizeof(float) * NP);
+  d.G = (float*)mlp_alloc(m, sizeof(float) * (NP + 2));   // then the loss and the error word
   d.M = (float*)mlp_alloc(m, sizeof(float) * NP);
   d.V = (float*)mlp_alloc(m, sizeof(float) * NP);
   d.Xn = (float*)mlp_alloc(m, sizeof(float) * NI * m->max_batch);
   d.Z1 = (float*)mlp_alloc(m, sizeof(float) * NH * m->max_batch);
   d.Z2 = (float*)mlp_alloc(m, sizeof(float) * NH * m->max_batch);
   d.Yn = (float*)mlp_alloc(m, sizeof(float) * NO * m->max_batch);
-  d.loss = (float*)mlp_alloc(m, sizeof(float) * 4);
-  d.err = reinterpret_cast<unsigned*>(d.loss + 1);
-  if (!d.P || !d.Pb || !d.G || !d.M || !d.V || !d.Xn || !d.Z1 || !d.Z2 || !d.Yn || !d.loss) {
+  if (!d.P || !d.Pb || !d.G || !d.M || !d.V || !d.Xn || !d.Z1 || !d.Z2 || !d.Yn) {
     dsdna_mlp_destroy(m);
     return DSDNA_ENOMEM;
   }
+  d.loss = d.G + NP;
+  d.err = reinterpret_cast<unsigned*>(d.loss + 1);
   for (int c = 0; c < NI; ++c) { d.norm.in_mean[c] = 0.0f; d.norm.in_scale[c] = 1.0f; }
   for (int c = 0; c < NO; ++c) { d.norm.out_mean[c] = 0.0f; d.norm.out_scale[c] = 1.0f; }
   if (cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_BYTES) != cudaSuccess ||
@@ -496,9 +557,8 @@ extern "C" int dsdna_mlp_create(int max_batch, const dsdna_allocator* alloc, voi
     dsdna_mlp_destroy(m);
     return DSDNA_ECUDA;
   }
-  cudaMemsetAsync(d.loss, 0, sizeof(float) * 4, m->st);
   cudaMemsetAsync(d.P, 0, sizeof(float) * NP, m->st);
-  cudaMemsetAsync(d.G, 0, sizeof(float) * NP, m->st);
+  cudaMemsetAsync(d.G, 0, sizeof(float) * (NP + 2), m->st);
   cudaMemsetAsync(d.M, 0, sizeof(float) * NP, m->st);
   cudaMemsetAsync(d.V, 0, sizeof(float) * NP, m->st);
   k_mlp_refresh_bf16<<<(NP + 255) / 256, 256, 0, m->st>>>(d);
@@ -544,15 +604,14 @@ extern "C" int dsdna_mlp_get_params(dsdna_mlp* m, float* params, float* grads) {
 
 extern "C" int dsdna_mlp_forward(dsdna_mlp* m, const float* X, int B, float* Y) {
   if (!m || !X || !Y || B < 1 || B > m->max_batch) return DSDNA_EINVAL;
-  k_mlp_forward<<<(B + TC_ROWS - 1) / TC_ROWS, TC_ROWS, F_BYTES, m->st>>>(m->d, X, B, Y);
+  k_mlp_forward<<<(B + TC_ROWS - 1) / TC_ROWS, TC_THREADS, F_BYTES, m->st>>>(m->d, X, B, Y);
   return cudaGetLastError() == cudaSuccess ? DSDNA_OK : DSDNA_ECUDA;
 }
 
 extern "C" int dsdna_mlp_backward(dsdna_mlp* m, const float* T, int B, float* loss_host) {
   if (!m || !T || B < 1 || B > m->max_batch) return DSDNA_EINVAL;
-  cudaMemsetAsync(m->d.G, 0, sizeof(float) * NP, m->st);
-  cudaMemsetAsync(m->d.loss, 0, sizeof(float), m->st);
-  k_mlp_backward<<<(B + TC_ROWS - 1) / TC_ROWS, TC_ROWS, B_BYTES, m->st>>>(m->d, T, B);
+  cudaMemsetAsync(m->d.G, 0, sizeof(float) * (NP + 1), m->st);   // gradients and loss
+  k_mlp_backward<<<(B + TC_ROWS - 1) / TC_ROWS, TC_THREADS, B_BYTES, m->st>>>(m->d, T, B);
   if (cudaGetLastError() != cudaSuccess) return DSDNA_ECUDA;
   if (loss_host) {
     float lw[2];
