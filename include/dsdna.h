@@ -127,7 +127,9 @@ typedef struct dsdna_params {
   int max_neighbors;                     /* neighbour capacity per bead (0: default 32; at most 32) */
   int block_threads;                     /* threads per CTA of the step kernel, a multiple of 32 in 64..1024
                                             (FP64 path 64..256); 0: 1024 in mixed precision when the system has
-                                            at least 32 tiles of 32 nucleotides per SM, else 256 */
+                                            at least 32 tiles of 32 nucleotides per SM, else 256.  Small
+                                            systems that rebuild inside the step kernel run a resident step
+                                            kernel with a CTA size of its own (rebuild_mode) */
   int blocks_per_sm;                     /* persistent CTAs per SM (0: as many as fit) */
   int steps_per_graph;                   /* steps per captured CUDA graph launch (0: default 50) */
   /* Sec. 5 denaturation.  A base pair is open when its hydrogen bond is
@@ -146,7 +148,11 @@ typedef struct dsdna_params {
   /* Neighbour-list rebuild: 1 separate kernels between step launches, 2
    * inside the persistent step kernel (grid barriers between its phases; one
    * launch runs a whole graph chunk of steps), 0 chooses 2 for systems of at
-   * most DSDNA_FUSED_REBUILD_MAX_NT nucleotides without a Morton cell table. */
+   * most DSDNA_FUSED_REBUILD_MAX_NT nucleotides without a Morton cell table.
+   * With the chain-window list (list_build 0) and at most 512 nucleotides per
+   * SM (256 in FP64), the steps that rebuild inside run in the resident kernel,
+   * which keeps its stretch of the chain on the SM from step to step; the
+   * trajectory is the same bit for bit. */
   int rebuild_mode;
   /* Sec. 2 gives sigma = 1 for steric beads and has ghosts see the other
    * strand at sigma = 0.5, without saying what two steric beads of opposite
@@ -162,8 +168,8 @@ typedef struct dsdna_params {
    * so both give the same forces and trajectories bit for bit. */
   int pair_halving;
   /* Neighbour-list build in the separate rebuild kernels and the force and
-   * energy passes (the rebuild inside the step kernel, rebuild_mode 2, walks
-   * cells).  0: chain-window build: every pair of beads whose 16-slot
+   * energy passes (the rebuild inside the step kernel, rebuild_mode 2, builds
+   * the chain window too in the resident kernel and walks cells otherwise).  0: chain-window build: every pair of beads whose 16-slot
    * segments (8 base pairs) are equal or adjacent is tested directly from
    * shared memory, and the other pairs are found through a grid of segment
    * bounding spheres (Sec. 6 lists, arranged for a chain whose list partners

@@ -23,6 +23,8 @@ template <class Real> cudaError_t engine_occupancy(int mode, int T, int* blocks_
 template <class Real> cudaError_t engine_launch(int mode, const KArgs<Real>& a, int grid, int T, size_t smem, cudaStream_t st);
 template <class Real> cudaError_t rebuild_launch(const KArgs<Real>& a, int scan_grid, cudaStream_t st);
 template <class Real> cudaError_t rebuild_prepare();
+template <class Real> cudaError_t resident_shape(int64_t n, int rings, bool ext, int nsm, int* grid, int* T, size_t* smem);
+template <class Real> cudaError_t resident_launch(int mode, const KArgs<Real>& a, int grid, int T, size_t smem, cudaStream_t st);
 }  // namespace dsdna
 
 using namespace dsdna;
@@ -55,10 +57,13 @@ struct dsdna_ctx {
   int* evl = nullptr; uint2* psrc = nullptr; int* tcnt = nullptr;   // pair halving (mixed precision)
   int64_t n_junc = 0;            // junction owners of circular molecules (8 per ring)
   bool fused = false;            // list rebuilt inside the step kernel
+  bool resident = false;         // ... by the resident kernel (steps; the other passes run engine_kernel)
+  int T_step = 0;                // threads per CTA of the step kernel
   // kernel instance: with circular molecules or the bubble rule, MODE_EXT;
   // steps with the rebuild inside, MODE_FUSED
   int kernel_flags(int mode) const {
-    return ((n_junc > 0 || p.bubble_rule > 0) ? MODE_EXT : 0) | ((fused && mode == MODE_STEP) ? MODE_FUSED : 0);
+    return ((n_junc > 0 || p.bubble_rule > 0) ? MODE_EXT : 0) |
+           (mode == MODE_STEP ? (resident ? MODE_RES : fused ? MODE_FUSED : 0) : 0);
   }
   int64_t* jslot = nullptr; int* jidx = nullptr; void* jout = nullptr;
   unsigned* cnt = nullptr; unsigned* start = nullptr; int* key = nullptr;
@@ -85,6 +90,7 @@ struct dsdna_ctx {
   // in-kernel rebuild keeps the cell walk
   bool chain = false;
   float4* segc = nullptr;
+  unsigned long long* rs_head = nullptr; unsigned* rs_next = nullptr; unsigned rs_mask = 0;   // resident kernel's cell lists
   int sg_nc[3] = {0, 0, 0};
   double sg_edge = 0;
   unsigned sg_H = 0, sg_mask = 0;
@@ -346,6 +352,7 @@ static void fill_args(dsdna_ctx* c, KArgs<Real>& a) {
   a.nseg16 = (c->n + 15) / 16;
   a.sg_H = c->sg_H;
   a.sg_mask = c->sg_mask;
+  a.rs_head = c->rs_head; a.rs_next = c->rs_next; a.rs_mask = c->rs_mask;
   a.sg_rcap = (float)DSDNA_SEG_RCAP;
   a.sg_reach = std::sqrt(a.c.rl_max2) + 0.002f;   // margin over the FP32 rounding of centres and radii
   for (int k = 0; k < 3; ++k) {
@@ -543,6 +550,32 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
     c->sg_H = Hs + 2048;   // a last tile of empty entries: start[Hs] is a scanned entry
   }
   c->H_alloc = std::max(c->H, c->sg_H);
+  // Steps of a small system with the chain-window list run in the resident
+  // kernel, whatever block_threads says (the CTA size of engine_kernel), as
+  // long as a stretch per SM fits a CTA (77,824 nucleotides in mixed precision
+  // and 38,912 in FP64 on 152 SMs): below that it is 1.7 to 2.9 times faster
+  // than engine_kernel with the rebuild inside (figures in resident.cuh), above
+  // it a CTA would have no thread and registers for each of its nucleotides.
+  cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device);
+  if (c->fused && c->chain) {
+    int64_t rings = 0;
+    for (int m = 0; m < c->n_mol; ++m) rings += c->circular[m];
+    const bool ext = rings > 0 || c->p.bubble_rule > 0;
+    int g = 0, t = 0;
+    size_t sm = 0;
+    const cudaError_t e = c->fp64() ? resident_shape<double>(n, rings > 0, ext, c->nsm, &g, &t, &sm)
+                                    : resident_shape<float>(n, rings > 0, ext, c->nsm, &g, &t, &sm);
+    if (e != cudaSuccess) return bad(fail(c, DSDNA_ECUDA, std::string("resident kernel: ") + cudaGetErrorString(e)));
+    if (g > 0) {
+      c->resident = true;
+      c->grid[MODE_STEP] = g;
+      c->T_step = t;
+      c->smem[MODE_STEP] = sm;
+      unsigned H = 2048;
+      while ((int64_t)H < n / 8) H <<= 1;
+      c->rs_mask = H - 1;
+    }
+  }
 
   // allocations
   const bool f64 = c->fp64();
@@ -575,6 +608,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   ALLOC(cnt, unsigned, c->H_alloc); ALLOC(start, unsigned, (size_t)c->H_alloc + 1); ALLOC(key, int, nn);
   ALLOC(cent, float4, nn); ALLOC(wpos, float4, nn);
   if (c->chain) ALLOC(segc, float4, (nn + 15) / 16 + 1);
+  if (c->resident) { ALLOC(rs_head, unsigned long long, (size_t)c->rs_mask + 1); ALLOC(rs_next, unsigned, (nn + 15) / 16 + nn); }
   ALLOC(mol_off, int64_t, c->n_mol + 1); ALLOC(ext_d, double, (size_t)c->n_mol * 8);
   ALLOC(bar, GridBar, 1); ALLOC(err, unsigned, 4); ALLOC(step_d, int64_t, 1); ALLOC(rebuild, int, 4);
   ALLOC(nrebuild, unsigned long long, 1);
@@ -591,10 +625,9 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   ALLOC(nlaunch, unsigned long long, 1);
 #undef ALLOC
   // launch shape per mode (cooperative: every CTA resident)
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
-  c->nsm = nsm;
-  for (int mode = 0; mode < 3; ++mode) {
+  const int nsm = c->nsm;
+  if (!c->resident) c->T_step = c->T;
+  for (int mode = c->resident ? 1 : 0; mode < 3; ++mode) {
     int bps = 0;
     const int m = mode | c->kernel_flags(mode);
     cudaError_t e = f64 ? engine_occupancy<double>(m, c->T, &bps, &c->smem[mode])
@@ -671,6 +704,8 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
       cudaMemset(c->X, 0, (f64 ? 48 : 24) * ns) != cudaSuccess || cudaMemset(c->kref, 0, 12 * ns) != cudaSuccess ||
       cudaMemset(c->img, 0, 4 * ns) != cudaSuccess)
     return bad(fail(c, DSDNA_ECUDA, "initialisation"));
+  if (c->resident && cudaMemset(c->rs_head, 0, sizeof(unsigned long long) * ((size_t)c->rs_mask + 1)) != cudaSuccess)
+    return bad(fail(c, DSDNA_ECUDA, "initialisation"));
   if (!f64 && (cudaMemset(c->Kw, 0, sizeof(int4) * 2 * ns) != cudaSuccess ||
                cudaMemset(c->U, 0, sizeof(float4) * 2 * ns) != cudaSuccess))
     return bad(fail(c, DSDNA_ECUDA, "initialisation"));
@@ -741,10 +776,14 @@ static cudaError_t launch_engine(dsdna_ctx* c, int mode, int64_t nsteps, int64_t
   if (c->fp64()) {
     KArgs<double> a = c->kd;
     a.nsteps = nsteps; a.steps_left = steps_left; a.use_cond = use_cond; a.h_while = hw;
+    if (mode == MODE_STEP && c->resident)
+      return resident_launch<double>(c->kernel_flags(mode), a, c->grid[mode], c->T_step, c->smem[mode], c->st);
     return engine_launch<double>(mode | c->kernel_flags(mode), a, c->grid[mode], c->T, c->smem[mode], c->st);
   }
   KArgs<float> a = c->kf;
   a.nsteps = nsteps; a.steps_left = steps_left; a.use_cond = use_cond; a.h_while = hw;
+  if (mode == MODE_STEP && c->resident)
+    return resident_launch<float>(c->kernel_flags(mode), a, c->grid[mode], c->T_step, c->smem[mode], c->st);
   return engine_launch<float>(mode | c->kernel_flags(mode), a, c->grid[mode], c->T, c->smem[mode], c->st);
 }
 
@@ -1176,7 +1215,7 @@ extern "C" int dsdna_get_info(const dsdna_ctx* c, dsdna_info* info) {
   info->rebuild_in_step = c->fused ? 1 : 0;
   info->chain_list = c->chain ? 1 : 0;
   info->grid_blocks = c->grid[MODE_STEP];
-  info->block_threads = c->T;
+  info->block_threads = c->T_step;
   info->max_neighbors = c->p.max_neighbors;
   info->precision = c->p.precision;
   info->skin = c->p.skin;

@@ -58,6 +58,39 @@ __device__ __forceinline__ unsigned seg_key(const KArgs<Real>& a, int mol, const
   return (unsigned)cc[0] + (unsigned)a.sg_nc[0] * ((unsigned)cc[1] + (unsigned)a.sg_nc[1] * (unsigned)cc[2]);
 }
 
+// Bounding sphere of each 16-slot segment (a 16-lane group of the warp, the
+// lanes with `in` set, the first lane first): radius returned, wrapped centre
+// in c3; positions relative to the segment's first bead by minimum image.
+template <class Real>
+__device__ __forceinline__ float seg_sphere(const KArgs<Real>& a, bool in, const float* pw, float* c3) {
+  const int lane = threadIdx.x & 31;
+  float r0[3], d[3];
+  for (int c = 0; c < 3; ++c) {
+    r0[c] = __shfl_sync(0xffffffffu, pw[c], 0, 16);
+    float x = pw[c] - r0[c];
+    x = fmaf(-rintf(x * a.invLf[c]), a.Lf[c], x);
+    d[c] = in ? x : 0.0f;
+  }
+  const int nin = __popc(__ballot_sync(0xffffffffu, in) & (0xffffu << (lane & 16)));
+  float m[3];
+  for (int c = 0; c < 3; ++c) {
+    float s = d[c];
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 16);
+    m[c] = nin > 0 ? s / (float)nin : 0.0f;
+  }
+  float r2 = 0.0f;
+  if (in) {
+    const float ex = d[0] - m[0], ey = d[1] - m[1], ez = d[2] - m[2];
+    r2 = ex * ex + ey * ey + ez * ez;
+  }
+  for (int o = 8; o > 0; o >>= 1) r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o, 16));
+  for (int c = 0; c < 3; ++c) {
+    const float x = r0[c] + m[c];
+    c3[c] = fmaf(-floorf(x * a.invLf[c]), a.Lf[c], x);
+  }
+  return sqrtf(r2) * 1.0001f + 1e-4f;   // rounded up past the FP32 error of the centre
+}
+
 // S1: bin every bead as the cell-walk build does (wrapped position, image
 // word, rebuild reference), then the bounding sphere of each 16-slot segment
 // (a 16-lane group of the warp; positions relative to the segment's first
@@ -74,40 +107,16 @@ __global__ void k_rebuild_segbin(const KArgs<Real> a) {
     float pw[3] = {0.0f, 0.0f, 0.0f};
     int mol = 0;
     if (in) mol = bin_bead(a, cur, g, fl, pw);
-    float r0[3], d[3];
-    for (int c = 0; c < 3; ++c) {
-      r0[c] = __shfl_sync(0xffffffffu, pw[c], 0, 16);
-      float x = pw[c] - r0[c];
-      x = fmaf(-rintf(x * a.invLf[c]), a.Lf[c], x);
-      d[c] = in ? x : 0.0f;
-    }
-    const int nin = __popc(__ballot_sync(0xffffffffu, in) & (0xffffu << (lane & 16)));
-    float m[3];
-    for (int c = 0; c < 3; ++c) {
-      float s = d[c];
-      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 16);
-      m[c] = nin > 0 ? s / (float)nin : 0.0f;
-    }
-    float r2 = 0.0f;
-    if (in) {
-      const float ex = d[0] - m[0], ey = d[1] - m[1], ez = d[2] - m[2];
-      r2 = ex * ex + ey * ey + ez * ez;
-    }
+    float c3[3];
+    const float R = seg_sphere(a, in, pw, c3);
     int mlo = in ? mol : INT_MAX, mhi = in ? mol : INT_MIN;
     for (int o = 8; o > 0; o >>= 1) {
-      r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o, 16));
       mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
       mhi = max(mhi, __shfl_xor_sync(0xffffffffu, mhi, o, 16));
     }
-    const float R = sqrtf(r2) * 1.0001f + 1e-4f;   // rounded up past the FP32 error of the centre
     const bool wide = !(R <= a.sg_rcap) || mlo != mhi;
     int ci[3];
-    if (nin > 0 && (lane & 15) == 0) {
-      float c3[3];
-      for (int c = 0; c < 3; ++c) {
-        const float x = r0[c] + m[c];
-        c3[c] = fmaf(-floorf(x * a.invLf[c]), a.Lf[c], x);
-      }
+    if (in && (lane & 15) == 0) {
       a.segc[g >> 4] = make_float4(c3[0], c3[1], c3[2], wide ? -1.0f : R);
       if (!wide) {
         seg_cell(a, c3[0], c3[1], c3[2], ci);
@@ -199,6 +208,223 @@ __device__ __forceinline__ void cl_item_pairs(const KArgs<Real>& a, int g, float
   }
 }
 
+// The staged window of a warp (slots g0 - 16 .. g0 + 47; raw, word, val: slots
+// g0 - 16 + lane and + 32) into win, unwrapped around the middle slot g0 + 16
+// when every slot belongs to its molecule and lies within a quarter box of it,
+// so that every difference is the minimum image (returns true: the fast path);
+// else as wrapped, each pair taking its own minimum image.
+template <class Real>
+__device__ __forceinline__ bool cl_stage(const KArgs<Real>& a, int lane, const float4* raw, const int* word,
+                                         const bool* val, float4* win) {
+  const float ref[3] = {__shfl_sync(0xffffffffu, raw[1].x, 0), __shfl_sync(0xffffffffu, raw[1].y, 0),
+                        __shfl_sync(0xffffffffu, raw[1].z, 0)};
+  const int rmol = __shfl_sync(0xffffffffu, val[1] ? __float_as_int(raw[1].w) : -1, 0);
+  bool ok = true;
+  float4 un[2];
+  for (int h = 0; h < 2; ++h) {
+    un[h] = make_float4(CL_FAR, CL_FAR, CL_FAR, __int_as_float(0));
+    if (!val[h]) continue;
+    float p[3] = {raw[h].x, raw[h].y, raw[h].z};
+    int code = word[h];
+    for (int c = 0; c < 3; ++c) {
+      const float tq = rintf((ref[c] - p[c]) * a.invLf[c]);
+      p[c] = fmaf(tq, a.Lf[c], p[c]);
+      code |= ((int)tq + 1) << (1 + 2 * c);
+      ok = ok && (!a.periodic || fabsf(p[c] - ref[c]) <= 0.24f * a.Lf[c]);
+    }
+    ok = ok && __float_as_int(raw[h].w) == rmol;
+    un[h] = make_float4(p[0], p[1], p[2], __int_as_float(code));
+  }
+  const bool fast = __all_sync(0xffffffffu, ok);
+  for (int h = 0; h < 2; ++h) {
+    const int k = lane + 32 * h;
+    win[k + (k >> 4)] = fast ? un[h]
+                             : make_float4(raw[h].x, raw[h].y, raw[h].z,
+                                           __int_as_float(word[h] | (__float_as_int(raw[h].w) << 8)));
+  }
+  __syncwarp();
+  return fast;
+}
+
+// Typed pairs of the lane's bead g0 + lane with the other slots of its own
+// 16-slot segment and its two neighbours, from the staged window, into its
+// empty list.
+template <class Real>
+__device__ __forceinline__ void cl_window(const KArgs<Real>& a, int64_t g0, int lane, bool in, bool fast,
+                                          const float4* win, bool& st_g, int* list, int& cnt, int& total) {
+  const int g = (int)g0 + lane;
+  const int kb = lane & 16;   // lanes 0-15 (segment 2t) test staged slots 0..47, lanes 16-31 slots 16..63
+  const float4* wb = win + kb + (kb >> 4);
+  const float4 me = win[lane + 16 + ((lane + 16) >> 4)];
+  const int mew = __float_as_int(me.w);
+  st_g = (mew & 1) != 0;
+  if (in) {
+    if (fast) {
+      // candidate c is slot g0 - 16 + kb + c: across strands iff c and lane differ in parity
+      const float rs_st = st_g ? a.c.rl_ss2 : -1.0f, rc_st = st_g ? a.c.rl_cs2 : a.c.rl_cr2;
+      const bool odd = lane & 1;
+      const float rE_st = odd ? rc_st : rs_st, rE_gh = odd ? a.c.rl_cr2 : -1.0f;
+      const float rO_st = odd ? rs_st : rc_st, rO_gh = odd ? -1.0f : a.c.rl_cr2;
+      // hits as a bit mask first (no branch in the loop; three blocks of 16
+      // candidates), then appended in slot order to the still empty list
+      unsigned long long hits = 0ull;
+      for (int c0 = 0; c0 < 48; c0 += 16) {
+        const float4* wc = wb + c0 + (c0 >> 4);
+        unsigned m16 = 0u;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          const float4 o = wc[k];
+          const float dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
+          const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+          const bool stj = (__float_as_int(o.w) & 1) != 0;
+          const float rl2 = (k & 1) ? (stj ? rO_st : rO_gh) : (stj ? rE_st : rE_gh);
+          if (r2 < rl2) m16 |= 1u << k;
+        }
+        hits |= (unsigned long long)m16 << c0;
+      }
+      hits &= ~(1ull << (lane + 16 - kb));   // the bead itself
+      total = __popcll(hits);
+      for (; hits && cnt < a.cap; hits &= hits - 1ull) {
+        const int c = __ffsll((long long)hits) - 1;
+        int ent = ent_make((int)g0 - 16 + kb + c, 0, 0, 0);
+        if constexpr (sizeof(Real) == 8) {
+          const int ow = __float_as_int(wb[c + (c >> 4)].w);
+          ent = ent_make((int)g0 - 16 + kb + c, ((ow >> 1) & 3) - ((mew >> 1) & 3), ((ow >> 3) & 3) - ((mew >> 3) & 3),
+                         ((ow >> 5) & 3) - ((mew >> 5) & 3));
+        }
+        list[cnt++] = ent;
+      }
+    } else {
+      for (int c = 0; c < 48; ++c) {
+        const float4 o = wb[c + (c >> 4)];
+        const int ow = __float_as_int(o.w);
+        const int j = (int)g0 - 16 + kb + c;
+        if (!(ow & CL_VALID) || j == g || (ow >> 8) != (mew >> 8)) continue;
+        float d[3] = {o.x - me.x, o.y - me.y, o.z - me.z};
+        int sc3[3];
+        for (int q = 0; q < 3; ++q) {
+          const float s = -rintf(d[q] * a.invLf[q]);
+          d[q] = fmaf(s, a.Lf[q], d[q]);
+          sc3[q] = (int)s;
+        }
+        const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        const float rl2 = list_r2(a.c, ((g ^ j) & 1) != 0, st_g && (ow & 1));
+        if (r2 < rl2) cl_append(list, cnt, total, a.cap, ent_make(j, sc3[0], sc3[1], sc3[2]));
+      }
+    }
+  }
+}
+
+// Pairs of the lanes' beads (wrapped position mp) with the beads of the lanes'
+// accepted grid items (acc: sphere it, slot range ir, of segment hq of the
+// warp's two, whose spheres are sc); warp-collective, win is its scratch.
+template <class Real>
+__device__ __forceinline__ void cl_items(const KArgs<Real>& a, int lane, int g, bool in, bool st_g, const float4* sc,
+                                         float4 mp, bool acc, int hq, int ir, float4 it, float4* win, int* gi,
+                                         float4* gc, int* list, int& cnt, int& total) {
+  // up to two accepted items of each segment at a time (item slot
+  // 2h + k: the k-th of segment 2t + h): their beads are staged in the
+  // window buffer, one load each and all in flight together, unwrapped
+  // around the segment's centre; only the beads within the segment's
+  // radius + reach of its centre are kept (compacted), and only the
+  // lanes whose bead lies within the item's radius + reach of the
+  // item's centre test them, both halves at once.  Any pair within list
+  // range passes both filters, and both unwrapped positions lie within
+  // 3 radii + 2 reaches of the centre, far below half the box.
+  unsigned bal[2] = {__ballot_sync(0xffffffffu, acc && hq == 0), __ballot_sync(0xffffffffu, acc && hq == 1)};
+  while (bal[0] | bal[1]) {
+    int nh[2];
+    for (int h = 0; h < 2; ++h) {
+      const int rank = __popc(bal[h] & ((1u << lane) - 1u));
+      if (((bal[h] >> lane) & 1u) && rank < 2) {
+        gi[2 * h + rank] = ir;
+        gc[2 * h + rank] = it;
+      }
+      unsigned rest = bal[h];
+      for (int q = 0; q < 2 && rest; ++q) rest &= rest - 1u;
+      nh[h] = __popc(bal[h]) - __popc(rest);
+      bal[h] = rest;
+    }
+    __syncwarp();
+    unsigned keep[2];
+    for (int r = 0; r < 2; ++r) {   // staging round r holds item slots 2r (lanes 0-15) and 2r + 1
+      const int q = 2 * r + (lane >> 4), b = lane & 15;
+      const float4 c = sc[r];        // item slots 2r, 2r + 1 belong to segment 2t + r
+      bool pass = false;
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if ((q & 1) < nh[r]) {
+        const int gq = gi[q];
+        const int j = (gq & ENT_JMASK) + b;
+        if (b <= (int)((unsigned)gq >> ENT_J_BITS)) {
+          const float4 pj = a.wpos[j];
+          float pp[3] = {pj.x, pj.y, pj.z};
+          const float cc[3] = {c.x, c.y, c.z};
+          int code = (a.topo[j] & F_STERIC) ? 1 : 0;
+          float r2 = 0.0f;
+          for (int k = 0; k < 3; ++k) {
+            const float tq = rintf((cc[k] - pp[k]) * a.invLf[k]);
+            pp[k] = fmaf(tq, a.Lf[k], pp[k]);
+            code |= ((int)tq + 1) << (1 + 2 * k);
+            r2 = fmaf(pp[k] - cc[k], pp[k] - cc[k], r2);
+          }
+          const float reach = c.w + a.sg_reach;
+          pass = r2 < reach * reach;
+          v = make_float4(pp[0], pp[1], pp[2], __int_as_float(code | (b << 8)));
+        }
+      }
+      keep[r] = __ballot_sync(0xffffffffu, pass);
+      const unsigned mine16 = (keep[r] >> (lane & 16)) & 0xffffu;
+      if (pass) win[16 * q + __popc(mine16 & ((1u << b) - 1u))] = v;
+    }
+    __syncwarp();
+    const int hme = lane >> 4, nme = hme ? nh[1] : nh[0];
+    const float4 cme = hme ? sc[1] : sc[0];
+    float pi[3] = {mp.x, mp.y, mp.z};
+    int ti[3];
+    {
+      const float cc[3] = {cme.x, cme.y, cme.z};
+      for (int k = 0; k < 3; ++k) {
+        const float tq = rintf((cc[k] - pi[k]) * a.invLf[k]);
+        pi[k] = fmaf(tq, a.Lf[k], pi[k]);
+        ti[k] = (int)tq;
+      }
+    }
+    for (int k = 0; k < 2; ++k) {
+      if (!in || k >= nme) continue;
+      const int q = 2 * hme + k;
+      const unsigned kq = (keep[hme] >> (16 * k)) & 0xffffu;   // round hme, half k
+      const float4 cj = gc[q];
+      float r2c = 0.0f;
+      {
+        const float cc[3] = {cj.x, cj.y, cj.z};
+        for (int k3 = 0; k3 < 3; ++k3) {
+          float d = cc[k3] - pi[k3];
+          d = fmaf(-rintf(d * a.invLf[k3]), a.Lf[k3], d);
+          r2c = fmaf(d, d, r2c);
+        }
+      }
+      const float reach = cj.w + a.sg_reach;
+      if (!(r2c < reach * reach)) continue;
+      const int j0 = gi[q] & ENT_JMASK, nk = __popc(kq);
+      for (int b = 0; b < nk; ++b) {
+        const float4 o = win[16 * q + b];
+        const int ow = __float_as_int(o.w);
+        const int j = j0 + (ow >> 8);
+        const float dx = o.x - pi[0], dy = o.y - pi[1], dz = o.z - pi[2];
+        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+        const float rl2 = list_r2(a.c, ((g ^ j) & 1) != 0, st_g && (ow & 1));
+        if (r2 < rl2) {
+          int ent = ent_make(j, 0, 0, 0);
+          if constexpr (sizeof(Real) == 8)
+            ent = ent_make(j, ((ow >> 1) & 3) - 1 - ti[0], ((ow >> 3) & 3) - 1 - ti[1], ((ow >> 5) & 3) - 1 - ti[2]);
+          cl_append(list, cnt, total, a.cap, ent);
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // S3: one warp per 32-slot tile (segments 2t and 2t + 1), one lane per bead.
 // The grid query is a chain of dependent loads (sphere -> table bounds ->
 // items), so both segments' loads are issued together and ahead of the window
@@ -276,95 +502,10 @@ __global__ void __launch_bounds__(CL_WARPS * 32, 4) k_rebuild_list_chain(const K
         re[h] = a.start[key[h] + 1];
       }
 
-    const float ref[3] = {__shfl_sync(0xffffffffu, raw[1].x, 0), __shfl_sync(0xffffffffu, raw[1].y, 0),
-                          __shfl_sync(0xffffffffu, raw[1].z, 0)};
-    const int rmol = __shfl_sync(0xffffffffu, val[1] ? __float_as_int(raw[1].w) : -1, 0);
-    bool ok = true;
-    float4 un[2];
-    for (int h = 0; h < 2; ++h) {
-      un[h] = make_float4(CL_FAR, CL_FAR, CL_FAR, __int_as_float(0));
-      if (!val[h]) continue;
-      float p[3] = {raw[h].x, raw[h].y, raw[h].z};
-      int code = word[h];
-      for (int c = 0; c < 3; ++c) {
-        const float tq = rintf((ref[c] - p[c]) * a.invLf[c]);
-        p[c] = fmaf(tq, a.Lf[c], p[c]);
-        code |= ((int)tq + 1) << (1 + 2 * c);
-        ok = ok && (!a.periodic || fabsf(p[c] - ref[c]) <= 0.24f * a.Lf[c]);
-      }
-      ok = ok && __float_as_int(raw[h].w) == rmol;
-      un[h] = make_float4(p[0], p[1], p[2], __int_as_float(code));
-    }
-    const bool fast = __all_sync(0xffffffffu, ok);
-    for (int h = 0; h < 2; ++h) {
-      const int k = lane + 32 * h;
-      win[k + (k >> 4)] = fast ? un[h]
-                               : make_float4(raw[h].x, raw[h].y, raw[h].z,
-                                             __int_as_float(word[h] | (__float_as_int(raw[h].w) << 8)));
-    }
-    __syncwarp();
-
+    const bool fast = cl_stage(a, lane, raw, word, val, win);
     int cnt = 0, total = 0;
-    const int kb = lane & 16;   // lanes 0-15 (segment 2t) test staged slots 0..47, lanes 16-31 slots 16..63
-    const float4* wb = win + kb + (kb >> 4);
-    const float4 me = win[lane + 16 + ((lane + 16) >> 4)];
-    const int mew = __float_as_int(me.w);
-    const bool st_g = (mew & 1) != 0;
-    if (in) {
-      if (fast) {
-        // candidate c is slot g0 - 16 + kb + c: across strands iff c and lane differ in parity
-        const float rs_st = st_g ? a.c.rl_ss2 : -1.0f, rc_st = st_g ? a.c.rl_cs2 : a.c.rl_cr2;
-        const bool odd = lane & 1;
-        const float rE_st = odd ? rc_st : rs_st, rE_gh = odd ? a.c.rl_cr2 : -1.0f;
-        const float rO_st = odd ? rs_st : rc_st, rO_gh = odd ? -1.0f : a.c.rl_cr2;
-        // hits as a bit mask first (no branch in the loop; three blocks of 16
-        // candidates), then appended in slot order to the still empty list
-        unsigned long long hits = 0ull;
-        for (int c0 = 0; c0 < 48; c0 += 16) {
-          const float4* wc = wb + c0 + (c0 >> 4);
-          unsigned m16 = 0u;
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float4 o = wc[k];
-            const float dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
-            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-            const bool stj = (__float_as_int(o.w) & 1) != 0;
-            const float rl2 = (k & 1) ? (stj ? rO_st : rO_gh) : (stj ? rE_st : rE_gh);
-            if (r2 < rl2) m16 |= 1u << k;
-          }
-          hits |= (unsigned long long)m16 << c0;
-        }
-        hits &= ~(1ull << (lane + 16 - kb));   // the bead itself
-        total = __popcll(hits);
-        for (; hits && cnt < a.cap; hits &= hits - 1ull) {
-          const int c = __ffsll((long long)hits) - 1;
-          int ent = ent_make((int)g0 - 16 + kb + c, 0, 0, 0);
-          if constexpr (sizeof(Real) == 8) {
-            const int ow = __float_as_int(wb[c + (c >> 4)].w);
-            ent = ent_make((int)g0 - 16 + kb + c, ((ow >> 1) & 3) - ((mew >> 1) & 3), ((ow >> 3) & 3) - ((mew >> 3) & 3),
-                           ((ow >> 5) & 3) - ((mew >> 5) & 3));
-          }
-          list[cnt++] = ent;
-        }
-      } else {
-        for (int c = 0; c < 48; ++c) {
-          const float4 o = wb[c + (c >> 4)];
-          const int ow = __float_as_int(o.w);
-          const int j = (int)g0 - 16 + kb + c;
-          if (!(ow & CL_VALID) || j == g || (ow >> 8) != (mew >> 8)) continue;
-          float d[3] = {o.x - me.x, o.y - me.y, o.z - me.z};
-          int sc3[3];
-          for (int q = 0; q < 3; ++q) {
-            const float s = -rintf(d[q] * a.invLf[q]);
-            d[q] = fmaf(s, a.Lf[q], d[q]);
-            sc3[q] = (int)s;
-          }
-          const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-          const float rl2 = list_r2(a.c, ((g ^ j) & 1) != 0, st_g && (ow & 1));
-          if (r2 < rl2) cl_append(list, cnt, total, a.cap, ent_make(j, sc3[0], sc3[1], sc3[2]));
-        }
-      }
-    }
+    bool st_g = false;
+    cl_window(a, g0, lane, in, fast, win, st_g, list, cnt, total);
 
     // partners in segments two or more away, through the segment grid: the
     // 54 ranges flattened over the lanes (range q < 27: cell q of segment 2t,
@@ -409,107 +550,7 @@ __global__ void __launch_bounds__(CL_WARPS * 32, 4) k_rebuild_list_chain(const K
           const int64_t lo_h = hq ? slo[1] : slo[0], hi_h = hq ? shi[1] : shi[0];
           if (j0 >= lo_h && j0 < hi_h && (js > s + 1 || js < s - 1)) acc = cl_spheres_meet(a, hq ? sc[1] : sc[0], it);
         }
-        // up to two accepted items of each segment at a time (item slot
-        // 2h + k: the k-th of segment 2t + h): their beads are staged in the
-        // window buffer, one load each and all in flight together, unwrapped
-        // around the segment's centre; only the beads within the segment's
-        // radius + reach of its centre are kept (compacted), and only the
-        // lanes whose bead lies within the item's radius + reach of the
-        // item's centre test them, both halves at once.  Any pair within list
-        // range passes both filters, and both unwrapped positions lie within
-        // 3 radii + 2 reaches of the centre, far below half the box.
-        unsigned bal[2] = {__ballot_sync(0xffffffffu, acc && hq == 0), __ballot_sync(0xffffffffu, acc && hq == 1)};
-        while (bal[0] | bal[1]) {
-          int nh[2];
-          for (int h = 0; h < 2; ++h) {
-            const int rank = __popc(bal[h] & ((1u << lane) - 1u));
-            if (((bal[h] >> lane) & 1u) && rank < 2) {
-              s_gi[w][2 * h + rank] = ir;
-              s_gc[w][2 * h + rank] = it;
-            }
-            unsigned rest = bal[h];
-            for (int q = 0; q < 2 && rest; ++q) rest &= rest - 1u;
-            nh[h] = __popc(bal[h]) - __popc(rest);
-            bal[h] = rest;
-          }
-          __syncwarp();
-          unsigned keep[2];
-          for (int r = 0; r < 2; ++r) {   // staging round r holds item slots 2r (lanes 0-15) and 2r + 1
-            const int q = 2 * r + (lane >> 4), b = lane & 15;
-            const float4 c = sc[r];        // item slots 2r, 2r + 1 belong to segment 2t + r
-            bool pass = false;
-            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if ((q & 1) < nh[r]) {
-              const int gq = s_gi[w][q];
-              const int j = (gq & ENT_JMASK) + b;
-              if (b <= (int)((unsigned)gq >> ENT_J_BITS)) {
-                const float4 pj = a.wpos[j];
-                float pp[3] = {pj.x, pj.y, pj.z};
-                const float cc[3] = {c.x, c.y, c.z};
-                int code = (a.topo[j] & F_STERIC) ? 1 : 0;
-                float r2 = 0.0f;
-                for (int k = 0; k < 3; ++k) {
-                  const float tq = rintf((cc[k] - pp[k]) * a.invLf[k]);
-                  pp[k] = fmaf(tq, a.Lf[k], pp[k]);
-                  code |= ((int)tq + 1) << (1 + 2 * k);
-                  r2 = fmaf(pp[k] - cc[k], pp[k] - cc[k], r2);
-                }
-                const float reach = c.w + a.sg_reach;
-                pass = r2 < reach * reach;
-                v = make_float4(pp[0], pp[1], pp[2], __int_as_float(code | (b << 8)));
-              }
-            }
-            keep[r] = __ballot_sync(0xffffffffu, pass);
-            const unsigned mine16 = (keep[r] >> (lane & 16)) & 0xffffu;
-            if (pass) win[16 * q + __popc(mine16 & ((1u << b) - 1u))] = v;
-          }
-          __syncwarp();
-          const int hme = lane >> 4, nme = hme ? nh[1] : nh[0];
-          const float4 cme = hme ? sc[1] : sc[0];
-          float pi[3] = {mp.x, mp.y, mp.z};
-          int ti[3];
-          {
-            const float cc[3] = {cme.x, cme.y, cme.z};
-            for (int k = 0; k < 3; ++k) {
-              const float tq = rintf((cc[k] - pi[k]) * a.invLf[k]);
-              pi[k] = fmaf(tq, a.Lf[k], pi[k]);
-              ti[k] = (int)tq;
-            }
-          }
-          for (int k = 0; k < 2; ++k) {
-            if (!in || k >= nme) continue;
-            const int q = 2 * hme + k;
-            const unsigned kq = (keep[hme] >> (16 * k)) & 0xffffu;   // round hme, half k
-            const float4 cj = s_gc[w][q];
-            float r2c = 0.0f;
-            {
-              const float cc[3] = {cj.x, cj.y, cj.z};
-              for (int k3 = 0; k3 < 3; ++k3) {
-                float d = cc[k3] - pi[k3];
-                d = fmaf(-rintf(d * a.invLf[k3]), a.Lf[k3], d);
-                r2c = fmaf(d, d, r2c);
-              }
-            }
-            const float reach = cj.w + a.sg_reach;
-            if (!(r2c < reach * reach)) continue;
-            const int j0 = s_gi[w][q] & ENT_JMASK, nk = __popc(kq);
-            for (int b = 0; b < nk; ++b) {
-              const float4 o = win[16 * q + b];
-              const int ow = __float_as_int(o.w);
-              const int j = j0 + (ow >> 8);
-              const float dx = o.x - pi[0], dy = o.y - pi[1], dz = o.z - pi[2];
-              const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-              const float rl2 = list_r2(a.c, ((g ^ j) & 1) != 0, st_g && (ow & 1));
-              if (r2 < rl2) {
-                int ent = ent_make(j, 0, 0, 0);
-                if constexpr (sizeof(Real) == 8)
-                  ent = ent_make(j, ((ow >> 1) & 3) - 1 - ti[0], ((ow >> 3) & 3) - 1 - ti[1], ((ow >> 5) & 3) - 1 - ti[2]);
-                cl_append(list, cnt, total, a.cap, ent);
-              }
-            }
-          }
-          __syncwarp();
-        }
+        cl_items(a, lane, g, in, st_g, sc, mp, acc, hq, ir, it, win, s_gi[w], s_gc[w], list, cnt, total);
       }
     }
     // a wide segment: each of its beads queries its own 27 cells

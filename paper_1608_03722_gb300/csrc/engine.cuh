@@ -48,6 +48,7 @@ constexpr unsigned B_ERRMASK = B_EFENE | B_ENAN | B_EOVF | B_ETIMEOUT | B_EIMG;
 enum : int { MODE_STEP = 0, MODE_FORCES = 1, MODE_ENERGY = 2 };
 constexpr int MODE_EXT = 4;   // launch flag: kernel instance with circular molecules / bubble rule
 constexpr int MODE_FUSED = 8; // launch flag (MODE_STEP): instance that rebuilds the list in the kernel
+constexpr int MODE_RES = 16;  // launch flag (MODE_STEP): the resident kernel (resident.cuh)
 constexpr int NTERMS = 10;
 constexpr int EOUT_STRIDE = 16;           // energy terms + 6 virial
 constexpr int NBR_J_BITS = 27;   // slot field of a cell-sorted bead word (bit 27: steric flag)
@@ -154,6 +155,10 @@ struct KArgs {
   unsigned sg_mask;  // open box: the table is hashed into sg_mask + 1 entries
   float sg_rcap;     // widest segment kept whole in the grid
   float sg_reach;    // largest list radius plus a margin (sphere test)
+  // resident kernel: hash of segment-grid cells to linked lists of grid items
+  unsigned long long* rs_head;   // [rs_mask + 1] epoch of the rebuild << 32 | first item
+  unsigned* rs_next;             // [nseg16 + n] next item of the list
+  unsigned rs_mask;
   int periodic;
   int nc[3];
   float cellh[3];
@@ -311,6 +316,27 @@ __device__ __forceinline__ V3<float> rel(const SPos<float>& o, const SPos<float>
 }
 __device__ __forceinline__ V3<double> rel(const SPos<double>& o, const SPos<double>& b, const float* /*q*/) {
   return V3<double>{b.x - o.x, b.y - o.y, b.z - o.z};
+}
+// rel(o, b) + hs u, in FP32 rounded once after the product of the mirror
+// difference (site_rel) or of hs u (rel_site).  Both are written out because the
+// compiler may fuse either product into the sum, and which one it picks depends
+// on the code around it: every kernel must round alike for their trajectories
+// to agree bit for bit.
+__device__ __forceinline__ V3<float> site_rel(const SPos<float>& o, const SPos<float>& b, const float* q, float hs, V3<float> u) {
+  return V3<float>{fmaf((float)(int)((unsigned)b.kx - (unsigned)o.kx), q[0], __fmul_rn(hs, u.x)),
+                   fmaf((float)(int)((unsigned)b.ky - (unsigned)o.ky), q[1], __fmul_rn(hs, u.y)),
+                   fmaf((float)(int)((unsigned)b.kz - (unsigned)o.kz), q[2], __fmul_rn(hs, u.z))};
+}
+__device__ __forceinline__ V3<float> rel_site(const SPos<float>& o, const SPos<float>& b, const float* q, float hs, V3<float> u) {
+  return V3<float>{fmaf(hs, u.x, __fmul_rn((float)(int)((unsigned)b.kx - (unsigned)o.kx), q[0])),
+                   fmaf(hs, u.y, __fmul_rn((float)(int)((unsigned)b.ky - (unsigned)o.ky), q[1])),
+                   fmaf(hs, u.z, __fmul_rn((float)(int)((unsigned)b.kz - (unsigned)o.kz), q[2]))};
+}
+__device__ __forceinline__ V3<double> site_rel(const SPos<double>& o, const SPos<double>& b, const float* q, double hs, V3<double> u) {
+  return rel(o, b, q) + hs * u;
+}
+__device__ __forceinline__ V3<double> rel_site(const SPos<double>& o, const SPos<double>& b, const float* q, double hs, V3<double> u) {
+  return rel(o, b, q) + hs * u;
 }
 template <class Real> __device__ __forceinline__ V3<Real> uvec(const SPos<Real>& s) { return V3<Real>{s.ux, s.uy, s.uz}; }
 

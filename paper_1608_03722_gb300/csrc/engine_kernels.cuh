@@ -129,7 +129,8 @@ struct GlobalSrc {
 // both base pairs of the step lie in a run of three or more open pairs, and
 // the bending when the pairs of o and of both its strand neighbours are open;
 // rule 2 also leaves out what the slot's removed bits (RM_SHIFT) mark and,
-// when `persist`, adds what it left out to them.
+// when `persist`, adds what it left out to them.  rm: the terms left out.
+
 // Terms of owner o that the bubble rule leaves out: bit 0 the dihedral, bit 1
 // the bending.  Out of line: it runs only with the rule on, and the step
 // kernel's common path keeps its registers.
@@ -148,19 +149,16 @@ __device__ __noinline__ unsigned bubble_bits(const KArgs<Real>& a, const Src src
   return r1;
 }
 
-template <class Real, bool EXT, class Src>
-__device__ __forceinline__ void owner_eval(const KArgs<Real>& a, const Src& src, int64_t o, int f, bool persist,
+template <class Real, class Src>
+__device__ __forceinline__ void owner_eval(const KArgs<Real>& a, const Src& src, int64_t o, int f, unsigned rm,
                                            unsigned& fl, Real* E, Real* W, OwnerOut<Real>& out) {
   const int dir = (o & 1) ? -2 : 2;   // strand A (even slot) runs up, strand B down
-  unsigned rm = 0u;
-  if constexpr (EXT) rm = a.bubble ? bubble_bits(a, src, o, f, persist) : 0u;
   const bool skip_dih = (rm & 1u) != 0, skip_bend = (rm & 2u) != 0;
   const SPos<Real> so = src.pos(o);
   const SPos<Real> sq = src.pos(src.step(o, dir));
   const Real h = a.c.h;
   const V3<Real> uo = uvec(so), uq = uvec(sq);
-  const V3<Real> Rq = rel(so, sq, a.fixq);
-  const V3<Real> bo = -h * uo, po = h * uo, bq = Rq - h * uq, pq = Rq + h * uq;
+  const V3<Real> bo = -h * uo, po = h * uo, bq = site_rel(so, sq, a.fixq, -h, uq), pq = site_rel(so, sq, a.fixq, h, uq);
   // FENE + WCA, Morse
   V3<Real> fb = t_fene(a.c, bq - bo, fl, E);
   out.nb += fb; out.sb -= fb;
@@ -181,7 +179,7 @@ __device__ __forceinline__ void owner_eval(const KArgs<Real>& a, const Src& src,
   if (W) { vir_add(W, po, f1); vir_add(W, bq, f2); vir_add(W, pq, -(f1 + f2)); }
   if ((f & F_PREV) && !skip_bend) {
     const SPos<Real> sr = src.pos(src.step(o, -dir));
-    const V3<Real> pr = rel(so, sr, a.fixq) + h * uvec(sr);
+    const V3<Real> pr = rel_site(so, sr, a.fixq, h, uvec(sr));
     V3<Real> g1, g2;
     t_bend(a.c, pr - po, pq - po, g1, g2, E);
     out.pp += g1; out.np += g2; out.sp -= (g1 + g2);
@@ -219,10 +217,11 @@ __device__ unsigned junction_pass(const KArgs<Real>& a, int cur) {
       Real E[NTERMS], W[6];
       for (int k = 0; k < NTERMS; ++k) E[k] = 0;
       for (int k = 0; k < 6; ++k) W[k] = 0;
-      owner_eval<Real, true>(a, src, o, f, false, fl, E, W, out);
+      owner_eval<Real>(a, src, o, f, a.bubble ? bubble_bits(a, src, o, f, false) : 0u, fl, E, W, out);
       flush_energy(a, mol, E, W);
     } else {
-      owner_eval<Real, true>(a, src, o, f, MODE == MODE_STEP, fl, (Real*)nullptr, (Real*)nullptr, out);
+      owner_eval<Real>(a, src, o, f, a.bubble ? bubble_bits(a, src, o, f, MODE == MODE_STEP) : 0u, fl, (Real*)nullptr,
+                       (Real*)nullptr, out);
     }
     Real* j = a.jout + 16 * t;
     const V3<Real> v[5] = {out.sb, out.sp, out.nb, out.np, out.pp};
@@ -273,7 +272,12 @@ __device__ __forceinline__ void owner_terms(const KArgs<Real>& a, const SegSmem<
     }
   }
   OwnerOut<Real> out{{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-  if (f & F_NEXT) owner_eval<Real, EXT>(a, RingSrc<Real>{sm.pos, sm.flg}, o, f, persist, fl, E, W, out);
+  if (f & F_NEXT) {
+    const RingSrc<Real> src{sm.pos, sm.flg};
+    unsigned rm = 0u;
+    if constexpr (EXT) rm = a.bubble ? bubble_bits(a, src, o, f, persist) : 0u;
+    owner_eval<Real>(a, src, o, f, rm, fl, E, W, out);
+  }
   store_owner(sm, ri, out);
 }
 
@@ -428,6 +432,39 @@ __device__ __forceinline__ int own_image(const KArgs<Real>& a, int cur, unsigned
   else return a.img[gu];
 }
 
+// Typed WCA force (App. A Eq. 11) on a bead from a partner: R the separation of
+// their centres (partner - own), um and uj their orientations, st2: both beads
+// steric; the bead separation and the pair energy go to *dout, *eout when
+// given.
+template <class Real>
+__device__ __forceinline__ V3<Real> pair_core(const KArgs<Real>& a, V3<Real> R, V3<Real> um, V3<Real> uj,
+                                              bool cross_strand, bool st2, V3<Real>* dout, Real* eout) {
+  const Real h = a.c.h;
+  // bead_j - bead_me; in FP32 formed as fma(h, u_me - u_j, R), which is
+  // antisymmetric bit for bit (the pair force from the partner's side is
+  // exactly its negative), as pair halving needs
+  V3<Real> d;
+  if constexpr (sizeof(Real) == 4) {
+    d = V3<Real>{fmaf(h, um.x - uj.x, R.x), fmaf(h, um.y - uj.y, R.y), fmaf(h, um.z - uj.z, R.z)};
+  } else {
+    d = R - h * uj + h * um;
+  }
+  // typed sigma (Sec. 2, reading A1): two steric beads (either strand) at
+  // sigma_ss, or at sigma_cross_steric across strands when that is set; any
+  // other pair across strands at sigma_cross
+  Real s2 = a.c.sss2, rc2 = a.c.rcss2;
+  if (cross_strand) {
+    const bool cs = st2 && a.c.scs2 > (Real)0;
+    s2 = cs ? a.c.scs2 : a.c.scr2;
+    rc2 = cs ? a.c.rccs2 : a.c.rccr2;
+  }
+  Real e;
+  const V3<Real> fw = t_wca(a.c, d, s2, rc2, &e);
+  if (dout) *dout = d;
+  if (eout) *eout = e;
+  return fw;
+}
+
 // Typed WCA force (App. A Eq. 11) on the bead of slot gu (staged record me,
 // orientation um, flags f, image word img_me) from its list entry ent; the
 // bead separation and the pair energy go to *dout, *eout when given.
@@ -435,7 +472,6 @@ template <class Real>
 __device__ __forceinline__ V3<Real> pair_force(const KArgs<Real>& a, int cur, unsigned gu, const SPos<Real>& me,
                                                V3<Real> um, int f, int img_me, int ent, V3<Real>* dout, Real* eout) {
   const unsigned ns = (unsigned)a.ns;
-  const Real h = a.c.h;
   const int j = ent & ENT_JMASK;
   V3<Real> R;
   V3<Real> uj;
@@ -461,32 +497,8 @@ __device__ __forceinline__ V3<Real> pair_force(const KArgs<Real>& a, int cur, un
       R.z += (double)(img_comp(img_me, 2) - img_comp(wj, 2) + ent_shift(ent, 2)) * a.L[2];
     }
   }
-  // bead_j - bead_me; in FP32 formed as fma(h, u_me - u_j, R), which is
-  // antisymmetric bit for bit (the pair force from the partner's side is
-  // exactly its negative), as pair halving needs
-  V3<Real> d;
-  if constexpr (sizeof(Real) == 4) {
-    d = V3<Real>{fmaf(h, um.x - uj.x, R.x), fmaf(h, um.y - uj.y, R.y), fmaf(h, um.z - uj.z, R.z)};
-  } else {
-    d = R - h * uj + h * um;
-  }
-  const bool cross_strand = ((gu ^ (unsigned)j) & 1u) != 0;
-  // typed sigma (Sec. 2, reading A1): two steric beads (either strand) at
-  // sigma_ss, or at sigma_cross_steric across strands when that is set; any
-  // other pair across strands at sigma_cross.  The partner's steric flag is
-  // bit 30 of its image word.
-  const bool st2 = (f & F_STERIC) && ((wj >> IMG_STERIC_SHIFT) & 1);
-  Real s2 = a.c.sss2, rc2 = a.c.rcss2;
-  if (cross_strand) {
-    const bool cs = st2 && a.c.scs2 > (Real)0;
-    s2 = cs ? a.c.scs2 : a.c.scr2;
-    rc2 = cs ? a.c.rccs2 : a.c.rccr2;
-  }
-  Real e;
-  const V3<Real> fw = t_wca(a.c, d, s2, rc2, &e);
-  if (dout) *dout = d;
-  if (eout) *eout = e;
-  return fw;
+  const bool st2 = (f & F_STERIC) && ((wj >> IMG_STERIC_SHIFT) & 1);   // the partner's steric flag: bit 30 of its image word
+  return pair_core(a, R, um, uj, ((gu ^ (unsigned)j) & 1u) != 0, st2, dout, eout);
 }
 
 // The list pairs of the tile's nucleotides B .. B+31 spread evenly over the
@@ -583,6 +595,97 @@ __device__ __forceinline__ void warp_pairs(const KArgs<Real>& a, const SegSmem<R
   }
 }
 
+// Hydrogen bond of patch me with its partner's (App. A Eq. 10), broken beyond
+// rc: d = patch_q - patch_me; false when broken, else k2 d is the force.
+template <class Real>
+__device__ __forceinline__ bool hbond(const KArgs<Real>& a, const SPos<Real>& me, const SPos<Real>& q, V3<Real> um, int f,
+                                      V3<Real>& d, Real& r2, Real& k2) {
+  const Real h = a.c.h;
+  d = site_rel(me, q, a.fixq, h, uvec(q)) - h * um;
+  r2 = dot(d, d);
+  if (!(r2 <= a.c.rchb2)) return false;
+  const Real khb = (f & F_GC) ? a.c.khb_gc : a.c.khb;   // Sec. 5: A.T / G.C stiffness
+  k2 = (Real)2 * khb;
+  if (a.c.r0hb != (Real)0) k2 *= (Real)1 - a.c.r0hb * rsqrt_(r2);
+  return true;
+}
+
+// Applied load on a nucleotide of the last base pair (Sec. 4.1, 4.2), q its
+// partner: f/2 at each centre, torque as a couple normal to its axis; half on
+// each site.
+template <class Real>
+__device__ __forceinline__ void add_load(const KArgs<Real>& a, int mol, const SPos<Real>& me, const SPos<Real>& q,
+                                         V3<Real>& Fb, V3<Real>& Fp) {
+  const double* ex = a.ext + 8 * mol;
+  V3<Real> Fe{(Real)(0.5 * ex[0]), (Real)(0.5 * ex[1]), (Real)(0.5 * ex[2])};
+  const V3<Real> Tq{(Real)ex[3], (Real)ex[4], (Real)ex[5]};
+  const Real tn2 = dot(Tq, Tq);
+  if (tn2 > (Real)0) {
+    const V3<Real> th = rsqrt_(tn2) * Tq;
+    V3<Real> rho = (Real)-0.5 * rel(me, q, a.fixq);   // centre offset from the pair centre
+    rho -= dot(rho, th) * th;
+    const Real S = (Real)2 * dot(rho, rho);
+    if (S > (Real)1e-12) Fe += ((Real)1 / S) * cross(Tq, rho);
+  }
+  Fb += (Real)0.5 * Fe;
+  Fp += (Real)0.5 * Fe;
+}
+
+// App. A Eq. 8 per site, friction -gamma v_s and noise eta_s, summed over the
+// dumbbell: force F and torque Tc about the centre become Ft, Tt.
+template <class Real>
+__device__ __forceinline__ void langevin(const KArgs<Real>& a, V3<Real> F, V3<Real> Tc, const double* Vd, V3<Real> Om,
+                                         V3<Real> um, V3<Real> eb, V3<Real> ep, V3<Real>& Ft, V3<Real>& Tt) {
+  V3<Real> Vh;
+  if constexpr (sizeof(Real) == 4) {
+    Vh = V3<Real>{d2f_bits(Vd[0]), d2f_bits(Vd[1]), d2f_bits(Vd[2])};
+  } else {
+    Vh = V3<Real>{Vd[0], Vd[1], Vd[2]};
+  }
+  Ft = F - a.c.gam2 * Vh + eb + ep;
+  Tt = Tc - a.c.gamr * Om + a.c.h * cross(um, ep - eb);
+}
+
+// Leapfrog kick and drift (Eq. 16) of a mobile nucleotide, FP64 accumulation of
+// V and X; un: the turned orientation.
+template <class Real>
+__device__ __forceinline__ void kick_drift(const KArgs<Real>& a, V3<Real> Ft, V3<Real> Tt, V3<Real> um, double* Xd,
+                                           double* Vd, V3<Real>& Om, V3<Real>& un, unsigned& fl) {
+  const V3<Real> dv = a.c.dtM * Ft;
+  if constexpr (sizeof(Real) == 4) {
+    Vd[0] += f2d_bits(dv.x); Vd[1] += f2d_bits(dv.y); Vd[2] += f2d_bits(dv.z);
+  } else {
+    Vd[0] += dv.x; Vd[1] += dv.y; Vd[2] += dv.z;
+  }
+  Om += a.c.dtI * Tt;
+  Om -= dot(Om, um) * um;
+  Xd[0] = fma(a.c.dt_d, Vd[0], Xd[0]);
+  Xd[1] = fma(a.c.dt_d, Vd[1], Xd[1]);
+  Xd[2] = fma(a.c.dt_d, Vd[2], Xd[2]);
+  const Real w2 = dot(Om, Om);
+  if (w2 > (Real)0) {
+    const Real w = sqrt_(w2);
+    Real sn, cs;
+    sincos_(w * a.c.dt, &sn, &cs);
+    const V3<Real> ax = ((Real)1 / w) * Om;
+    un = cs * um + sn * cross(ax, um);
+    un = rsqrt_(dot(un, un)) * un;
+  }
+  // a NaN or infinity in any component makes the sum non-finite
+  if (!isfinite((Ft.x + Ft.y) + (Ft.z + Om.x) + (Om.y + Om.z))) fl |= B_ENAN;
+}
+
+// Rebuild trigger: the bead with mirror k0, k1, k2 and orientation un has moved
+// more than skin/2 since the last build (reference kr).
+template <class Real>
+__device__ __forceinline__ bool moved(const KArgs<Real>& a, int k0, int k1, int k2, V3<Real> un, const int* kr) {
+  const float hf = (float)a.c.h;
+  const float ddx = (float)(int)((unsigned)(k0 + bead_off(hf * (float)un.x, a.fixSf[0])) - (unsigned)kr[0]) * a.fixq[0];
+  const float ddy = (float)(int)((unsigned)(k1 + bead_off(hf * (float)un.y, a.fixSf[1])) - (unsigned)kr[1]) * a.fixq[1];
+  const float ddz = (float)(int)((unsigned)(k2 + bead_off(hf * (float)un.z, a.fixSf[2])) - (unsigned)kr[2]) * a.fixq[2];
+  return ddx * ddx + ddy * ddy + ddz * ddz > a.c.skin_half2;
+}
+
 // Forces on nucleotide g from the owner rings, its H-bond and its list
 // pairs, then (MODE_STEP) its Langevin update; MODE_FORCES writes the site
 // forces, MODE_ENERGY adds its per-nucleotide energies and virial to Eb.
@@ -614,18 +717,15 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
       const int on = ring(g + dir);
       Fp += V3<Real>{sm.cp[0 * RING + on], sm.cp[1 * RING + on], sm.cp[2 * RING + on]};
     }
-    // hydrogen bond with the partner (App. A Eq. 10), broken beyond rc
+    // hydrogen bond with the partner
     {
-      const SPos<Real>& q = sm.pos[ring(g ^ 1)];
-      const V3<Real> d = rel(me, q, a.fixq) + h * uvec(q) - h * um;   // patch_q - patch_me
-      const Real r2 = dot(d, d);
-      if (r2 <= a.c.rchb2) {
-        const Real khb = (f & F_GC) ? a.c.khb_gc : a.c.khb;   // Sec. 5: A.T / G.C stiffness
-        Real k2 = (Real)2 * khb;
-        if (a.c.r0hb != (Real)0) k2 *= (Real)1 - a.c.r0hb * rsqrt_(r2);
+      V3<Real> d;
+      Real r2, k2;
+      if (hbond(a, me, sm.pos[ring(g ^ 1)], um, f, d, r2, k2)) {
         Fp += k2 * d;
         if constexpr (MODE == MODE_ENERGY) {
           if ((g & 1) == 0) {
+            const Real khb = (f & F_GC) ? a.c.khb_gc : a.c.khb;
             const Real r = sqrt_(r2);
             const Real rc = sqrt_(a.c.rchb2);
             Eb[2] += khb * ((r - a.c.r0hb) * (r - a.c.r0hb) - (rc - a.c.r0hb) * (rc - a.c.r0hb));
@@ -654,24 +754,7 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
       warp_pairs(a, sm, g, act, cur, Fb);
     }
     if (!act) return;
-    // applied load on the last base pair (Sec. 4.1, 4.2): f/2 at each centre,
-    // torque as a couple normal to its axis; half on each site
-    if (f & F_TOP) {
-      const int mol = f >> MOL_SHIFT;
-      const double* ex = a.ext + 8 * mol;
-      V3<Real> Fe{(Real)(0.5 * ex[0]), (Real)(0.5 * ex[1]), (Real)(0.5 * ex[2])};
-      const V3<Real> Tq{(Real)ex[3], (Real)ex[4], (Real)ex[5]};
-      const Real tn2 = dot(Tq, Tq);
-      if (tn2 > (Real)0) {
-        const V3<Real> th = rsqrt_(tn2) * Tq;
-        V3<Real> rho = (Real)-0.5 * rel(me, sm.pos[ring(g ^ 1)], a.fixq);   // centre offset from the pair centre
-        rho -= dot(rho, th) * th;
-        const Real S = (Real)2 * dot(rho, rho);
-        if (S > (Real)1e-12) Fe += ((Real)1 / S) * cross(Tq, rho);
-      }
-      Fb += (Real)0.5 * Fe;
-      Fp += (Real)0.5 * Fe;
-    }
+    if (f & F_TOP) add_load(a, f >> MOL_SHIFT, me, sm.pos[ring(g ^ 1)], Fb, Fp);
     if constexpr (MODE == MODE_FORCES) {
       double* o = a.fout + 6 * g;
       o[0] = Fb.x; o[1] = Fb.y; o[2] = Fb.z; o[3] = Fp.x; o[4] = Fp.y; o[5] = Fp.z;
@@ -699,17 +782,9 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
       const bool frozen = (f & F_FROZEN) != 0;
       V3<Real> Ft{0, 0, 0}, Tt{0, 0, 0};
       if (!frozen) {
-        // App. A Eq. 8 per site: friction -gamma v_s and noise eta_s, summed over the dumbbell
         V3<Real> eb, ep;
         nucleotide_noise(a, local, step, mol, eb, ep);
-        V3<Real> Vh;
-        if constexpr (sizeof(Real) == 4) {
-          Vh = V3<Real>{d2f_bits(Vd[0]), d2f_bits(Vd[1]), d2f_bits(Vd[2])};
-        } else {
-          Vh = V3<Real>{Vd[0], Vd[1], Vd[2]};
-        }
-        Ft = F - a.c.gam2 * Vh + eb + ep;
-        Tt = Tc - a.c.gamr * Om + h * cross(um, ep - eb);
+        langevin(a, F, Tc, Vd, Om, um, eb, ep, Ft, Tt);
       }
       if constexpr (MODE == MODE_ENERGY) {
         if (!frozen) {
@@ -721,31 +796,9 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
           Eb[9] += (Real)0.5 * a.c.I * dot(Of, Of);
         }
       } else {
-        // MODE_STEP: leapfrog kick and drift (Eq. 16), FP64 accumulation of V and X
         V3<Real> un = um;
         if (!frozen) {
-          const V3<Real> dv = a.c.dtM * Ft;
-          if constexpr (sizeof(Real) == 4) {
-            Vd[0] += f2d_bits(dv.x); Vd[1] += f2d_bits(dv.y); Vd[2] += f2d_bits(dv.z);
-          } else {
-            Vd[0] += dv.x; Vd[1] += dv.y; Vd[2] += dv.z;
-          }
-          Om += a.c.dtI * Tt;
-          Om -= dot(Om, um) * um;
-          Xd[0] = fma(a.c.dt_d, Vd[0], Xd[0]);
-          Xd[1] = fma(a.c.dt_d, Vd[1], Xd[1]);
-          Xd[2] = fma(a.c.dt_d, Vd[2], Xd[2]);
-          const Real w2 = dot(Om, Om);
-          if (w2 > (Real)0) {
-            const Real w = sqrt_(w2);
-            Real sn, cs;
-            sincos_(w * a.c.dt, &sn, &cs);
-            const V3<Real> ax = ((Real)1 / w) * Om;
-            un = cs * um + sn * cross(ax, um);
-            un = rsqrt_(dot(un, un)) * un;
-          }
-          // a NaN or infinity in any component makes the sum non-finite
-          if (!isfinite((Ft.x + Ft.y) + (Ft.z + Om.x) + (Om.y + Om.z))) fl |= B_ENAN;
+          kick_drift(a, Ft, Tt, um, Xd, Vd, Om, un, fl);
           a.V[gu] = Vd[0]; a.V[ns + gu] = Vd[1]; a.V[2 * ns + gu] = Vd[2];
           a.Om[gu] = Om.x; a.Om[ns + gu] = Om.y; a.Om[2 * ns + gu] = Om.z;
           if constexpr (sizeof(Real) == 4) {
@@ -755,12 +808,7 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
         // the new position's mirror (in the FP64 path it serves the rebuild trigger only)
         const int k0 = fixs(Xd[0], a.fixS[0]), k1 = fixs(Xd[1], a.fixS[1]), k2 = fixs(Xd[2], a.fixS[2]);
         store_state(a, nxt, g, k0, k1, k2, Xd, un, packed);
-        // rebuild trigger: a bead moved more than skin/2 since the last build
-        const float hf = (float)h;
-        const float ddx = (float)(int)((unsigned)(k0 + bead_off(hf * (float)un.x, a.fixSf[0])) - (unsigned)kr[0]) * a.fixq[0];
-        const float ddy = (float)(int)((unsigned)(k1 + bead_off(hf * (float)un.y, a.fixSf[1])) - (unsigned)kr[1]) * a.fixq[1];
-        const float ddz = (float)(int)((unsigned)(k2 + bead_off(hf * (float)un.z, a.fixSf[2])) - (unsigned)kr[2]) * a.fixq[2];
-        if (ddx * ddx + ddy * ddy + ddz * ddz > a.c.skin_half2) fl |= B_STALE;
+        if (moved(a, k0, k1, k2, un, kr)) fl |= B_STALE;
       }
     }
   }

@@ -6,6 +6,7 @@
 #include "engine_kernels.cuh"
 #include "rebuild.cuh"
 #include "chainlist.cuh"
+#include "resident.cuh"
 
 namespace dsdna {
 
@@ -60,6 +61,51 @@ cudaError_t engine_launch(int mode, const KArgs<Real>& a, int grid, int T, size_
   // the instance chosen by mode, launched with its parameter block
   void* args[] = {const_cast<KArgs<Real>*>(&a)};
   return cudaLaunchKernelExC(&cfg, engine_fn<Real>(mode), args);
+}
+
+// Launch shape of the resident kernel: blocks, threads and shared memory for n
+// slots (0 blocks: a stretch would be longer than a CTA holds).  One stretch of
+// whole segments per SM; warps for all owners and pairs of the stretch at once
+// (about two warps per 32 slots), at least one thread per slot.
+template <class Real>
+cudaError_t resident_shape(int64_t n, int rings, bool ext, int nsm, int* grid, int* T, size_t* smem) {
+  const int64_t nu = (n + SEG_W - 1) / SEG_W;
+  *grid = (int)std::max<int64_t>(1, std::min<int64_t>(nsm, nu));
+  const int64_t len = SEG_W * ((nu + *grid - 1) / *grid);
+  if (nsm < 1 || nsm > 1023 || len > res_max_len<Real>()) {
+    *grid = 0;
+    return cudaSuccess;
+  }
+  const int tiles = (int)(len + 31) / 32;
+  *T = 32 * std::min(res_max_threads<Real>() / 32, 2 * tiles + 2);
+  *smem = res_layout<Real>((int)len, rings, *T).bytes;
+  const void* fn = ext ? (const void*)resident_kernel<Real, true> : (const void*)resident_kernel<Real, false>;
+  // the attribute is per kernel, shared by every context: the largest any may use
+  const size_t most = res_layout<Real>(res_max_len<Real>(), 1, res_max_threads<Real>()).bytes;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  int bps = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, *T, *smem);
+  if (e == cudaSuccess && bps < 1) *grid = 0;
+  return e;
+}
+
+// Steps of a small system (mode as engine_launch's, MODE_STEP).
+template <class Real>
+cudaError_t resident_launch(int mode, const KArgs<Real>& a, int grid, int T, size_t smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)T);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ResLayout lay = res_layout<Real>((int)(SEG_W * ((a.nseg16 + grid - 1) / grid)), a.n_junc > 0, T);
+  void* args[] = {const_cast<KArgs<Real>*>(&a), &lay};
+  const void* fn = (mode & MODE_EXT) ? (const void*)resident_kernel<Real, true> : (const void*)resident_kernel<Real, false>;
+  return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 // Kernel attributes of the rebuild kernels for the current device, set when a

@@ -1,0 +1,665 @@
+// resident.cuh -- step kernel of small systems: every CTA keeps its stretch of
+// the chain in shared memory and registers from step to step.  Included by
+// kern_launch.cuh after engine_kernels.cuh and chainlist.cuh.
+//
+// Up to 512 nucleotides per SM (256 in FP64) the strip kernel (engine_kernel)
+// waits rather than works: a warp walks one tile by itself through a chain of
+// memory latencies and two passes of bonded terms (its prologue's and its
+// own), reloads the whole state every step, and a stale list costs five more
+// grid barriers and a cell walk.  Here
+//  * the CTAs split the chain into stretches of whole 16-slot segments, one
+//    CTA per SM; positions and flags of the stretch live in shared memory,
+//    X, V, Omega and the rebuild reference of a nucleotide in its thread's
+//    registers, so a step reads only the few slots beyond its ends and the
+//    list partners of other stretches;
+//  * owners and list pairs are dealt to the warps together (they need only
+//    positions), one block barrier later every nucleotide adds its forces and
+//    moves, and the noise of the next step is drawn while the grid barrier
+//    completes;
+//  * the grid barrier is one release add and one acquire poll on a word that
+//    also counts the stale flags;
+//  * a rebuild is one phase that bins the beads and threads each 16-slot
+//    segment into a hash of cells (linked lists, no table scan), one grid
+//    barrier, and the chain-window list build of the CTA's own beads, whose
+//    result stays in shared memory.
+// All forces, sums and updates are those of engine_kernel, term by term in the
+// same order, so trajectories agree bit for bit.  100 steps and one state
+// download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1960 ->
+// 847 us, periodic walk of 30 kbp 2241 -> 1140 us, 64 rings of 500 bp 3463 ->
+// 2029 us; 50 FP64 steps of 200 bp 3733 -> 1298 us (a warp per SM instead of
+// eight sharing one SM's FP64 pipe).
+#pragma once
+#include "chainlist.cuh"
+#include "engine_kernels.cuh"
+
+namespace dsdna {
+
+template <class Real> __host__ __device__ constexpr int res_max_len() { return sizeof(Real) == 4 ? 512 : 256; }
+template <class Real> __host__ __device__ constexpr int res_max_threads() { return res_max_len<Real>(); }
+constexpr int RES_PAIRS_PER_SLOT = 4;   // list entries kept in shared memory per slot (else the lists are walked in memory)
+
+// Shared-memory layout of a CTA whose stretch holds at most `len` slots.
+struct ResLayout {
+  int len, own, pairs, warps;
+  size_t pos, flg, cs, cn, cp, pf, ent, off, po, jx, xo, list, win, gi, gc, bytes;
+};
+template <class Real>
+__host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
+  ResLayout l;
+  l.len = len;
+  l.own = len + 4 + (rings ? len / 3 + 8 : 0);   // owners of a stretch, and those across the junctions of its rings
+  l.pairs = RES_PAIRS_PER_SLOT * len + 64;
+  l.warps = T / 32;
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o = (o + bytes + 15) & ~(size_t)15;
+    return at;
+  };
+  l.pos = take(sizeof(SPos<Real>) * len);
+  l.cs = take(sizeof(Real) * 6 * l.own);
+  l.cn = take(sizeof(Real) * 6 * l.own);
+  l.cp = take(sizeof(Real) * 3 * l.own);
+  l.pf = take(sizeof(Real) * 3 * l.pairs);
+  l.win = take(sizeof(float4) * (CL_WIN + CL_WIN / 16) * l.warps);
+  l.gc = take(sizeof(float4) * 4 * l.warps);
+  l.gi = take(sizeof(int) * 4 * l.warps);
+  l.flg = take(sizeof(int) * len);
+  l.ent = take(sizeof(int) * l.pairs);
+  l.off = take(sizeof(int) * (len + 33));
+  l.xo = take(sizeof(int) * (rings ? len / 3 + 8 : 0));
+  l.list = take(sizeof(int) * 32 * LIST_CAP * l.warps);
+  l.po = take(sizeof(unsigned short) * l.pairs);
+  l.jx = take(sizeof(short) * len);
+  l.bytes = o;
+  return l;
+}
+
+// ---------------------------------------------------------------- grid barrier
+// Barrier number k of a launch counts on word k mod 3 of bar->acc: arrivals in
+// bits 0-9, stale stretches in bits 10-19, stretches with an error in bits
+// 20-29 (their bits are in bar->gen).  The word of barrier k - 1 is cleared
+// after barrier k by block 0, two barriers before it is used again.  Returns
+// the flags, or B_ETIMEOUT when the clock budget runs out.
+__device__ __forceinline__ void res_arrive(GridBar* bar, unsigned k, unsigned fl) {
+  if (fl & B_ERRMASK) {
+    atomicOr(&bar->gen, fl & B_ERRMASK);
+    __threadfence();
+  }
+  const unsigned v = 1u | ((fl & B_STALE) ? 1u << 10 : 0u) | ((fl & B_ERRMASK) ? 1u << 20 : 0u);
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&bar->acc[k % 3]), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned res_wait(GridBar* bar, unsigned k, unsigned nblocks, unsigned long long budget) {
+  const unsigned long long t0 = clock64();
+  unsigned v;
+  while (((v = ld_acquire(&bar->acc[k % 3])) & 1023u) != nblocks)
+    if ((unsigned long long)(clock64() - t0) > budget) return B_ETIMEOUT;
+  if (blockIdx.x == 0) bar->acc[(k + 2) % 3] = 0u;
+  unsigned r = ((v >> 10) & 1023u) ? B_STALE : 0u;
+  if (v >> 20) r |= ld_acquire(&bar->gen);
+  return r;
+}
+
+// ---------------------------------------------------------------- neighbourhood of an owner
+// Slots of the CTA's stretch from shared memory, others from global memory;
+// junction owners of circular molecules (wrap) take their neighbours modulo
+// the molecule.
+template <class Real>
+struct ResSrc {
+  const KArgs<Real>& a;
+  const SPos<Real>* spos;
+  const int* flg;
+  int cur;
+  int64_t s0;
+  int len;
+  bool wrap;
+  int64_t off, N;   // base-pair offset and length of the owner's molecule (wrap only)
+  __device__ __forceinline__ int64_t bp(int64_t k) const {
+    if (!wrap) return k;
+    const int64_t r = (k - off) % N;
+    return off + (r < 0 ? r + N : r);
+  }
+  __device__ __forceinline__ SPos<Real> pos(int64_t g) const {
+    const unsigned l = (unsigned)(g - s0);
+    if (l < (unsigned)len) return spos[l];
+    SPos<Real> s;
+    load_slot(a, cur, g, s);
+    return s;
+  }
+  __device__ __forceinline__ int64_t step(int64_t g, int d) const {
+    return wrap ? 2 * bp((g >> 1) + d / 2) + (g & 1) : g + d;
+  }
+  __device__ __forceinline__ bool open(int64_t k, int mol) const {
+    k = bp(k);
+    const unsigned l = (unsigned)(2 * k - s0);
+    if (l < (unsigned)len) {
+      const int f = flg[l];
+      return (f & F_OPEN) && (f >> MOL_SHIFT) == mol;
+    }
+    if (k < 0 || 2 * k >= a.n || (a.topo[2 * k] >> MOL_SHIFT) != mol) return false;
+    const SPos<Real> pa = pos(2 * k), pb = pos(2 * k + 1);
+    const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
+    return dot(d, d) > a.c.rchb2;
+  }
+};
+
+// ---------------------------------------------------------------- list build
+constexpr unsigned RES_NONE = 0xffffffffu;
+
+// Bucket of neighbour q (0..26; 13 is the cell itself) of cell ci.
+template <class Real>
+__device__ __forceinline__ unsigned res_key(const KArgs<Real>& a, int mol, const int* ci, int q) {
+  int cc[3] = {ci[0] + q % 3 - 1, ci[1] + (q / 3) % 3 - 1, ci[2] + q / 9 - 1};
+  if (a.periodic)
+    for (int c = 0; c < 3; ++c) cc[c] = cc[c] < 0 ? cc[c] + a.sg_nc[c] : (cc[c] >= a.sg_nc[c] ? cc[c] - a.sg_nc[c] : cc[c]);
+  return hash_block(mol, cc[0], cc[1], cc[2]) & a.rs_mask;
+}
+
+// Grid item `id` (a segment, or bead id - nseg16 of a wide one) to the front of
+// its cell's list; a head of an earlier rebuild (another epoch) is an empty list.
+template <class Real>
+__device__ __forceinline__ void res_insert(const KArgs<Real>& a, int mol, const float* p, unsigned id, unsigned epoch) {
+  int ci[3];
+  seg_cell(a, p[0], p[1], p[2], ci);
+  const unsigned long long old =
+      atomicExch(a.rs_head + res_key(a, mol, ci, 13), ((unsigned long long)epoch << 32) | id);
+  a.rs_next[id] = (unsigned)(old >> 32) == epoch ? (unsigned)old : RES_NONE;
+}
+
+// Lists of the `nb` (16 or 32) beads from slot g0 on, one lane per bead.
+template <class Real>
+__device__ __forceinline__ void res_list(const KArgs<Real>& a, int64_t g0, int nb, unsigned epoch, float4* win, int* gi,
+                                         float4* gc, int* list, int& cnt, int& total) {
+  const int lane = threadIdx.x & 31;
+  const int g = (int)g0 + lane;
+  const bool in = lane < nb && g < a.n;
+  float4 raw[2];
+  int word[2];
+  bool val[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int64_t j = g0 - 16 + lane + 32 * h;
+    val[h] = j >= 0 && j < a.n;
+    raw[h] = val[h] ? a.wpos[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    word[h] = val[h] ? ((a.topo[j] & F_STERIC) | CL_VALID) : 0;
+  }
+  const int64_t sA = g0 / SEG_W;
+  const bool hasB = nb > 16 && sA + 1 < a.nseg16;
+  const float4 sc[2] = {a.segc[sA], hasB ? a.segc[sA + 1] : make_float4(0.0f, 0.0f, 0.0f, -1.0f)};
+  const float4 mp = in ? a.wpos[g] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  // molecule of each segment (staged slots 16 and 32) and its slot range
+  const int qmol[2] = {__shfl_sync(0xffffffffu, __float_as_int(raw[0].w), 16),
+                       __shfl_sync(0xffffffffu, __float_as_int(raw[1].w), 0)};
+  // the cell lists around both segments: each lane walks one cell of either (a
+  // bucket that a lower lane of the same segment also reads is dropped)
+  unsigned id[2] = {RES_NONE, RES_NONE};
+  unsigned key[2] = {RES_NONE, RES_NONE};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (lane < 27 && sc[h].w >= 0.0f) {
+      int ci[3];
+      seg_cell(a, sc[h].x, sc[h].y, sc[h].z, ci);
+      key[h] = res_key(a, qmol[h], ci, lane);
+    }
+    const unsigned same = __match_any_sync(0xffffffffu, key[h]);
+    if (key[h] != RES_NONE && __ffs(same) - 1 == lane) {
+      const unsigned long long e = a.rs_head[key[h]];
+      if ((unsigned)(e >> 32) == epoch) id[h] = (unsigned)e;
+    }
+  }
+  int64_t slo[2] = {0, 0}, shi[2] = {a.n, a.n};
+  if (a.n_mol > 1) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (h == 0 || hasB) {
+        slo[h] = 2 * a.mol_off[qmol[h]];
+        shi[h] = 2 * a.mol_off[qmol[h] + 1];
+      }
+  }
+  const bool fast = cl_stage(a, lane, raw, word, val, win);
+  bool st_g = false;
+  cl_window(a, g0, lane, in, fast, win, st_g, list, cnt, total);
+  __syncwarp();
+  const unsigned most = (unsigned)(a.nseg16 + a.n);   // items there are at most
+  for (unsigned walked = 0; walked <= most && __any_sync(0xffffffffu, id[0] != RES_NONE || id[1] != RES_NONE); ++walked) {
+    const int hq = id[0] != RES_NONE ? 0 : 1;
+    const unsigned e = hq ? id[1] : id[0];
+    bool acc = false;
+    int ir = 0;
+    float4 it = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (e != RES_NONE) {
+      const unsigned nx = a.rs_next[e];
+      if (hq) id[1] = nx; else id[0] = nx;
+      if (e < (unsigned)a.nseg16) {
+        it = a.segc[e];
+        const int64_t b0 = (int64_t)e * SEG_W;
+        ir = (int)b0 | (((int)min((int64_t)SEG_W, a.n - b0) - 1) << ENT_J_BITS);
+      } else {
+        const float4 p = a.wpos[e - (unsigned)a.nseg16];
+        it = make_float4(p.x, p.y, p.z, 0.0f);
+        ir = (int)(e - (unsigned)a.nseg16);
+      }
+      const int64_t j0 = ir & ENT_JMASK, js = j0 / SEG_W, s = sA + hq;
+      const int64_t lo_h = hq ? slo[1] : slo[0], hi_h = hq ? shi[1] : shi[0];
+      if (j0 >= lo_h && j0 < hi_h && (js > s + 1 || js < s - 1)) acc = cl_spheres_meet(a, hq ? sc[1] : sc[0], it);
+    }
+    cl_items(a, lane, g, in, st_g, sc, mp, acc, hq, ir, it, win, gi, gc, list, cnt, total);
+  }
+  // a wide segment: each of its beads queries its own 27 cells
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (!(in && (lane >> 4) == h && (h == 0 || hasB) && sc[h].w < 0.0f)) continue;
+    const int64_t s = sA + h;
+    int ci[3];
+    seg_cell(a, mp.x, mp.y, mp.z, ci);
+    const int pmol = __float_as_int(mp.w);
+    const int64_t plo = a.n_mol > 1 ? 2 * a.mol_off[pmol] : 0, phi = a.n_mol > 1 ? 2 * a.mol_off[pmol + 1] : a.n;
+    const float4 pt = make_float4(mp.x, mp.y, mp.z, 0.0f);
+    for (int q = 0; q < 27; ++q) {
+      const unsigned k = res_key(a, pmol, ci, q);
+      bool dup = false;
+      for (int o = 0; o < q; ++o) dup = dup || res_key(a, pmol, ci, o) == k;
+      if (dup) continue;
+      const unsigned long long hd = a.rs_head[k];
+      unsigned walked = 0;
+      for (unsigned e = (unsigned)(hd >> 32) == epoch ? (unsigned)hd : RES_NONE; e != RES_NONE && walked <= most;
+           e = a.rs_next[e], ++walked) {
+        const bool seg = e < (unsigned)a.nseg16;
+        const int64_t j0 = seg ? (int64_t)e * SEG_W : (int64_t)(e - (unsigned)a.nseg16), js = j0 / SEG_W;
+        if (j0 < plo || j0 >= phi || (js <= s + 1 && js >= s - 1)) continue;
+        float4 it;
+        int ir = (int)j0;
+        if (seg) {
+          it = a.segc[e];
+          ir |= ((int)min((int64_t)SEG_W, a.n - j0) - 1) << ENT_J_BITS;
+        } else {
+          const float4 p = a.wpos[j0];
+          it = make_float4(p.x, p.y, p.z, 0.0f);
+        }
+        if (cl_spheres_meet(a, pt, it)) cl_item_pairs(a, g, mp, st_g, ir, list, cnt, total);
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// ---------------------------------------------------------------- the kernel
+// Bound by latency: a step is the grid barrier, one pass of owners and pairs
+// out of shared memory and one pass of updates.
+template <class Real, bool EXT>
+__global__ void __launch_bounds__(res_max_threads<Real>(), 1)
+    resident_kernel(const __grid_constant__ KArgs<Real> a, const __grid_constant__ ResLayout lay) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ unsigned s_fl[2], s_word;
+  __shared__ int s_scan[33], s_nx;
+  SPos<Real>* const spos = reinterpret_cast<SPos<Real>*>(sm + lay.pos);
+  int* const flg = reinterpret_cast<int*>(sm + lay.flg);
+  Real* const cs = reinterpret_cast<Real*>(sm + lay.cs);
+  Real* const cn = reinterpret_cast<Real*>(sm + lay.cn);
+  Real* const cp = reinterpret_cast<Real*>(sm + lay.cp);
+  Real* const pf = reinterpret_cast<Real*>(sm + lay.pf);
+  int* const ent = reinterpret_cast<int*>(sm + lay.ent);
+  int* const off = reinterpret_cast<int*>(sm + lay.off);
+  unsigned short* const po = reinterpret_cast<unsigned short*>(sm + lay.po);
+  short* const jx = reinterpret_cast<short*>(sm + lay.jx);
+  int* const xo = reinterpret_cast<int*>(sm + lay.xo);
+  const int OC = lay.own;
+  const unsigned ns = (unsigned)a.ns;
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nwarp = (int)(blockDim.x >> 5);
+  int* const list = reinterpret_cast<int*>(sm + lay.list) + (warp * 32 + lane) * LIST_CAP;
+  float4* const win = reinterpret_cast<float4*>(sm + lay.win) + warp * (CL_WIN + CL_WIN / 16);
+  int* const gi = reinterpret_cast<int*>(sm + lay.gi) + warp * 4;
+  float4* const gc = reinterpret_cast<float4*>(sm + lay.gc) + warp * 4;
+
+  // the CTA's stretch, and the nucleotide of this thread
+  const int64_t s0 = SEG_W * ((int64_t)blockIdx.x * a.nseg16 / gridDim.x);
+  const int64_t s1 = min(a.n, SEG_W * ((int64_t)(blockIdx.x + 1) * a.nseg16 / gridDim.x));
+  const int len = (int)(s1 - s0);
+  const bool mine = i < len;
+  const int64_t g = s0 + i;
+  const unsigned gu = (unsigned)(mine ? g : s0);
+
+  const int64_t step0 = *a.step;
+  int64_t budget = a.steps_left ? *a.steps_left : a.nsteps;
+  if (*a.err & B_ERRMASK) budget = 0;
+  unsigned epoch = (unsigned)*a.nrebuild;
+  int cur = (int)(step0 & 1);
+
+  // state into registers and shared memory
+  double Xd[3] = {0, 0, 0}, Vd[3] = {0, 0, 0};
+  V3<Real> Om{0, 0, 0};
+  int kr[3] = {0, 0, 0}, packed = 0, f = 0;
+  if (mine) {
+    SPos<Real> me;
+    load_slot(a, cur, g, me);
+    spos[i] = me;
+    f = a.topo[gu];
+    flg[i] = f;
+    if constexpr (sizeof(Real) == 4) {
+      Xd[0] = a.X[gu]; Xd[1] = a.X[ns + gu]; Xd[2] = a.X[2 * ns + gu];
+      packed = a.Kw[(unsigned)cur * ns + gu].w;
+    } else {
+      Xd[0] = me.x; Xd[1] = me.y; Xd[2] = me.z;
+    }
+    Vd[0] = a.V[gu]; Vd[1] = a.V[ns + gu]; Vd[2] = a.V[2 * ns + gu];
+    Om = V3<Real>{a.Om[gu], a.Om[ns + gu], a.Om[2 * ns + gu]};
+    kr[0] = a.kref[gu]; kr[1] = a.kref[ns + gu]; kr[2] = a.kref[2 * ns + gu];
+  }
+  const int mol = f >> MOL_SHIFT;
+  const bool frozen = (f & F_FROZEN) != 0;
+  const uint32_t local = mine ? (uint32_t)(g - 2 * a.mol_off[mol]) : 0u;
+  if (i == 0) { s_fl[0] = 0u; s_fl[1] = 0u; s_nx = 0; }
+  __syncthreads();
+  if constexpr (EXT) {
+    // circular molecules: the end nucleotides of a strand also take the forces
+    // of the owner across the junction, evaluated here a second time
+    if (a.n_junc && mine) {
+      jx[i] = -1;
+      if (f & F_JUNC) {
+        const int64_t k0 = a.mol_off[mol], k1 = a.mol_off[mol + 1] - 1, k = g >> 1;
+        if (k == k0 || k == k1) {
+          const int x = atomicAdd(&s_nx, 1);
+          jx[i] = (short)x;
+          xo[x] = (int)(2 * (k == k0 ? k1 : k0) + (g & 1));
+        }
+      }
+    }
+    if (a.bubble && mine && !(i & 1)) {
+      const SPos<Real> pa = spos[i], pb = spos[i + 1];
+      const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
+      if (dot(d, d) > a.c.rchb2) flg[i] = f | F_OPEN;
+    }
+  }
+
+  // offsets of the nucleotides' list entries in the CTA's pair table (block scan)
+  int npair = 0;
+  auto number_pairs = [&](int cnt) {
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_scan[warp] = incl;
+    __syncthreads();
+    int before = 0, tot = 0;
+    for (int w = 0; w < nwarp; ++w) {
+      if (w == warp) before = tot;
+      tot += s_scan[w];
+    }
+    if (mine) off[i] = before + incl - cnt;
+    if (i == 0) off[len] = tot;
+    npair = tot;
+    __syncthreads();
+  };
+  auto keep_entry = [&](int q, int e) {
+    const int p = off[i] + q;
+    if (p < lay.pairs) { ent[p] = e; po[p] = (unsigned short)i; }
+  };
+  {
+    const int cnt = mine ? a.ncnt[gu] : 0;
+    number_pairs(cnt);
+    for (int q = 0; q < cnt; ++q) keep_entry(q, a.nbr[(unsigned)q * ns + gu]);
+  }
+  const int nx = EXT ? s_nx : 0;
+  const int nown = len + 4 + nx;
+  V3<Real> eb{0, 0, 0}, ep{0, 0, 0};
+  if (mine && !frozen && budget > 0) nucleotide_noise(a, local, step0, mol, eb, ep);
+  __syncthreads();
+
+  int64_t done = 0;
+  unsigned errbits = 0, pend = 0, phase = 0;
+  for (int64_t it = 0; it < budget; ++it) {
+    cur = (int)((step0 + it) & 1);
+    const int nxt = cur ^ 1;
+    unsigned fl = pend;
+    pend = 0;
+    // owners and list pairs, 32 at a time to the warps
+    const int nco = (nown + 31) >> 5, ncp = npair <= lay.pairs ? (npair + 31) >> 5 : 0;
+    for (int c = warp; c < nco + ncp; c += nwarp) {
+      if (c < nco) {
+        const int w = 32 * c + lane;
+        if (w >= nown) continue;
+        const bool extra = EXT && w >= len + 4;
+        const int64_t o = extra ? (int64_t)xo[w - (len + 4)] : s0 - 2 + w;
+        const bool home = w >= 2 && w < len + 2;
+        OwnerOut<Real> out{{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+        if (o >= 0 && o < a.n) {
+          const unsigned lo = (unsigned)(o - s0);
+          int fo = lo < (unsigned)len ? flg[lo] : a.topo[o];
+          ResSrc<Real> src{a, spos, flg, cur, s0, len, false, 0, 0};
+          if constexpr (EXT) {
+            if (fo & F_JUNC) {   // both neighbours exist on a ring
+              fo |= F_PREV | F_NEXT;
+              src.wrap = true;
+              src.off = a.mol_off[fo >> MOL_SHIFT];
+              src.N = a.mol_off[(fo >> MOL_SHIFT) + 1] - src.off;
+            }
+          }
+          if (fo & F_NEXT) {
+            unsigned rm = 0u;
+            if constexpr (EXT) {
+              if (a.bubble) {
+                rm = bubble_bits(a, src, o, fo, home);
+                if (home && rm) atomicOr(&flg[lo], (int)(rm << RM_SHIFT));   // as in the topology word
+              }
+            }
+            owner_eval<Real>(a, src, o, fo, rm, fl, (Real*)nullptr, (Real*)nullptr, out);
+          }
+        }
+        cs[0 * OC + w] = out.sb.x; cs[1 * OC + w] = out.sb.y; cs[2 * OC + w] = out.sb.z;
+        cs[3 * OC + w] = out.sp.x; cs[4 * OC + w] = out.sp.y; cs[5 * OC + w] = out.sp.z;
+        cn[0 * OC + w] = out.nb.x; cn[1 * OC + w] = out.nb.y; cn[2 * OC + w] = out.nb.z;
+        cn[3 * OC + w] = out.np.x; cn[4 * OC + w] = out.np.y; cn[5 * OC + w] = out.np.z;
+        cp[0 * OC + w] = out.pp.x; cp[1 * OC + w] = out.pp.y; cp[2 * OC + w] = out.pp.z;
+      } else {
+        const int p = 32 * (c - nco) + lane;
+        if (p >= npair) continue;
+        const int e = ent[p], b = po[p], j = e & ENT_JMASK;
+        const SPos<Real> me = spos[b];
+        const unsigned l = (unsigned)(j - (int)s0);
+        V3<Real> fw;
+        if ((sizeof(Real) == 4 || !a.periodic) && l < (unsigned)len) {   // partner in the stretch: no memory access
+          const SPos<Real> q = spos[l];
+          fw = pair_core(a, rel(me, q, a.fixq), uvec(me), uvec(q), ((b ^ (int)l) & 1) != 0,
+                         ((flg[b] & flg[l]) & F_STERIC) != 0, (V3<Real>*)nullptr, (Real*)nullptr);
+        } else {
+          const unsigned gb = (unsigned)s0 + (unsigned)b;
+          const int img = (sizeof(Real) == 8 && a.periodic) ? own_image(a, cur, gb) : 0;
+          fw = pair_force(a, cur, gb, me, uvec(me), flg[b], img, e, (V3<Real>*)nullptr, (Real*)nullptr);
+        }
+        Real* o = pf + 3 * p;
+        o[0] = fw.x; o[1] = fw.y; o[2] = fw.z;
+      }
+    }
+    __syncthreads();
+    // every nucleotide: forces in the order of nucleotide_pass, then its step
+    SPos<Real> nw;
+    if (mine) {
+      const SPos<Real> me = spos[i], q = spos[i ^ 1];
+      const Real h = a.c.h;
+      const V3<Real> um = uvec(me);
+      const int w = i + 2, dir = (i & 1) ? -2 : 2;
+      V3<Real> Fb{cs[0 * OC + w], cs[1 * OC + w], cs[2 * OC + w]};
+      V3<Real> Fp{cs[3 * OC + w], cs[4 * OC + w], cs[5 * OC + w]};
+      if constexpr (EXT) {
+        if ((f & F_JUNC) && jx[i] >= 0) {   // the owner across the junction: the previous or the next one
+          const int x = len + 4 + jx[i];
+          const bool first = (i & 1) ? g >> 1 != a.mol_off[mol] : g >> 1 == a.mol_off[mol];
+          if (first) {
+            Fb += V3<Real>{cn[0 * OC + x], cn[1 * OC + x], cn[2 * OC + x]};
+            Fp += V3<Real>{cn[3 * OC + x], cn[4 * OC + x], cn[5 * OC + x]};
+          } else {
+            Fp += V3<Real>{cp[0 * OC + x], cp[1 * OC + x], cp[2 * OC + x]};
+          }
+        }
+      }
+      if (f & F_PREV) {
+        const int op = w - dir;
+        Fb += V3<Real>{cn[0 * OC + op], cn[1 * OC + op], cn[2 * OC + op]};
+        Fp += V3<Real>{cn[3 * OC + op], cn[4 * OC + op], cn[5 * OC + op]};
+      }
+      if (f & F_NEXT) {
+        const int on = w + dir;
+        Fp += V3<Real>{cp[0 * OC + on], cp[1 * OC + on], cp[2 * OC + on]};
+      }
+      {
+        V3<Real> d;
+        Real r2, k2;
+        if (hbond(a, me, q, um, f, d, r2, k2)) Fp += k2 * d;
+      }
+      if (npair <= lay.pairs) {
+        for (int p = off[i], p1 = off[i + 1]; p < p1; ++p) Fb += V3<Real>{pf[3 * p], pf[3 * p + 1], pf[3 * p + 2]};
+      } else {   // more entries than the table holds: this nucleotide's list, from memory
+        const int img = (sizeof(Real) == 8 && a.periodic) ? own_image(a, cur, gu) : 0;
+        for (int p = 0, nn = off[i + 1] - off[i]; p < nn; ++p)
+          Fb += pair_force(a, cur, gu, me, um, f, img, a.nbr[(unsigned)p * ns + gu], (V3<Real>*)nullptr, (Real*)nullptr);
+      }
+      if (f & F_TOP) add_load(a, mol, me, q, Fb, Fp);
+      const V3<Real> F = Fb + Fp;
+      const V3<Real> Tc = h * cross(um, Fp - Fb);
+      V3<Real> un = um;
+      if (!frozen) {
+        V3<Real> Ft, Tt;
+        langevin(a, F, Tc, Vd, Om, um, eb, ep, Ft, Tt);
+        kick_drift(a, Ft, Tt, um, Xd, Vd, Om, un, fl);
+      }
+      const int k0 = fixs(Xd[0], a.fixS[0]), k1 = fixs(Xd[1], a.fixS[1]), k2 = fixs(Xd[2], a.fixS[2]);
+      store_state(a, nxt, (int64_t)gu, k0, k1, k2, Xd, un, packed);
+      if (moved(a, k0, k1, k2, un, kr)) fl |= B_STALE;
+      if constexpr (sizeof(Real) == 4) nw = SPos<Real>{k0, k1, k2, un.x, un.y, un.z};
+      else nw = SPos<Real>{Xd[0], Xd[1], Xd[2], un.x, un.y, un.z};
+    }
+    fl = __reduce_or_sync(0xffffffffu, fl);
+    if (lane == 0 && fl) atomicOr(&s_fl[it & 1], fl);
+    __syncthreads();   // flags complete; every read of this step's positions is done
+    if (i == 0) {
+      res_arrive(a.bar, phase, s_fl[it & 1]);
+      s_fl[(it + 1) & 1] = 0u;
+    }
+    // while the barrier completes: the new positions into shared memory and the next step's noise
+    if (mine) {
+      spos[i] = nw;
+      if (!frozen && it + 1 < budget) nucleotide_noise(a, local, step0 + it + 1, mol, eb, ep);
+    }
+    if constexpr (EXT) {
+      if (a.bubble) {
+        __syncwarp();
+        if (mine && !(i & 1)) {
+          const SPos<Real> pb = spos[i + 1];
+          const V3<Real> d = rel(nw, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(nw));
+          const int fi = flg[i] & ~F_OPEN;
+          flg[i] = dot(d, d) > a.c.rchb2 ? fi | F_OPEN : fi;
+        }
+      }
+    }
+    if (i == 0) s_word = res_wait(a.bar, phase, gridDim.x, a.spin_budget);
+    ++phase;
+    __syncthreads();
+    const unsigned r = s_word;
+    if (r & B_ERRMASK) { errbits = r; break; }
+    ++done;
+    if (!(r & B_STALE)) continue;
+
+    // ---- rebuild: bin the beads, segments into the hash, barrier, own lists
+    ++epoch;
+    {
+      const int nw_i = (len + 31) & ~31;
+      if (i < nw_i) {   // whole warps
+        float pw[3] = {0.0f, 0.0f, 0.0f};
+        if (mine) {
+          const float hf = (float)a.c.h;
+          const SPos<Real> me = spos[i];
+          float b[3];
+          if constexpr (sizeof(Real) == 4) {
+            b[0] = d2f_bits(Xd[0]) - hf * me.ux;
+            b[1] = d2f_bits(Xd[1]) - hf * me.uy;
+            b[2] = d2f_bits(Xd[2]) - hf * me.uz;
+            kr[0] = me.kx + bead_off(hf * me.ux, a.fixSf[0]);
+            kr[1] = me.ky + bead_off(hf * me.uy, a.fixSf[1]);
+            kr[2] = me.kz + bead_off(hf * me.uz, a.fixSf[2]);
+          } else {
+            const double uu[3] = {me.ux, me.uy, me.uz};
+            for (int c = 0; c < 3; ++c) {
+              b[c] = (float)(Xd[c] - (double)hf * uu[c]);
+              kr[c] = fixs(Xd[c], a.fixS[c]) + bead_off(hf * (float)uu[c], a.fixSf[c]);
+            }
+          }
+          int wi[3] = {0, 0, 0};
+          for (int c = 0; c < 3; ++c) {
+            float x = b[c];
+            if (a.periodic) {
+              const float qf = floorf(x * a.invLf[c]);
+              wi[c] = (int)qf;
+              x = fmaf(-qf, a.Lf[c], x);
+              if (wi[c] > 511 || wi[c] < -512) pend |= B_EIMG;
+            }
+            pw[c] = x;
+          }
+          packed = (wi[0] & 0x3ff) | ((wi[1] & 0x3ff) << 10) | ((wi[2] & 0x3ff) << 20) | ((f & F_STERIC) << IMG_STERIC_SHIFT);
+          a.wpos[gu] = make_float4(pw[0], pw[1], pw[2], __int_as_float(mol));
+          if constexpr (sizeof(Real) == 8) a.img[gu] = packed;
+          else a.Kw[(unsigned)nxt * ns + gu].w = packed;
+        }
+        float c3[3];
+        const float R = seg_sphere(a, mine, pw, c3);
+        int mlo = mine ? mol : INT_MAX, mhi = mine ? mol : INT_MIN;
+        for (int o = 8; o > 0; o >>= 1) {
+          mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
+          mhi = max(mhi, __shfl_xor_sync(0xffffffffu, mhi, o, 16));
+        }
+        const bool wide = !(R <= a.sg_rcap) || mlo != mhi;
+        if (mine && (lane & 15) == 0) {
+          a.segc[g >> 4] = make_float4(c3[0], c3[1], c3[2], wide ? -1.0f : R);
+          if (!wide) res_insert(a, mol, c3, (unsigned)(g >> 4), epoch);
+        }
+        if (mine && wide) res_insert(a, mol, pw, (unsigned)a.nseg16 + gu, epoch);
+      }
+      pend = __reduce_or_sync(0xffffffffu, pend);
+      if (lane == 0 && pend) atomicOr(&s_fl[(it + 1) & 1], pend);
+      pend = 0;
+      __syncthreads();
+      if (i == 0) {
+        res_arrive(a.bar, phase, s_fl[(it + 1) & 1]);
+        s_fl[(it + 1) & 1] = 0u;
+        s_word = res_wait(a.bar, phase, gridDim.x, a.spin_budget);
+      }
+      ++phase;
+      __syncthreads();
+      if (s_word & B_ERRMASK) { errbits = s_word; break; }
+      int cnt = 0, total = 0;
+      if (i < nw_i) {
+        const int64_t g0 = s0 + 32 * warp;
+        res_list(a, g0, (int)min((int64_t)32, SEG_W * ((s1 - g0 + SEG_W - 1) / SEG_W)), epoch, win, gi, gc, list, cnt, total);
+        if (mine) {
+          if (total > a.cap) pend |= B_EOVF;
+          for (int q = 0; q < cnt; ++q) a.nbr[(unsigned)q * ns + gu] = list[q];
+          a.ncnt[gu] = cnt;
+        }
+      }
+      number_pairs(mine ? cnt : 0);
+      for (int q = 0; q < cnt; ++q) keep_entry(q, list[q]);
+      if (blockIdx.x == 0 && i == 0) *a.nrebuild += 1;
+      __syncthreads();
+    }
+  }
+  // state back to memory
+  if (mine) {
+    if (sizeof(Real) == 4 && !frozen) { a.X[gu] = Xd[0]; a.X[ns + gu] = Xd[1]; a.X[2 * ns + gu] = Xd[2]; }
+    a.V[gu] = Vd[0]; a.V[ns + gu] = Vd[1]; a.V[2 * ns + gu] = Vd[2];
+    a.Om[gu] = Om.x; a.Om[ns + gu] = Om.y; a.Om[2 * ns + gu] = Om.z;
+    a.kref[gu] = kr[0]; a.kref[ns + gu] = kr[1]; a.kref[2 * ns + gu] = kr[2];
+  }
+  errbits |= __syncthreads_or((int)pend) ? (unsigned)B_EOVF : 0u;
+  if (i == 0) {
+    if (errbits & B_ERRMASK) atomicOr(a.err, errbits & B_ERRMASK);
+    if (blockIdx.x == 0) {
+      *a.step = step0 + done;
+      const int64_t left = budget - done;
+      if (a.steps_left) *a.steps_left = left;
+      if (a.use_cond) cudaGraphSetConditional(a.h_while, left > 0 && done > 0 && (errbits & B_ERRMASK) == 0 ? 1u : 0u);
+    }
+  }
+}
+
+}  // namespace dsdna
