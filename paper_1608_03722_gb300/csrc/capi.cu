@@ -91,6 +91,7 @@ struct dsdna_ctx {
   bool chain = false;
   float4* segc = nullptr;
   unsigned long long* rs_head = nullptr; unsigned* rs_next = nullptr; unsigned rs_mask = 0;   // resident kernel's cell lists
+  uint4* rs_xch = nullptr; unsigned* rs_seq = nullptr;                 // and exchange
   int sg_nc[3] = {0, 0, 0};
   double sg_edge = 0;
   unsigned sg_H = 0, sg_mask = 0;
@@ -353,6 +354,7 @@ static void fill_args(dsdna_ctx* c, KArgs<Real>& a) {
   a.sg_H = c->sg_H;
   a.sg_mask = c->sg_mask;
   a.rs_head = c->rs_head; a.rs_next = c->rs_next; a.rs_mask = c->rs_mask;
+  a.rs_xch = c->rs_xch; a.rs_seq = c->rs_seq;
   a.sg_rcap = (float)DSDNA_SEG_RCAP;
   a.sg_reach = std::sqrt(a.c.rl_max2) + 0.002f;   // margin over the FP32 rounding of centres and radii
   for (int k = 0; k < 3; ++k) {
@@ -608,7 +610,10 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   ALLOC(cnt, unsigned, c->H_alloc); ALLOC(start, unsigned, (size_t)c->H_alloc + 1); ALLOC(key, int, nn);
   ALLOC(cent, float4, nn); ALLOC(wpos, float4, nn);
   if (c->chain) ALLOC(segc, float4, (nn + 15) / 16 + 1);
-  if (c->resident) { ALLOC(rs_head, unsigned long long, (size_t)c->rs_mask + 1); ALLOC(rs_next, unsigned, (nn + 15) / 16 + nn); }
+  if (c->resident) {
+    ALLOC(rs_head, unsigned long long, (size_t)c->rs_mask + 1); ALLOC(rs_next, unsigned, (nn + 15) / 16 + nn);
+    ALLOC(rs_xch, uint4, (f64 ? 4 : 2) * 2 * ns); ALLOC(rs_seq, unsigned, 1);
+  }
   ALLOC(mol_off, int64_t, c->n_mol + 1); ALLOC(ext_d, double, (size_t)c->n_mol * 8);
   ALLOC(bar, GridBar, 1); ALLOC(err, unsigned, 4); ALLOC(step_d, int64_t, 1); ALLOC(rebuild, int, 4);
   ALLOC(nrebuild, unsigned long long, 1);
@@ -704,7 +709,11 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
       cudaMemset(c->X, 0, (f64 ? 48 : 24) * ns) != cudaSuccess || cudaMemset(c->kref, 0, 12 * ns) != cudaSuccess ||
       cudaMemset(c->img, 0, 4 * ns) != cudaSuccess)
     return bad(fail(c, DSDNA_ECUDA, "initialisation"));
-  if (c->resident && cudaMemset(c->rs_head, 0, sizeof(unsigned long long) * ((size_t)c->rs_mask + 1)) != cudaSuccess)
+  // sequence numbers start at 1: zeroed records match no step
+  const unsigned first_seq = 1;
+  if (c->resident && (cudaMemset(c->rs_head, 0, sizeof(unsigned long long) * ((size_t)c->rs_mask + 1)) != cudaSuccess ||
+                      cudaMemset(c->rs_xch, 0, sizeof(uint4) * (f64 ? 4 : 2) * 2 * ns) != cudaSuccess ||
+                      cudaMemcpy(c->rs_seq, &first_seq, sizeof(first_seq), cudaMemcpyHostToDevice) != cudaSuccess))
     return bad(fail(c, DSDNA_ECUDA, "initialisation"));
   if (!f64 && (cudaMemset(c->Kw, 0, sizeof(int4) * 2 * ns) != cudaSuccess ||
                cudaMemset(c->U, 0, sizeof(float4) * 2 * ns) != cudaSuccess))

@@ -70,7 +70,8 @@ struct GridBar {
   unsigned count;
   unsigned gen;
   unsigned acc[3];
-  unsigned pad[3];
+  unsigned pad[27];
+  unsigned res[3][32];   // words of the resident kernel's agreements, a 128-byte line each
 };
 
 template <class Real>
@@ -159,6 +160,8 @@ struct KArgs {
   unsigned long long* rs_head;   // [rs_mask + 1] epoch of the rebuild << 32 | first item
   unsigned* rs_next;             // [nseg16 + n] next item of the list
   unsigned rs_mask;
+  uint4* rs_xch;      // [2][ns][records] positions passed between CTAs
+  unsigned* rs_seq;   // sequence number of the next launch's first step
   int periodic;
   int nc[3];
   float cellh[3];

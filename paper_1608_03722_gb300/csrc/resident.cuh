@@ -14,20 +14,26 @@
 //    list partners of other stretches;
 //  * owners and list pairs are dealt to the warps together (they need only
 //    positions), one block barrier later every nucleotide adds its forces and
-//    moves, and the noise of the next step is drawn while the grid barrier
-//    completes;
-//  * the grid barrier is one release add and one acquire poll on a word that
-//    also counts the stale flags;
+//    moves;
+//  * positions pass between CTAs as 16-byte records that carry the step they
+//    belong to, stored and polled as single 128-bit accesses: a reader waits
+//    for the slots it needs and for nothing else;
+//  * the grid-wide agreement that no bead has outrun the list (and that no
+//    error happened) is needed only before the pair forces are used, so a
+//    warp of its own publishes the CTA's word and polls the others' while the
+//    rest evaluate the next step's owners and pairs; a stale list throws away
+//    the pair forces only.  As a barrier after every step (a release add on
+//    one word, polled by all) it took 2.6 us of the 5.9 us of a 10 kbp step;
 //  * a rebuild is one phase that bins the beads and threads each 16-slot
 //    segment into a hash of cells (linked lists, no table scan), one grid
 //    barrier, and the chain-window list build of the CTA's own beads, whose
 //    result stays in shared memory.
 // All forces, sums and updates are those of engine_kernel, term by term in the
 // same order, so trajectories agree bit for bit.  100 steps and one state
-// download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1960 ->
-// 847 us, periodic walk of 30 kbp 2241 -> 1140 us, 64 rings of 500 bp 3463 ->
-// 2029 us; 50 FP64 steps of 200 bp 3733 -> 1298 us (a warp per SM instead of
-// eight sharing one SM's FP64 pipe).
+// download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1957 ->
+// 778 us, periodic walk of 30 kbp 2244 -> 1089 us, 64 rings of 500 bp 3409 ->
+// 1745 us, melting 16 x 1000 bp 1811 -> 1059 us; 50 FP64 steps of 200 bp 3719
+// -> 1247 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
 #pragma once
 #include "chainlist.cuh"
 #include "engine_kernels.cuh"
@@ -39,9 +45,10 @@ template <class Real> __host__ __device__ constexpr int res_max_threads() { retu
 constexpr int RES_PAIRS_PER_SLOT = 4;   // list entries kept in shared memory per slot (else the lists are walked in memory)
 
 // Shared-memory layout of a CTA whose stretch holds at most `len` slots.
+constexpr int RES_HALO = 8;   // slots staged beyond either end of a stretch (the neighbourhoods of its owners)
 struct ResLayout {
   int len, own, pairs, warps;
-  size_t pos, flg, cs, cn, cp, pf, ent, off, po, jx, xo, list, win, gi, gc, bytes;
+  size_t pos, flg, cs, cn, cp, pf, ent, off, po, jx, xo, xw, list, win, gi, gc, bytes;
 };
 template <class Real>
 __host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
@@ -56,7 +63,7 @@ __host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
     o = (o + bytes + 15) & ~(size_t)15;
     return at;
   };
-  l.pos = take(sizeof(SPos<Real>) * len);
+  l.pos = take(2 * sizeof(SPos<Real>) * (len + 2 * RES_HALO));   // this step's and the next one's
   l.cs = take(sizeof(Real) * 6 * l.own);
   l.cn = take(sizeof(Real) * 6 * l.own);
   l.cp = take(sizeof(Real) * 3 * l.own);
@@ -64,10 +71,11 @@ __host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
   l.win = take(sizeof(float4) * (CL_WIN + CL_WIN / 16) * l.warps);
   l.gc = take(sizeof(float4) * 4 * l.warps);
   l.gi = take(sizeof(int) * 4 * l.warps);
-  l.flg = take(sizeof(int) * len);
+  l.flg = take(sizeof(int) * (len + 2 * RES_HALO));
   l.ent = take(sizeof(int) * l.pairs);
   l.off = take(sizeof(int) * (len + 33));
-  l.xo = take(sizeof(int) * (rings ? len / 3 + 8 : 0));
+  l.xo = take(sizeof(int) * (rings ? l.own : 0));
+  l.xw = take(sizeof(short) * (rings ? l.own : 0));
   l.list = take(sizeof(int) * 32 * LIST_CAP * l.warps);
   l.po = take(sizeof(unsigned short) * l.pairs);
   l.jx = take(sizeof(short) * len);
@@ -75,73 +83,165 @@ __host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
   return l;
 }
 
-// ---------------------------------------------------------------- grid barrier
-// Barrier number k of a launch counts on word k mod 3 of bar->acc: arrivals in
-// bits 0-9, stale stretches in bits 10-19, stretches with an error in bits
-// 20-29 (their bits are in bar->gen).  The word of barrier k - 1 is cleared
-// after barrier k by block 0, two barriers before it is used again.  Returns
-// the flags, or B_ETIMEOUT when the clock budget runs out.
-__device__ __forceinline__ void res_arrive(GridBar* bar, unsigned k, unsigned fl) {
-  if (fl & B_ERRMASK) {
-    atomicOr(&bar->gen, fl & B_ERRMASK);
-    __threadfence();
-  }
-  const unsigned v = 1u | ((fl & B_STALE) ? 1u << 10 : 0u) | ((fl & B_ERRMASK) ? 1u << 20 : 0u);
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&bar->acc[k % 3]), "r"(v) : "memory");
+// ---------------------------------------------------------------- exchange between CTAs
+// A slot's position and orientation as records of three words and a tag: the
+// sequence number of the step (rs_seq + steps of this launch, so that records
+// of earlier launches never match; 30 bits) and the slot's removed terms
+// (bubble rule 2, two bits); double-buffered by step parity.  A CTA
+// overwrites the records of step t when it finishes step t + 1, after every
+// CTA's word for step t, and so after every read of them.
+constexpr unsigned RES_SEQ = 0x3fffffffu;
+template <class Real> __host__ __device__ constexpr int res_records() { return (int)sizeof(SPos<Real>) / 12; }
+
+__device__ __forceinline__ void st128(uint4* p, uint4 v) {
+  asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p),
+               "l"((unsigned long long)v.x | ((unsigned long long)v.y << 32)),
+               "l"((unsigned long long)v.z | ((unsigned long long)v.w << 32))
+               : "memory");
 }
-__device__ __forceinline__ unsigned res_wait(GridBar* bar, unsigned k, unsigned nblocks, unsigned long long budget) {
+__device__ __forceinline__ uint4 ld128(const uint4* p) {
+  unsigned long long lo, hi;
+  asm volatile("{\n .reg .b128 t;\n ld.relaxed.gpu.global.b128 t, [%2];\n mov.b128 {%0, %1}, t;\n}\n"
+               : "=l"(lo), "=l"(hi)
+               : "l"(p)
+               : "memory");
+  return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
+}
+
+template <class Real>
+__device__ __forceinline__ void rec_store(const KArgs<Real>& a, int cur, unsigned g, unsigned seq, int flags, const SPos<Real>& s) {
+  constexpr int R = res_records<Real>();
+  uint4* p = a.rs_xch + R * ((size_t)cur * a.ns + g);
+  unsigned w[3 * R];
+  memcpy(w, &s, sizeof(s));
+  const unsigned tag = (seq & RES_SEQ) | ((unsigned)(flags >> RM_SHIFT) << 30);
+#pragma unroll
+  for (int r = 0; r < R; ++r) st128(p + r, make_uint4(w[3 * r], w[3 * r + 1], w[3 * r + 2], tag));
+}
+
+// Waits for slot g's records of step seq, at most the launch's clock budget;
+// then *timeout is set and the records are returned as they are.  *removed: the
+// slot's removed terms.
+template <class Real>
+__device__ __forceinline__ SPos<Real> rec_load(const KArgs<Real>& a, int cur, unsigned g, unsigned seq, unsigned* timeout,
+                                              unsigned* removed = nullptr) {
+  constexpr int R = res_records<Real>();
+  const uint4* p = a.rs_xch + R * ((size_t)cur * a.ns + g);
+  unsigned w[3 * R];
+  const unsigned long long t0 = clock64();
+  for (;;) {
+    bool ok = true;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint4 v = ld128(p + r);
+      w[3 * r] = v.x; w[3 * r + 1] = v.y; w[3 * r + 2] = v.z;
+      ok = ok && ((v.w ^ seq) & RES_SEQ) == 0u;
+      if (removed) *removed = v.w >> 30;
+    }
+    if (ok) break;
+    if ((unsigned long long)(clock64() - t0) > a.spin_budget) { *timeout = 1u; break; }
+  }
+  SPos<Real> s;
+  memcpy(&s, w, sizeof(s));
+  return s;
+}
+
+// Agreement number p of a launch (step agreements and rebuild barriers share
+// one count) on word p mod 3 of bar->res: arrivals in bits 0-9, stale
+// stretches in bits 10-19, stretches with an error in bits 20-29 (their bits
+// are in bar->gen).  The word of p - 1 is cleared after p by block 0, two
+// agreements before it is used again.  Publishing releases the CTA's writes
+// (after a block barrier), reading acquires the others'.  One word and one
+// release add take 1.28 us over 152 CTAs; a word per CTA, polled by all, took
+// 2.8 to 5 us, the polls queueing behind one another and the stores.
+template <class Real>
+__device__ __forceinline__ void res_publish(const KArgs<Real>& a, unsigned p, unsigned fl) {
+  if (fl & B_ERRMASK) atomicOr(&a.bar->gen, fl & B_ERRMASK);
+  const unsigned v = 1u | ((fl & B_STALE) ? 1u << 10 : 0u) | ((fl & B_ERRMASK) ? 1u << 20 : 0u);
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar->res[p % 3]), "r"(v) : "memory");
+}
+// All CTAs' flags of agreement p (one thread); B_ETIMEOUT when the clock budget
+// runs out.
+template <class Real>
+__device__ __forceinline__ unsigned res_agree(const KArgs<Real>& a, unsigned p) {
   const unsigned long long t0 = clock64();
   unsigned v;
-  while (((v = ld_acquire(&bar->acc[k % 3])) & 1023u) != nblocks)
-    if ((unsigned long long)(clock64() - t0) > budget) return B_ETIMEOUT;
-  if (blockIdx.x == 0) bar->acc[(k + 2) % 3] = 0u;
+  while (((v = ld_acquire(a.bar->res[p % 3])) & 1023u) != gridDim.x)
+    if ((unsigned long long)(clock64() - t0) > a.spin_budget) return B_ETIMEOUT;
+  if (blockIdx.x == 0) a.bar->res[(p + 2) % 3][0] = 0u;
   unsigned r = ((v >> 10) & 1023u) ? B_STALE : 0u;
-  if (v >> 20) r |= ld_acquire(&bar->gen);
+  if (v >> 20) r |= ld_acquire(&a.bar->gen);
   return r;
 }
 
 // ---------------------------------------------------------------- neighbourhood of an owner
-// Slots of the CTA's stretch from shared memory, others from global memory;
-// junction owners of circular molecules (wrap) take their neighbours modulo
-// the molecule.
+// ResSrc: the stretch and its halo in shared memory (every owner but those
+// next to the junction of a circular molecule; spos and flg point at the first
+// slot of the stretch).
 template <class Real>
 struct ResSrc {
+  const SPos<Real>* spos;
+  const int* flg;
+  int s0;
+  __device__ __forceinline__ SPos<Real> pos(int64_t g) const { return spos[(int)g - s0]; }
+  __device__ __forceinline__ int64_t step(int64_t g, int d) const { return (int)g + d; }
+  __device__ __forceinline__ bool open(int64_t k, int mol) const {
+    const int f = flg[2 * (int)k - s0];
+    return (f & F_OPEN) && (f >> MOL_SHIFT) == mol;
+  }
+};
+
+// ResJunc: owners next to a junction, whose neighbours are taken modulo the
+// molecule (base pairs off .. off + N - 1): the stretch from shared memory,
+// other slots from their records.
+template <class Real>
+struct ResJunc {
   const KArgs<Real>& a;
   const SPos<Real>* spos;
   const int* flg;
+  unsigned* timeout;
   int cur;
-  int64_t s0;
-  int len;
-  bool wrap;
-  int64_t off, N;   // base-pair offset and length of the owner's molecule (wrap only)
-  __device__ __forceinline__ int64_t bp(int64_t k) const {
-    if (!wrap) return k;
-    const int64_t r = (k - off) % N;
-    return off + (r < 0 ? r + N : r);
+  unsigned seq;
+  int s0, len, off, N;
+  __device__ __forceinline__ int bp(int k) const {   // at most three base pairs outside the molecule
+    return k < off ? k + N : (k >= off + N ? k - N : k);
   }
   __device__ __forceinline__ SPos<Real> pos(int64_t g) const {
-    const unsigned l = (unsigned)(g - s0);
+    const unsigned l = (unsigned)((int)g - s0);
     if (l < (unsigned)len) return spos[l];
-    SPos<Real> s;
-    load_slot(a, cur, g, s);
-    return s;
+    return rec_load(a, cur, (unsigned)g, seq, timeout);
   }
   __device__ __forceinline__ int64_t step(int64_t g, int d) const {
-    return wrap ? 2 * bp((g >> 1) + d / 2) + (g & 1) : g + d;
+    return 2 * bp(((int)g >> 1) + d / 2) + ((int)g & 1);
   }
-  __device__ __forceinline__ bool open(int64_t k, int mol) const {
-    k = bp(k);
+  __device__ __forceinline__ bool open(int64_t k64, int /*mol*/) const {
+    const int k = bp((int)k64);
     const unsigned l = (unsigned)(2 * k - s0);
-    if (l < (unsigned)len) {
-      const int f = flg[l];
-      return (f & F_OPEN) && (f >> MOL_SHIFT) == mol;
-    }
-    if (k < 0 || 2 * k >= a.n || (a.topo[2 * k] >> MOL_SHIFT) != mol) return false;
+    if (l < (unsigned)len) return (flg[l] & F_OPEN) != 0;
     const SPos<Real> pa = pos(2 * k), pb = pos(2 * k + 1);
     const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
     return dot(d, d) > a.c.rchb2;
   }
 };
+
+// Typed WCA force of list entry e on bead b of the stretch (record me, partner
+// q with flags fj).
+template <class Real>
+__device__ __forceinline__ V3<Real> res_pair(const KArgs<Real>& a, int s0, int b, const SPos<Real>& me, int fb, int e,
+                                             const SPos<Real>& q, int fj) {
+  const int j = e & ENT_JMASK;
+  V3<Real> R = rel(me, q, a.fixq);
+  if constexpr (sizeof(Real) == 8) {
+    if (a.periodic) {
+      const int wi = a.img[s0 + b], wj = a.img[j];
+      R.x += (double)(img_comp(wi, 0) - img_comp(wj, 0) + ent_shift(e, 0)) * a.L[0];
+      R.y += (double)(img_comp(wi, 1) - img_comp(wj, 1) + ent_shift(e, 1)) * a.L[1];
+      R.z += (double)(img_comp(wi, 2) - img_comp(wj, 2) + ent_shift(e, 2)) * a.L[2];
+    }
+  }
+  return pair_core(a, R, uvec(me), uvec(q), ((s0 + b) ^ j) & 1, (fb & fj & F_STERIC) != 0, (V3<Real>*)nullptr,
+                   (Real*)nullptr);
+}
 
 // ---------------------------------------------------------------- list build
 constexpr unsigned RES_NONE = 0xffffffffu;
@@ -255,15 +355,23 @@ __device__ __forceinline__ void res_list(const KArgs<Real>& a, int64_t g0, int n
     const int pmol = __float_as_int(mp.w);
     const int64_t plo = a.n_mol > 1 ? 2 * a.mol_off[pmol] : 0, phi = a.n_mol > 1 ? 2 * a.mol_off[pmol + 1] : a.n;
     const float4 pt = make_float4(mp.x, mp.y, mp.z, 0.0f);
+    // the buckets first, all heads in flight together; a bucket two cells share is walked once
+    unsigned keys[27], hd[27];
+#pragma unroll
     for (int q = 0; q < 27; ++q) {
-      const unsigned k = res_key(a, pmol, ci, q);
-      bool dup = false;
-      for (int o = 0; o < q; ++o) dup = dup || res_key(a, pmol, ci, o) == k;
-      if (dup) continue;
-      const unsigned long long hd = a.rs_head[k];
+      keys[q] = res_key(a, pmol, ci, q);
+      const unsigned long long e = a.rs_head[keys[q]];
+      hd[q] = (unsigned)(e >> 32) == epoch ? (unsigned)e : RES_NONE;
+    }
+#pragma unroll
+    for (int q = 1; q < 27; ++q)
+#pragma unroll
+      for (int o = 0; o < q; ++o)
+        if (keys[o] == keys[q]) hd[q] = RES_NONE;
+#pragma unroll 1
+    for (int q = 0; q < 27; ++q) {
       unsigned walked = 0;
-      for (unsigned e = (unsigned)(hd >> 32) == epoch ? (unsigned)hd : RES_NONE; e != RES_NONE && walked <= most;
-           e = a.rs_next[e], ++walked) {
+      for (unsigned e = hd[q]; e != RES_NONE && walked <= most; e = a.rs_next[e], ++walked) {
         const bool seg = e < (unsigned)a.nseg16;
         const int64_t j0 = seg ? (int64_t)e * SEG_W : (int64_t)(e - (unsigned)a.nseg16), js = j0 / SEG_W;
         if (j0 < plo || j0 >= phi || (js <= s + 1 && js >= s - 1)) continue;
@@ -290,10 +398,11 @@ template <class Real, bool EXT>
 __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     resident_kernel(const __grid_constant__ KArgs<Real> a, const __grid_constant__ ResLayout lay) {
   extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ unsigned s_fl[2], s_word;
-  __shared__ int s_scan[33], s_nx;
-  SPos<Real>* const spos = reinterpret_cast<SPos<Real>*>(sm + lay.pos);
-  int* const flg = reinterpret_cast<int*>(sm + lay.flg);
+  __shared__ unsigned s_fl[2], s_word, s_to;
+  __shared__ int s_scan[33], s_nx, s_nj;
+  SPos<Real>* const spos2[2] = {reinterpret_cast<SPos<Real>*>(sm + lay.pos) + RES_HALO,
+                                reinterpret_cast<SPos<Real>*>(sm + lay.pos) + lay.len + 3 * RES_HALO};
+  int* const flg = reinterpret_cast<int*>(sm + lay.flg) + RES_HALO;
   Real* const cs = reinterpret_cast<Real*>(sm + lay.cs);
   Real* const cn = reinterpret_cast<Real*>(sm + lay.cn);
   Real* const cp = reinterpret_cast<Real*>(sm + lay.cp);
@@ -303,25 +412,29 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   unsigned short* const po = reinterpret_cast<unsigned short*>(sm + lay.po);
   short* const jx = reinterpret_cast<short*>(sm + lay.jx);
   int* const xo = reinterpret_cast<int*>(sm + lay.xo);
+  short* const xw = reinterpret_cast<short*>(sm + lay.xw);
   const int OC = lay.own;
   const unsigned ns = (unsigned)a.ns;
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nwarp = (int)(blockDim.x >> 5);
+  const int nwork = nwarp - 1;          // the last warp agrees with the other CTAs while these evaluate forces
+  const bool sync_warp = warp == nwork;
   int* const list = reinterpret_cast<int*>(sm + lay.list) + (warp * 32 + lane) * LIST_CAP;
   float4* const win = reinterpret_cast<float4*>(sm + lay.win) + warp * (CL_WIN + CL_WIN / 16);
   int* const gi = reinterpret_cast<int*>(sm + lay.gi) + warp * 4;
   float4* const gc = reinterpret_cast<float4*>(sm + lay.gc) + warp * 4;
 
   // the CTA's stretch, and the nucleotide of this thread
-  const int64_t s0 = SEG_W * ((int64_t)blockIdx.x * a.nseg16 / gridDim.x);
-  const int64_t s1 = min(a.n, SEG_W * ((int64_t)(blockIdx.x + 1) * a.nseg16 / gridDim.x));
-  const int len = (int)(s1 - s0);
+  const int s0 = SEG_W * (int)((int64_t)blockIdx.x * a.nseg16 / gridDim.x);
+  const int s1 = min((int)a.n, SEG_W * (int)((int64_t)(blockIdx.x + 1) * a.nseg16 / gridDim.x));
+  const int len = s1 - s0;
   const bool mine = i < len;
-  const int64_t g = s0 + i;
+  const int g = s0 + i;
   const unsigned gu = (unsigned)(mine ? g : s0);
 
   const int64_t step0 = *a.step;
   int64_t budget = a.steps_left ? *a.steps_left : a.nsteps;
   if (*a.err & B_ERRMASK) budget = 0;
+  const unsigned seq0 = *a.rs_seq;
   unsigned epoch = (unsigned)*a.nrebuild;
   int cur = (int)(step0 & 1);
 
@@ -332,8 +445,9 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   if (mine) {
     SPos<Real> me;
     load_slot(a, cur, g, me);
-    spos[i] = me;
+    spos2[0][i] = me;
     f = a.topo[gu];
+    rec_store(a, cur, gu, seq0, f, me);
     flg[i] = f;
     if constexpr (sizeof(Real) == 4) {
       Xd[0] = a.X[gu]; Xd[1] = a.X[ns + gu]; Xd[2] = a.X[2 * ns + gu];
@@ -347,25 +461,37 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   }
   const int mol = f >> MOL_SHIFT;
   const bool frozen = (f & F_FROZEN) != 0;
-  const uint32_t local = mine ? (uint32_t)(g - 2 * a.mol_off[mol]) : 0u;
-  if (i == 0) { s_fl[0] = 0u; s_fl[1] = 0u; s_nx = 0; }
+  const uint32_t local = mine ? (uint32_t)(g - 2 * (int)a.mol_off[mol]) : 0u;
+  if (i == 0) { s_fl[0] = 0u; s_fl[1] = 0u; s_nx = 0; s_nj = 0; s_to = 0u; s_word = 0u; }
   __syncthreads();
   if constexpr (EXT) {
-    // circular molecules: the end nucleotides of a strand also take the forces
-    // of the owner across the junction, evaluated here a second time
-    if (a.n_junc && mine) {
-      jx[i] = -1;
-      if (f & F_JUNC) {
-        const int64_t k0 = a.mol_off[mol], k1 = a.mol_off[mol + 1] - 1, k = g >> 1;
-        if (k == k0 || k == k1) {
-          const int x = atomicAdd(&s_nx, 1);
-          jx[i] = (short)x;
-          xo[x] = (int)(2 * (k == k0 ? k1 : k0) + (g & 1));
+    // circular molecules: the owners next to a junction, listed apart (slot xo,
+    // place xw in the owner table); the end nucleotides of a strand also take
+    // the forces of the owner across the junction, evaluated here a second time
+    // (places len + 4 + jx)
+    if (a.n_junc) {
+      for (int w = i; w < len + 4; w += blockDim.x) {
+        const int o = s0 - 2 + w;
+        if (o < 0 || o >= (int)a.n || !(a.topo[o] & F_JUNC)) continue;
+        const int x = atomicAdd(&s_nj, 1);
+        xo[x] = o;
+        xw[x] = (short)w;
+      }
+      if (mine) {
+        jx[i] = -1;
+        if (f & F_JUNC) {
+          const int k0 = (int)a.mol_off[mol], k1 = (int)a.mol_off[mol + 1] - 1, k = g >> 1;
+          if (k == k0 || k == k1) {
+            const int x = atomicAdd(&s_nj, 1), y = atomicAdd(&s_nx, 1);
+            jx[i] = (short)y;
+            xo[x] = 2 * (k == k0 ? k1 : k0) + (g & 1);
+            xw[x] = (short)(len + 4 + y);
+          }
         }
       }
     }
     if (a.bubble && mine && !(i & 1)) {
-      const SPos<Real> pa = spos[i], pb = spos[i + 1];
+      const SPos<Real> pa = spos2[0][i], pb = spos2[0][i + 1];
       const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
       if (dot(d, d) > a.c.rchb2) flg[i] = f | F_OPEN;
     }
@@ -401,80 +527,259 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     number_pairs(cnt);
     for (int q = 0; q < cnt; ++q) keep_entry(q, a.nbr[(unsigned)q * ns + gu]);
   }
-  const int nx = EXT ? s_nx : 0;
-  const int nown = len + 4 + nx;
-  V3<Real> eb{0, 0, 0}, ep{0, 0, 0};
-  if (mine && !frozen && budget > 0) nucleotide_noise(a, local, step0, mol, eb, ep);
+  const int njo = EXT ? s_nj : 0;
+  // halo slot of this lane (edge_chunk), its static flags
+  const int hl = lane < RES_HALO ? lane - RES_HALO : len + lane - RES_HALO, hs = s0 + hl;
+  const bool halo = lane < 2 * RES_HALO && hs >= 0 && hs < (int)a.n;
+  const int hf = halo ? a.topo[hs] : 0;
   __syncthreads();
 
-  int64_t done = 0;
-  unsigned errbits = 0, pend = 0, phase = 0;
-  for (int64_t it = 0; it < budget; ++it) {
-    cur = (int)((step0 + it) & 1);
-    const int nxt = cur ^ 1;
-    unsigned fl = pend;
-    pend = 0;
-    // owners and list pairs, 32 at a time to the warps
-    const int nco = (nown + 31) >> 5, ncp = npair <= lay.pairs ? (npair + 31) >> 5 : 0;
-    for (int c = warp; c < nco + ncp; c += nwarp) {
-      if (c < nco) {
-        const int w = 32 * c + lane;
-        if (w >= nown) continue;
-        const bool extra = EXT && w >= len + 4;
-        const int64_t o = extra ? (int64_t)xo[w - (len + 4)] : s0 - 2 + w;
-        const bool home = w >= 2 && w < len + 2;
-        OwnerOut<Real> out{{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-        if (o >= 0 && o < a.n) {
-          const unsigned lo = (unsigned)(o - s0);
-          int fo = lo < (unsigned)len ? flg[lo] : a.topo[o];
-          ResSrc<Real> src{a, spos, flg, cur, s0, len, false, 0, 0};
-          if constexpr (EXT) {
-            if (fo & F_JUNC) {   // both neighbours exist on a ring
-              fo |= F_PREV | F_NEXT;
-              src.wrap = true;
-              src.off = a.mol_off[fo >> MOL_SHIFT];
-              src.N = a.mol_off[(fo >> MOL_SHIFT) + 1] - src.off;
-            }
-          }
-          if (fo & F_NEXT) {
-            unsigned rm = 0u;
-            if constexpr (EXT) {
-              if (a.bubble) {
-                rm = bubble_bits(a, src, o, fo, home);
-                if (home && rm) atomicOr(&flg[lo], (int)(rm << RM_SHIFT));   // as in the topology word
-              }
-            }
-            owner_eval<Real>(a, src, o, fo, rm, fl, (Real*)nullptr, (Real*)nullptr, out);
-          }
+  unsigned errbits = 0, phase = 0, seq = seq0;
+  SPos<Real>* spos = spos2[0];
+  unsigned fl = 0;   // this thread's flags of the step
+  // owners within `edge` slots of an end read the halo (five base pairs with the bubble rule)
+  const int edge = EXT && a.bubble ? 6 : 2;
+  const int e0 = min(edge, len), e1 = max(len - edge, e0);   // interior: local slots [e0, e1)
+
+  auto store_out = [&](int w, const OwnerOut<Real>& out) {
+    cs[0 * OC + w] = out.sb.x; cs[1 * OC + w] = out.sb.y; cs[2 * OC + w] = out.sb.z;
+    cs[3 * OC + w] = out.sp.x; cs[4 * OC + w] = out.sp.y; cs[5 * OC + w] = out.sp.z;
+    cn[0 * OC + w] = out.nb.x; cn[1 * OC + w] = out.nb.y; cn[2 * OC + w] = out.nb.z;
+    cn[3 * OC + w] = out.np.x; cn[4 * OC + w] = out.np.y; cn[5 * OC + w] = out.np.z;
+    cp[0 * OC + w] = out.pp.x; cp[1 * OC + w] = out.pp.y; cp[2 * OC + w] = out.pp.z;
+  };
+  // owner of local slot l (-2 .. len + 1; lanes with `on`)
+  auto owner = [&](int l, bool on) {
+    const int fo = on ? flg[l] : 0;
+    if (!on || (EXT && (fo & F_JUNC))) return;
+    OwnerOut<Real> out{{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+    if (fo & F_NEXT) {
+      const ResSrc<Real> src{spos, flg, s0};
+      unsigned rm = 0u;
+      if constexpr (EXT) {
+        if (a.bubble) {
+          const bool home = l >= 0 && l < len;
+          rm = bubble_bits(a, src, s0 + l, fo, home);
+          if (home && rm) atomicOr(&flg[l], (int)(rm << RM_SHIFT));   // as in the topology word
         }
-        cs[0 * OC + w] = out.sb.x; cs[1 * OC + w] = out.sb.y; cs[2 * OC + w] = out.sb.z;
-        cs[3 * OC + w] = out.sp.x; cs[4 * OC + w] = out.sp.y; cs[5 * OC + w] = out.sp.z;
-        cn[0 * OC + w] = out.nb.x; cn[1 * OC + w] = out.nb.y; cn[2 * OC + w] = out.nb.z;
-        cn[3 * OC + w] = out.np.x; cn[4 * OC + w] = out.np.y; cn[5 * OC + w] = out.np.z;
-        cp[0 * OC + w] = out.pp.x; cp[1 * OC + w] = out.pp.y; cp[2 * OC + w] = out.pp.z;
-      } else {
-        const int p = 32 * (c - nco) + lane;
-        if (p >= npair) continue;
-        const int e = ent[p], b = po[p], j = e & ENT_JMASK;
-        const SPos<Real> me = spos[b];
-        const unsigned l = (unsigned)(j - (int)s0);
-        V3<Real> fw;
-        if ((sizeof(Real) == 4 || !a.periodic) && l < (unsigned)len) {   // partner in the stretch: no memory access
-          const SPos<Real> q = spos[l];
-          fw = pair_core(a, rel(me, q, a.fixq), uvec(me), uvec(q), ((b ^ (int)l) & 1) != 0,
-                         ((flg[b] & flg[l]) & F_STERIC) != 0, (V3<Real>*)nullptr, (Real*)nullptr);
+      }
+      owner_eval<Real>(a, src, s0 + l, fo, rm, fl, (Real*)nullptr, (Real*)nullptr, out);
+    }
+    store_out(l + 2, out);
+  };
+  // the halo into shared memory, then the owners near both ends
+  auto edge_chunk = [&] {
+    int fh = 0;
+    if (halo) {
+      unsigned rm0 = 0u;
+      spos[hl] = rec_load(a, cur, (unsigned)hs, seq, &s_to, &rm0);
+      fh = (hf & ~(3 << RM_SHIFT)) | (int)(rm0 << RM_SHIFT);
+    }
+    __syncwarp();
+    if (lane < 2 * RES_HALO) {
+      if (EXT && a.bubble && halo && !(lane & 1)) {
+        const SPos<Real> pa = spos[hl], pb = spos[hl + 1];
+        const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
+        if (dot(d, d) > a.c.rchb2) fh |= F_OPEN;
+      }
+      flg[hl] = fh;
+    }
+    __syncwarp();
+    const int lo = 2 + e0, hi = len + 2 - e1;   // owners at either end
+    owner(lane < lo ? lane - 2 : e1 + lane - lo, lane < lo + hi);
+    __syncwarp();
+  };
+  // owners next to junctions of circular molecules
+  auto junction_chunk = [&](int c) {
+    const int x = 32 * c + lane;
+    if (x < njo) {
+      const int o = xo[x], w = xw[x];
+      const unsigned l = (unsigned)(o - s0);
+      const bool home = w >= 2 && w < len + 2;
+      int fo = (l < (unsigned)len ? flg[l] : a.topo[o]) | F_PREV | F_NEXT;   // both neighbours exist on a ring
+      const int m = fo >> MOL_SHIFT, off0 = (int)a.mol_off[m];
+      const ResJunc<Real> src{a, spos, flg, &s_to, cur, seq, s0, len, off0, (int)a.mol_off[m + 1] - off0};
+      unsigned rm = 0u;
+      if constexpr (EXT) {
+        if (a.bubble) {
+          if (l >= (unsigned)len) {   // removed terms as of this step: the topology word may be a step ahead
+            unsigned rm0 = 0u;
+            rec_load(a, cur, (unsigned)o, seq, &s_to, &rm0);
+            fo = (fo & ~(3 << RM_SHIFT)) | (int)(rm0 << RM_SHIFT);
+          }
+          rm = bubble_bits(a, src, o, fo, home);
+          if (home && rm) atomicOr(&flg[l], (int)(rm << RM_SHIFT));
+        }
+      }
+      OwnerOut<Real> out{{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+      owner_eval<Real>(a, src, o, fo, rm, fl, (Real*)nullptr, (Real*)nullptr, out);
+      store_out(w, out);
+    }
+    __syncwarp();
+  };
+  // partner of list entry e: from shared memory, or its records
+  auto partner = [&](int e, int& fj) {
+    const int j = e & ENT_JMASK;
+    const unsigned l = (unsigned)(j - s0);
+    if (l < (unsigned)len) {
+      fj = flg[l];
+      return spos[l];
+    }
+    fj = a.topo[j];
+    return rec_load(a, cur, (unsigned)j, seq, &s_to);
+  };
+  // pairs 32 c .. of the table
+  auto pair_chunk = [&](int c) {
+    const int p = 32 * c + lane;
+    const bool on = p < npair;
+    int b = 0, e = 0, fj = 0;
+    SPos<Real> q{};
+    if (on) {
+      b = po[p];
+      e = ent[p];
+      q = partner(e, fj);
+    }
+    __syncwarp();   // the lanes that waited for a record join the others
+    if (on) {
+      const V3<Real> fw = res_pair(a, s0, b, spos[b], flg[b], e, q, fj);
+      Real* o = pf + 3 * p;
+      o[0] = fw.x; o[1] = fw.y; o[2] = fw.z;
+    }
+  };
+  // the sync warp: this CTA's flags out, every CTA's in (to s_word)
+  auto agree = [&](unsigned* flags, auto meanwhile) {
+    ++phase;
+    if (sync_warp) {
+      if (lane == 0) {
+        res_publish(a, phase, *flags);
+        *flags = 0u;
+      }
+      meanwhile();
+      if (lane == 0) s_word = res_agree(a, phase);
+    }
+  };
+  // bin the beads, thread the segments into the hash, wait for all, build the
+  // CTA's own lists
+  auto rebuild = [&](unsigned* flags) {
+    ++epoch;
+    const int nw_i = (len + 31) & ~31;
+    unsigned e = 0;
+    if (i < nw_i) {   // whole warps
+      float pw[3] = {0.0f, 0.0f, 0.0f};
+      if (mine) {
+        const float hf = (float)a.c.h;
+        const SPos<Real> me = spos[i];
+        float b[3];
+        if constexpr (sizeof(Real) == 4) {
+          b[0] = d2f_bits(Xd[0]) - hf * me.ux;
+          b[1] = d2f_bits(Xd[1]) - hf * me.uy;
+          b[2] = d2f_bits(Xd[2]) - hf * me.uz;
+          kr[0] = me.kx + bead_off(hf * me.ux, a.fixSf[0]);
+          kr[1] = me.ky + bead_off(hf * me.uy, a.fixSf[1]);
+          kr[2] = me.kz + bead_off(hf * me.uz, a.fixSf[2]);
         } else {
-          const unsigned gb = (unsigned)s0 + (unsigned)b;
-          const int img = (sizeof(Real) == 8 && a.periodic) ? own_image(a, cur, gb) : 0;
-          fw = pair_force(a, cur, gb, me, uvec(me), flg[b], img, e, (V3<Real>*)nullptr, (Real*)nullptr);
+          const double uu[3] = {me.ux, me.uy, me.uz};
+          for (int c = 0; c < 3; ++c) {
+            b[c] = (float)(Xd[c] - (double)hf * uu[c]);
+            kr[c] = fixs(Xd[c], a.fixS[c]) + bead_off(hf * (float)uu[c], a.fixSf[c]);
+          }
         }
-        Real* o = pf + 3 * p;
-        o[0] = fw.x; o[1] = fw.y; o[2] = fw.z;
+        int wi[3] = {0, 0, 0};
+        for (int c = 0; c < 3; ++c) {
+          float x = b[c];
+          if (a.periodic) {
+            const float qf = floorf(x * a.invLf[c]);
+            wi[c] = (int)qf;
+            x = fmaf(-qf, a.Lf[c], x);
+            if (wi[c] > 511 || wi[c] < -512) e |= B_EIMG;
+          }
+          pw[c] = x;
+        }
+        packed = (wi[0] & 0x3ff) | ((wi[1] & 0x3ff) << 10) | ((wi[2] & 0x3ff) << 20) | ((f & F_STERIC) << IMG_STERIC_SHIFT);
+        a.wpos[gu] = make_float4(pw[0], pw[1], pw[2], __int_as_float(mol));
+        if constexpr (sizeof(Real) == 8) a.img[gu] = packed;
+      }
+      float c3[3];
+      const float R = seg_sphere(a, mine, pw, c3);
+      int mlo = mine ? mol : INT_MAX, mhi = mine ? mol : INT_MIN;
+      for (int o = 8; o > 0; o >>= 1) {
+        mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
+        mhi = max(mhi, __shfl_xor_sync(0xffffffffu, mhi, o, 16));
+      }
+      const bool wide = !(R <= a.sg_rcap) || mlo != mhi;
+      if (mine && (lane & 15) == 0) {
+        a.segc[g >> 4] = make_float4(c3[0], c3[1], c3[2], wide ? -1.0f : R);
+        if (!wide) res_insert(a, mol, c3, (unsigned)(g >> 4), epoch);
+      }
+      if (mine && wide) res_insert(a, mol, pw, (unsigned)a.nseg16 + gu, epoch);
+    }
+    e = __reduce_or_sync(0xffffffffu, e);
+    if (lane == 0 && e) atomicOr(flags, e);
+    __syncthreads();
+    agree(flags, [] {});
+    __syncthreads();
+    if (s_word & B_ERRMASK) return false;
+    int cnt = 0, total = 0;
+    if (i < nw_i) {
+      const int g0 = s0 + 32 * warp;
+      res_list(a, g0, min(32, SEG_W * ((s1 - g0 + SEG_W - 1) / SEG_W)), epoch, win, gi, gc, list, cnt, total);
+      if (mine) {
+        if (total > a.cap) fl |= B_EOVF;
+        for (int q = 0; q < cnt; ++q) a.nbr[(unsigned)q * ns + gu] = list[q];
+        a.ncnt[gu] = cnt;
       }
     }
+    number_pairs(mine ? cnt : 0);
+    for (int q = 0; q < cnt; ++q) keep_entry(q, list[q]);
+    if (blockIdx.x == 0 && i == 0) *a.nrebuild += 1;
     __syncthreads();
+    return true;
+  };
+
+  int64_t it = 0;   // steps taken
+  for (;; ++it) {
+    const bool end = it == budget;
+    const int64_t step = step0 + it;
+    cur = (int)(step & 1);
+    const int nxt = cur ^ 1;
+    spos = (it & 1) ? spos2[1] : spos2[0];
+    SPos<Real>* const snxt = (it & 1) ? spos2[0] : spos2[1];
+    seq = seq0 + (unsigned)it;
+    V3<Real> eb{0, 0, 0}, ep{0, 0, 0};
+    unsigned* const before = &s_fl[(it + 1) & 1];   // flags of the step before
+    auto draw_noise = [&] {
+      if (mine && !frozen && !end) nucleotide_noise(a, local, step, mol, eb, ep);
+    };
+    if (!sync_warp && !end) {
+      // owners and list pairs, 32 at a time: the ends and the other owners to the
+      // last warps first, so that the first ones, whose threads also draw the
+      // noise, hold pairs
+      const int nin = (e1 - e0 + 31) >> 5, nco = 1 + nin + ((njo + 31) >> 5);
+      const int ncp = npair <= lay.pairs ? (npair + 31) >> 5 : 0;
+      for (int c = nwork - 1 - warp; c < nco + ncp; c += nwork) {
+        if (c == 0) edge_chunk();
+        else if (c <= nin) owner(e0 + 32 * (c - 1) + lane, e0 + 32 * (c - 1) + lane < e1);
+        else if (c < nco) junction_chunk(c - 1 - nin);
+        else pair_chunk(c - nco);
+      }
+    }
+    if (it > 0) agree(before, [&] { if (sync_warp) draw_noise(); });
+    if (!sync_warp || it == 0) draw_noise();
+    __syncthreads();
+    if (it > 0) {
+      const unsigned r = s_word;
+      if (r & B_ERRMASK) { errbits = r; --it; break; }   // the last step was not taken
+      if (r & B_STALE) {
+        if (!rebuild(before)) { errbits = s_word; break; }
+        if (!end) {   // the pair forces once more, from the new lists
+          const int ncp = npair <= lay.pairs ? (npair + 31) >> 5 : 0;
+          for (int c = warp; c < ncp; c += nwarp) pair_chunk(c);
+          __syncthreads();
+        }
+      }
+    }
+    if (end) break;
     // every nucleotide: forces in the order of nucleotide_pass, then its step
-    SPos<Real> nw;
     if (mine) {
       const SPos<Real> me = spos[i], q = spos[i ^ 1];
       const Real h = a.c.h;
@@ -485,7 +790,7 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
       if constexpr (EXT) {
         if ((f & F_JUNC) && jx[i] >= 0) {   // the owner across the junction: the previous or the next one
           const int x = len + 4 + jx[i];
-          const bool first = (i & 1) ? g >> 1 != a.mol_off[mol] : g >> 1 == a.mol_off[mol];
+          const bool first = (i & 1) ? g >> 1 != (int)a.mol_off[mol] : g >> 1 == (int)a.mol_off[mol];
           if (first) {
             Fb += V3<Real>{cn[0 * OC + x], cn[1 * OC + x], cn[2 * OC + x]};
             Fp += V3<Real>{cn[3 * OC + x], cn[4 * OC + x], cn[5 * OC + x]};
@@ -511,9 +816,12 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
       if (npair <= lay.pairs) {
         for (int p = off[i], p1 = off[i + 1]; p < p1; ++p) Fb += V3<Real>{pf[3 * p], pf[3 * p + 1], pf[3 * p + 2]};
       } else {   // more entries than the table holds: this nucleotide's list, from memory
-        const int img = (sizeof(Real) == 8 && a.periodic) ? own_image(a, cur, gu) : 0;
-        for (int p = 0, nn = off[i + 1] - off[i]; p < nn; ++p)
-          Fb += pair_force(a, cur, gu, me, um, f, img, a.nbr[(unsigned)p * ns + gu], (V3<Real>*)nullptr, (Real*)nullptr);
+        for (int p = 0, nn = off[i + 1] - off[i]; p < nn; ++p) {
+          const int e = a.nbr[(unsigned)p * ns + gu];
+          int fj;
+          const SPos<Real> qj = partner(e, fj);
+          Fb += res_pair(a, s0, i, me, f, e, qj, fj);
+        }
       }
       if (f & F_TOP) add_load(a, mol, me, q, Fb, Fp);
       const V3<Real> F = Fb + Fp;
@@ -525,136 +833,55 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
         kick_drift(a, Ft, Tt, um, Xd, Vd, Om, un, fl);
       }
       const int k0 = fixs(Xd[0], a.fixS[0]), k1 = fixs(Xd[1], a.fixS[1]), k2 = fixs(Xd[2], a.fixS[2]);
-      store_state(a, nxt, (int64_t)gu, k0, k1, k2, Xd, un, packed);
-      if (moved(a, k0, k1, k2, un, kr)) fl |= B_STALE;
+      SPos<Real> nw;
       if constexpr (sizeof(Real) == 4) nw = SPos<Real>{k0, k1, k2, un.x, un.y, un.z};
       else nw = SPos<Real>{Xd[0], Xd[1], Xd[2], un.x, un.y, un.z};
-    }
-    fl = __reduce_or_sync(0xffffffffu, fl);
-    if (lane == 0 && fl) atomicOr(&s_fl[it & 1], fl);
-    __syncthreads();   // flags complete; every read of this step's positions is done
-    if (i == 0) {
-      res_arrive(a.bar, phase, s_fl[it & 1]);
-      s_fl[(it + 1) & 1] = 0u;
-    }
-    // while the barrier completes: the new positions into shared memory and the next step's noise
-    if (mine) {
-      spos[i] = nw;
-      if (!frozen && it + 1 < budget) nucleotide_noise(a, local, step0 + it + 1, mol, eb, ep);
+      rec_store(a, nxt, gu, seq0 + (unsigned)it + 1u, EXT ? flg[i] : 0, nw);
+      snxt[i] = nw;
+      if (moved(a, k0, k1, k2, un, kr)) fl |= B_STALE;
     }
     if constexpr (EXT) {
       if (a.bubble) {
         __syncwarp();
         if (mine && !(i & 1)) {
-          const SPos<Real> pb = spos[i + 1];
-          const V3<Real> d = rel(nw, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(nw));
+          const SPos<Real> pa = snxt[i], pb = snxt[i + 1];
+          const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
           const int fi = flg[i] & ~F_OPEN;
           flg[i] = dot(d, d) > a.c.rchb2 ? fi | F_OPEN : fi;
         }
       }
     }
-    if (i == 0) s_word = res_wait(a.bar, phase, gridDim.x, a.spin_budget);
-    ++phase;
-    __syncthreads();
-    const unsigned r = s_word;
-    if (r & B_ERRMASK) { errbits = r; break; }
-    ++done;
-    if (!(r & B_STALE)) continue;
-
-    // ---- rebuild: bin the beads, segments into the hash, barrier, own lists
-    ++epoch;
-    {
-      const int nw_i = (len + 31) & ~31;
-      if (i < nw_i) {   // whole warps
-        float pw[3] = {0.0f, 0.0f, 0.0f};
-        if (mine) {
-          const float hf = (float)a.c.h;
-          const SPos<Real> me = spos[i];
-          float b[3];
-          if constexpr (sizeof(Real) == 4) {
-            b[0] = d2f_bits(Xd[0]) - hf * me.ux;
-            b[1] = d2f_bits(Xd[1]) - hf * me.uy;
-            b[2] = d2f_bits(Xd[2]) - hf * me.uz;
-            kr[0] = me.kx + bead_off(hf * me.ux, a.fixSf[0]);
-            kr[1] = me.ky + bead_off(hf * me.uy, a.fixSf[1]);
-            kr[2] = me.kz + bead_off(hf * me.uz, a.fixSf[2]);
-          } else {
-            const double uu[3] = {me.ux, me.uy, me.uz};
-            for (int c = 0; c < 3; ++c) {
-              b[c] = (float)(Xd[c] - (double)hf * uu[c]);
-              kr[c] = fixs(Xd[c], a.fixS[c]) + bead_off(hf * (float)uu[c], a.fixSf[c]);
-            }
-          }
-          int wi[3] = {0, 0, 0};
-          for (int c = 0; c < 3; ++c) {
-            float x = b[c];
-            if (a.periodic) {
-              const float qf = floorf(x * a.invLf[c]);
-              wi[c] = (int)qf;
-              x = fmaf(-qf, a.Lf[c], x);
-              if (wi[c] > 511 || wi[c] < -512) pend |= B_EIMG;
-            }
-            pw[c] = x;
-          }
-          packed = (wi[0] & 0x3ff) | ((wi[1] & 0x3ff) << 10) | ((wi[2] & 0x3ff) << 20) | ((f & F_STERIC) << IMG_STERIC_SHIFT);
-          a.wpos[gu] = make_float4(pw[0], pw[1], pw[2], __int_as_float(mol));
-          if constexpr (sizeof(Real) == 8) a.img[gu] = packed;
-          else a.Kw[(unsigned)nxt * ns + gu].w = packed;
-        }
-        float c3[3];
-        const float R = seg_sphere(a, mine, pw, c3);
-        int mlo = mine ? mol : INT_MAX, mhi = mine ? mol : INT_MIN;
-        for (int o = 8; o > 0; o >>= 1) {
-          mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
-          mhi = max(mhi, __shfl_xor_sync(0xffffffffu, mhi, o, 16));
-        }
-        const bool wide = !(R <= a.sg_rcap) || mlo != mhi;
-        if (mine && (lane & 15) == 0) {
-          a.segc[g >> 4] = make_float4(c3[0], c3[1], c3[2], wide ? -1.0f : R);
-          if (!wide) res_insert(a, mol, c3, (unsigned)(g >> 4), epoch);
-        }
-        if (mine && wide) res_insert(a, mol, pw, (unsigned)a.nseg16 + gu, epoch);
-      }
-      pend = __reduce_or_sync(0xffffffffu, pend);
-      if (lane == 0 && pend) atomicOr(&s_fl[(it + 1) & 1], pend);
-      pend = 0;
-      __syncthreads();
-      if (i == 0) {
-        res_arrive(a.bar, phase, s_fl[(it + 1) & 1]);
-        s_fl[(it + 1) & 1] = 0u;
-        s_word = res_wait(a.bar, phase, gridDim.x, a.spin_budget);
-      }
-      ++phase;
-      __syncthreads();
-      if (s_word & B_ERRMASK) { errbits = s_word; break; }
-      int cnt = 0, total = 0;
-      if (i < nw_i) {
-        const int64_t g0 = s0 + 32 * warp;
-        res_list(a, g0, (int)min((int64_t)32, SEG_W * ((s1 - g0 + SEG_W - 1) / SEG_W)), epoch, win, gi, gc, list, cnt, total);
-        if (mine) {
-          if (total > a.cap) pend |= B_EOVF;
-          for (int q = 0; q < cnt; ++q) a.nbr[(unsigned)q * ns + gu] = list[q];
-          a.ncnt[gu] = cnt;
-        }
-      }
-      number_pairs(mine ? cnt : 0);
-      for (int q = 0; q < cnt; ++q) keep_entry(q, list[q]);
-      if (blockIdx.x == 0 && i == 0) *a.nrebuild += 1;
-      __syncthreads();
-    }
+    if (i == 0 && s_to) fl |= B_ETIMEOUT;
+    fl = __reduce_or_sync(0xffffffffu, fl);
+    if (lane == 0 && fl) atomicOr(&s_fl[it & 1], fl);
+    fl = 0;
+    __syncthreads();   // the next step's positions and this step's flags are complete
   }
-  // state back to memory
+  const int64_t done = it;
+  // state back to memory: orientation and mirror into the buffer of the step
+  // the launch ends at, into both after an error
   if (mine) {
+    const SPos<Real> me = spos[i];
+    for (int o = 0; o < (errbits ? 2 : 1); ++o) {
+      const int buf = (int)((step0 + done + o) & 1);
+      if constexpr (sizeof(Real) == 4) {
+        const double none[3] = {0, 0, 0};
+        store_state(a, buf, (int64_t)gu, me.kx, me.ky, me.kz, none, uvec(me), packed);
+      } else {
+        store_state(a, buf, (int64_t)gu, 0, 0, 0, Xd, uvec(me), 0);
+      }
+    }
     if (sizeof(Real) == 4 && !frozen) { a.X[gu] = Xd[0]; a.X[ns + gu] = Xd[1]; a.X[2 * ns + gu] = Xd[2]; }
     a.V[gu] = Vd[0]; a.V[ns + gu] = Vd[1]; a.V[2 * ns + gu] = Vd[2];
     a.Om[gu] = Om.x; a.Om[ns + gu] = Om.y; a.Om[2 * ns + gu] = Om.z;
     a.kref[gu] = kr[0]; a.kref[ns + gu] = kr[1]; a.kref[2 * ns + gu] = kr[2];
   }
-  errbits |= __syncthreads_or((int)pend) ? (unsigned)B_EOVF : 0u;
+  if (__syncthreads_or((int)(fl & B_EOVF))) errbits |= B_EOVF;   // of a rebuild after the last step
   if (i == 0) {
     if (errbits & B_ERRMASK) atomicOr(a.err, errbits & B_ERRMASK);
     if (blockIdx.x == 0) {
       *a.step = step0 + done;
+      *a.rs_seq = seq0 + (unsigned)budget + 2u;
       const int64_t left = budget - done;
       if (a.steps_left) *a.steps_left = left;
       if (a.use_cond) cudaGraphSetConditional(a.h_while, left > 0 && done > 0 && (errbits & B_ERRMASK) == 0 ? 1u : 0u);
