@@ -106,6 +106,8 @@ enum { DSDNA_NOISE_OFF = 0, DSDNA_NOISE_UNIFORM = 1, DSDNA_NOISE_GAUSSIAN = 2 };
 /* Chain-window list build: radius (nm) of the widest 16-slot segment (8 base
  * pairs; about 1.3 nm in the relaxed helix) that enters the segment grid whole. */
 #define DSDNA_SEG_RCAP 1.8
+/* The same for the resident step kernel in an open box. */
+#define DSDNA_RES_RCAP 3.2
 
 typedef struct dsdna_params {
   double K1, R0, eps_bb, sigma_bb;       /* FENE + backbone WCA */

@@ -91,7 +91,7 @@ struct dsdna_ctx {
   bool chain = false;
   float4* segc = nullptr;
   unsigned long long* rs_head = nullptr; unsigned* rs_next = nullptr; unsigned rs_mask = 0;   // resident kernel's cell lists
-  uint4* rs_xch = nullptr; unsigned* rs_seq = nullptr;                 // and exchange
+  uint4* rs_xch = nullptr; unsigned* rs_seq = nullptr; int* rs_part = nullptr; float4* rs_sph1 = nullptr;                 // and exchange
   int sg_nc[3] = {0, 0, 0};
   double sg_edge = 0;
   unsigned sg_H = 0, sg_mask = 0;
@@ -355,6 +355,9 @@ static void fill_args(dsdna_ctx* c, KArgs<Real>& a) {
   a.sg_mask = c->sg_mask;
   a.rs_head = c->rs_head; a.rs_next = c->rs_next; a.rs_mask = c->rs_mask;
   a.rs_xch = c->rs_xch; a.rs_seq = c->rs_seq;
+  a.rs_part = c->rs_part; a.rs_sph1 = c->rs_sph1;
+  a.rs_rcap = c->p.box[0] > 0.0 ? (float)DSDNA_SEG_RCAP : (float)DSDNA_RES_RCAP;
+  a.rs_invh = (float)(1.0 / ((2.0 * DSDNA_RES_RCAP + std::sqrt((double)a.c.rl_max2)) * 1.001 + 0.01));
   a.sg_rcap = (float)DSDNA_SEG_RCAP;
   a.sg_reach = std::sqrt(a.c.rl_max2) + 0.002f;   // margin over the FP32 rounding of centres and radii
   for (int k = 0; k < 3; ++k) {
@@ -555,7 +558,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   // Steps of a small system with the chain-window list run in the resident
   // kernel, whatever block_threads says (the CTA size of engine_kernel), as
   // long as a stretch per SM fits a CTA (77,824 nucleotides in mixed precision
-  // and 38,912 in FP64 on 152 SMs): below that it is 1.7 to 2.9 times faster
+  // and 38,912 in FP64 on 152 SMs): below that it is 2 to 3 times faster
   // than engine_kernel with the rebuild inside (figures in resident.cuh), above
   // it a CTA would have no thread and registers for each of its nucleotides.
   cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device);
@@ -613,6 +616,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   if (c->resident) {
     ALLOC(rs_head, unsigned long long, (size_t)c->rs_mask + 1); ALLOC(rs_next, unsigned, (nn + 15) / 16 + nn);
     ALLOC(rs_xch, uint4, (f64 ? 4 : 2) * 2 * ns); ALLOC(rs_seq, unsigned, 1);
+    ALLOC(rs_part, int, (nn + 15) / 16); ALLOC(rs_sph1, float4, (nn + 15) / 16);
   }
   ALLOC(mol_off, int64_t, c->n_mol + 1); ALLOC(ext_d, double, (size_t)c->n_mol * 8);
   ALLOC(bar, GridBar, 1); ALLOC(err, unsigned, 4); ALLOC(step_d, int64_t, 1); ALLOC(rebuild, int, 4);
@@ -1270,9 +1274,11 @@ extern "C" int dsdna_autotune(const dsdna_params* base, const dsdna_system* sys,
   if (base->rebuild_mode == 0 && n_nt >= DSDNA_FUSED_REBUILD_MAX_NT / 4 && n_nt <= 4 * (int64_t)DSDNA_FUSED_REBUILD_MAX_NT)
     modes = {1, 2};
   // one timed trial of candidate p (ns per nucleotide-step), keeping the fastest
+  // (returns whether the steps ran in the resident kernel, which has its own CTA size)
   auto trial = [&](const dsdna_params& p) {
     dsdna_ctx* c = nullptr;
-    if (dsdna_create(&p, sys, alloc, cuda_stream, &c) != DSDNA_OK) { why = g_create_error; return; }
+    if (dsdna_create(&p, sys, alloc, cuda_stream, &c) != DSDNA_OK) { why = g_create_error; return false; }
+    const bool resident = c->resident;
     float ms = 0.f;
     bool ok = dsdna_step(c, trial_steps) == DSDNA_OK && dsdna_synchronize(c) == DSDNA_OK;   // warm-up + first build
     if (ok) {
@@ -1283,22 +1289,26 @@ extern "C" int dsdna_autotune(const dsdna_params* base, const dsdna_system* sys,
     const double t = 1e6 * (double)ms / ((double)trial_steps * (double)c->n);   // ns per nucleotide-step
     if (!ok) why = c->errmsg.empty() ? std::string("event timing failed") : c->errmsg;
     dsdna_destroy(c);
-    if (!ok) return;
+    if (!ok) return resident;
     ++tried;
     if (t < best_t) { best_t = t; winner = p; }
+    return resident;
   };
   for (int rm : modes)
-  for (double sk : skins)
+  for (double sk : skins) {
+    bool resident = false;
     for (int T : blocks)
       for (int ps : per_sm) {
         if (T > 256 && ps > 1) continue;   // one CTA of this size per SM at most
+        if (resident) continue;            // the launch shape is the kernel's own: one trial per skin
         dsdna_params p = *base;
         p.rebuild_mode = rm;
         p.skin = sk;
         p.block_threads = T;
         p.blocks_per_sm = ps;
-        trial(p);
+        resident = trial(p);
       }
+  }
   // the winner with the other neighbour-list build (the cell walk for the
   // chain window, or the reverse), in case this system favours it
   if (tried) {

@@ -58,15 +58,15 @@ __device__ __forceinline__ unsigned seg_key(const KArgs<Real>& a, int mol, const
   return (unsigned)cc[0] + (unsigned)a.sg_nc[0] * ((unsigned)cc[1] + (unsigned)a.sg_nc[1] * (unsigned)cc[2]);
 }
 
-// Bounding sphere of each 16-slot segment (a 16-lane group of the warp, the
-// lanes with `in` set, the first lane first): radius returned, wrapped centre
-// in c3; positions relative to the segment's first bead by minimum image.
+// Bounding sphere of the beads of each 16-slot segment with `in` set (a 16-lane
+// group of the warp): radius returned, wrapped centre in c3; positions relative
+// to the bead of lane `first` of the group, one of them, by minimum image.
 template <class Real>
-__device__ __forceinline__ float seg_sphere(const KArgs<Real>& a, bool in, const float* pw, float* c3) {
+__device__ __forceinline__ float seg_sphere(const KArgs<Real>& a, bool in, int first, const float* pw, float* c3) {
   const int lane = threadIdx.x & 31;
   float r0[3], d[3];
   for (int c = 0; c < 3; ++c) {
-    r0[c] = __shfl_sync(0xffffffffu, pw[c], 0, 16);
+    r0[c] = __shfl_sync(0xffffffffu, pw[c], first, 16);
     float x = pw[c] - r0[c];
     x = fmaf(-rintf(x * a.invLf[c]), a.Lf[c], x);
     d[c] = in ? x : 0.0f;
@@ -108,7 +108,7 @@ __global__ void k_rebuild_segbin(const KArgs<Real> a) {
     int mol = 0;
     if (in) mol = bin_bead(a, cur, g, fl, pw);
     float c3[3];
-    const float R = seg_sphere(a, in, pw, c3);
+    const float R = seg_sphere(a, in, 0, pw, c3);
     int mlo = in ? mol : INT_MAX, mhi = in ? mol : INT_MIN;
     for (int o = 8; o > 0; o >>= 1) {
       mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
@@ -252,7 +252,6 @@ __device__ __forceinline__ bool cl_stage(const KArgs<Real>& a, int lane, const f
 template <class Real>
 __device__ __forceinline__ void cl_window(const KArgs<Real>& a, int64_t g0, int lane, bool in, bool fast,
                                           const float4* win, bool& st_g, int* list, int& cnt, int& total) {
-  const int g = (int)g0 + lane;
   const int kb = lane & 16;   // lanes 0-15 (segment 2t) test staged slots 0..47, lanes 16-31 slots 16..63
   const float4* wb = win + kb + (kb >> 4);
   const float4 me = win[lane + 16 + ((lane + 16) >> 4)];
@@ -295,21 +294,29 @@ __device__ __forceinline__ void cl_window(const KArgs<Real>& a, int64_t g0, int 
         list[cnt++] = ent;
       }
     } else {
+      // (as above: hits first; branches in the loop cost 35,000 cycles a tile)
+      unsigned long long hits = 0ull;
       for (int c = 0; c < 48; ++c) {
         const float4 o = wb[c + (c >> 4)];
         const int ow = __float_as_int(o.w);
-        const int j = (int)g0 - 16 + kb + c;
-        if (!(ow & CL_VALID) || j == g || (ow >> 8) != (mew >> 8)) continue;
         float d[3] = {o.x - me.x, o.y - me.y, o.z - me.z};
-        int sc3[3];
-        for (int q = 0; q < 3; ++q) {
-          const float s = -rintf(d[q] * a.invLf[q]);
-          d[q] = fmaf(s, a.Lf[q], d[q]);
-          sc3[q] = (int)s;
-        }
+        for (int q = 0; q < 3; ++q) d[q] = fmaf(-rintf(d[q] * a.invLf[q]), a.Lf[q], d[q]);
         const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        const float rl2 = list_r2(a.c, ((g ^ j) & 1) != 0, st_g && (ow & 1));
-        if (r2 < rl2) cl_append(list, cnt, total, a.cap, ent_make(j, sc3[0], sc3[1], sc3[2]));
+        const float rl2 = list_r2(a.c, ((lane ^ c) & 1) != 0, st_g && (ow & 1));
+        const bool hit = r2 < rl2 && (ow & CL_VALID) && (ow >> 8) == (mew >> 8);
+        hits |= (unsigned long long)hit << c;
+      }
+      hits &= ~(1ull << (lane + 16 - kb));   // the bead itself
+      total = __popcll(hits);
+      for (; hits && cnt < a.cap; hits &= hits - 1ull) {
+        const int c = __ffsll((long long)hits) - 1;
+        int sc3[3] = {0, 0, 0};
+        if constexpr (sizeof(Real) == 8) {
+          const float4 o = wb[c + (c >> 4)];
+          const float d[3] = {o.x - me.x, o.y - me.y, o.z - me.z};
+          for (int q = 0; q < 3; ++q) sc3[q] = (int)-rintf(d[q] * a.invLf[q]);
+        }
+        list[cnt++] = ent_make((int)g0 - 16 + kb + c, sc3[0], sc3[1], sc3[2]);
       }
     }
   }

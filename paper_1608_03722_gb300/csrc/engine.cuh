@@ -160,6 +160,9 @@ struct KArgs {
   unsigned long long* rs_head;   // [rs_mask + 1] epoch of the rebuild << 32 | first item
   unsigned* rs_next;             // [nseg16 + n] next item of the list
   unsigned rs_mask;
+  int* rs_part;                  // [nseg16] slots of each segment's first part (16 in one molecule)
+  float4* rs_sph1;               // [nseg16] bounding sphere of the second part
+  float rs_rcap, rs_invh;        // widest part kept whole; cells per nm in an open box
   uint4* rs_xch;      // [2][ns][records] positions passed between CTAs
   unsigned* rs_seq;   // sequence number of the next launch's first step
   int periodic;

@@ -611,22 +611,34 @@ __device__ __forceinline__ bool hbond(const KArgs<Real>& a, const SPos<Real>& me
 }
 
 // Applied load on a nucleotide of the last base pair (Sec. 4.1, 4.2), q its
-// partner: f/2 at each centre, torque as a couple normal to its axis; half on
-// each site.
+// partner: Fe = f/2 at each centre, torque Tq as a couple normal to its axis;
+// half on each site.
 template <class Real>
-__device__ __forceinline__ void add_load(const KArgs<Real>& a, int mol, const SPos<Real>& me, const SPos<Real>& q,
-                                         V3<Real>& Fb, V3<Real>& Fp) {
+__device__ __forceinline__ void read_load(const KArgs<Real>& a, int mol, V3<Real>& Fe, V3<Real>& Tq) {
   const double* ex = a.ext + 8 * mol;
-  V3<Real> Fe{(Real)(0.5 * ex[0]), (Real)(0.5 * ex[1]), (Real)(0.5 * ex[2])};
-  const V3<Real> Tq{(Real)ex[3], (Real)ex[4], (Real)ex[5]};
+  Fe = V3<Real>{(Real)(0.5 * ex[0]), (Real)(0.5 * ex[1]), (Real)(0.5 * ex[2])};
+  Tq = V3<Real>{(Real)ex[3], (Real)ex[4], (Real)ex[5]};
+}
+template <class Real>
+__device__ __forceinline__ V3<Real> load_force(V3<Real> Fe, V3<Real> Tq, V3<Real> r) {   // r: partner's centre - own
   const Real tn2 = dot(Tq, Tq);
   if (tn2 > (Real)0) {
     const V3<Real> th = rsqrt_(tn2) * Tq;
-    V3<Real> rho = (Real)-0.5 * rel(me, q, a.fixq);   // centre offset from the pair centre
+    V3<Real> rho = (Real)-0.5 * r;   // centre offset from the pair centre
     rho -= dot(rho, th) * th;
     const Real S = (Real)2 * dot(rho, rho);
     if (S > (Real)1e-12) Fe += ((Real)1 / S) * cross(Tq, rho);
   }
+  return Fe;
+}
+// FP64 out of line: the compiler fuses products into sums kernel by kernel, and
+// every kernel has to round alike.
+static __device__ __noinline__ V3<double> load_force_fp64(V3<double> Fe, V3<double> Tq, V3<double> r) { return load_force(Fe, Tq, r); }
+template <class Real>
+__device__ __forceinline__ void add_load(const KArgs<Real>& a, V3<Real> Fe, V3<Real> Tq, const SPos<Real>& me,
+                                         const SPos<Real>& q, V3<Real>& Fb, V3<Real>& Fp) {
+  if constexpr (sizeof(Real) == 8) Fe = load_force_fp64(Fe, Tq, rel(me, q, a.fixq));
+  else Fe = load_force(Fe, Tq, rel(me, q, a.fixq));
   Fb += (Real)0.5 * Fe;
   Fp += (Real)0.5 * Fe;
 }
@@ -754,7 +766,11 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
       warp_pairs(a, sm, g, act, cur, Fb);
     }
     if (!act) return;
-    if (f & F_TOP) add_load(a, f >> MOL_SHIFT, me, sm.pos[ring(g ^ 1)], Fb, Fp);
+    if (f & F_TOP) {
+      V3<Real> Fe, Tq;
+      read_load(a, f >> MOL_SHIFT, Fe, Tq);
+      add_load(a, Fe, Tq, me, sm.pos[ring(g ^ 1)], Fb, Fp);
+    }
     if constexpr (MODE == MODE_FORCES) {
       double* o = a.fout + 6 * g;
       o[0] = Fb.x; o[1] = Fb.y; o[2] = Fb.z; o[3] = Fp.x; o[4] = Fp.y; o[5] = Fp.z;

@@ -30,10 +30,10 @@
 //    result stays in shared memory.
 // All forces, sums and updates are those of engine_kernel, term by term in the
 // same order, so trajectories agree bit for bit.  100 steps and one state
-// download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1957 ->
-// 778 us, periodic walk of 30 kbp 2244 -> 1089 us, 64 rings of 500 bp 3409 ->
-// 1745 us, melting 16 x 1000 bp 1811 -> 1059 us; 50 FP64 steps of 200 bp 3719
-// -> 1247 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
+// download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1953 ->
+// 682 us, periodic walk of 30 kbp 2232 -> 1104 us, 64 rings of 500 bp 3435 ->
+// 1220 us, melting 16 x 1000 bp 1807 -> 749 us; 50 FP64 steps of 200 bp 3722
+// -> 1224 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
 #pragma once
 #include "chainlist.cuh"
 #include "engine_kernels.cuh"
@@ -48,7 +48,7 @@ constexpr int RES_PAIRS_PER_SLOT = 4;   // list entries kept in shared memory pe
 constexpr int RES_HALO = 8;   // slots staged beyond either end of a stretch (the neighbourhoods of its owners)
 struct ResLayout {
   int len, own, pairs, warps;
-  size_t pos, flg, cs, cn, cp, pf, ent, off, po, jx, xo, xw, list, win, gi, gc, bytes;
+  size_t pos, flg, cs, cn, cp, pf, ent, off, po, jx, xo, xw, load, list, win, gi, gc, bytes;
 };
 template <class Real>
 __host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
@@ -68,6 +68,7 @@ __host__ __device__ inline ResLayout res_layout(int len, int rings, int T) {
   l.cn = take(sizeof(Real) * 6 * l.own);
   l.cp = take(sizeof(Real) * 3 * l.own);
   l.pf = take(sizeof(Real) * 3 * l.pairs);
+  l.load = take(sizeof(Real) * 6 * len);
   l.win = take(sizeof(float4) * (CL_WIN + CL_WIN / 16) * l.warps);
   l.gc = take(sizeof(float4) * 4 * l.warps);
   l.gi = take(sizeof(int) * 4 * l.warps);
@@ -146,6 +147,39 @@ __device__ __forceinline__ SPos<Real> rec_load(const KArgs<Real>& a, int cur, un
   return s;
 }
 
+// The same for three slots together; slots of the stretch come from spos.
+template <class Real>
+__device__ __forceinline__ void rec_load3(const KArgs<Real>& a, int cur, const int* slot, unsigned seq, unsigned* timeout,
+                                          const SPos<Real>* spos, int s0, int len, SPos<Real>* out) {
+  constexpr int R = res_records<Real>();
+  unsigned w[3][3 * R];
+  bool out_of[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) out_of[k] = (unsigned)(slot[k] - s0) >= (unsigned)len;
+  const unsigned long long t0 = clock64();
+  for (;;) {
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (out_of[k]) {
+        const uint4* p = a.rs_xch + R * ((size_t)cur * a.ns + (unsigned)slot[k]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const uint4 v = ld128(p + r);
+          w[k][3 * r] = v.x; w[k][3 * r + 1] = v.y; w[k][3 * r + 2] = v.z;
+          ok = ok && ((v.w ^ seq) & RES_SEQ) == 0u;
+        }
+      }
+    if (ok) break;
+    if ((unsigned long long)(clock64() - t0) > a.spin_budget) { *timeout = 1u; break; }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (out_of[k]) memcpy(&out[k], w[k], sizeof(SPos<Real>));
+    else out[k] = spos[slot[k] - s0];
+  }
+}
+
 // Agreement number p of a launch (step agreements and rebuild barriers share
 // one count) on word p mod 3 of bar->res: arrivals in bits 0-9, stale
 // stretches in bits 10-19, stretches with an error in bits 20-29 (their bits
@@ -191,9 +225,9 @@ struct ResSrc {
   }
 };
 
-// ResJunc: owners next to a junction, whose neighbours are taken modulo the
-// molecule (base pairs off .. off + N - 1): the stretch from shared memory,
-// other slots from their records.
+// ResJunc: an owner next to a junction, whose neighbours are taken modulo the
+// molecule (base pairs off .. off + N - 1): its three slots, waited for
+// together; the base pairs of the bubble rule one by one.
 template <class Real>
 struct ResJunc {
   const KArgs<Real>& a;
@@ -203,13 +237,25 @@ struct ResJunc {
   int cur;
   unsigned seq;
   int s0, len, off, N;
+  int slot[3];        // the owner, the next and the previous nucleotide of its strand
+  SPos<Real> p3[3];
   __device__ __forceinline__ int bp(int k) const {   // at most three base pairs outside the molecule
     return k < off ? k + N : (k >= off + N ? k - N : k);
   }
-  __device__ __forceinline__ SPos<Real> pos(int64_t g) const {
-    const unsigned l = (unsigned)((int)g - s0);
+  __device__ __forceinline__ void load(int o) {
+    const int dir = (o & 1) ? -2 : 2;
+    slot[0] = o;
+    slot[1] = (int)step(o, dir);
+    slot[2] = (int)step(o, -dir);
+    rec_load3(a, cur, slot, seq, timeout, spos, s0, len, p3);
+  }
+  __device__ __forceinline__ SPos<Real> at(int g) const {
+    const unsigned l = (unsigned)(g - s0);
     if (l < (unsigned)len) return spos[l];
     return rec_load(a, cur, (unsigned)g, seq, timeout);
+  }
+  __device__ __forceinline__ SPos<Real> pos(int64_t g) const {
+    return (int)g == slot[0] ? p3[0] : ((int)g == slot[1] ? p3[1] : p3[2]);
   }
   __device__ __forceinline__ int64_t step(int64_t g, int d) const {
     return 2 * bp(((int)g >> 1) + d / 2) + ((int)g & 1);
@@ -218,7 +264,7 @@ struct ResJunc {
     const int k = bp((int)k64);
     const unsigned l = (unsigned)(2 * k - s0);
     if (l < (unsigned)len) return (flg[l] & F_OPEN) != 0;
-    const SPos<Real> pa = pos(2 * k), pb = pos(2 * k + 1);
+    const SPos<Real> pa = at(2 * k), pb = at(2 * k + 1);
     const V3<Real> d = rel(pa, pb, a.fixq) + a.c.h * (uvec(pb) - uvec(pa));
     return dot(d, d) > a.c.rchb2;
   }
@@ -246,6 +292,19 @@ __device__ __forceinline__ V3<Real> res_pair(const KArgs<Real>& a, int s0, int b
 // ---------------------------------------------------------------- list build
 constexpr unsigned RES_NONE = 0xffffffffu;
 
+// The segment grid of the resident kernel: cells of the wide kernel's segment
+// grid in a periodic box; in an open box wider ones that keep segments of up to
+// DSDNA_RES_RCAP whole (a molten stretch spreads its 16 slots over 2 nm and
+// more, and bead by bead they cost four times a whole segment), hashed by
+// molecule and cell.
+template <class Real>
+__device__ __forceinline__ void res_cell(const KArgs<Real>& a, const float* p, int* ci) {
+  if (a.periodic) {
+    seg_cell(a, p[0], p[1], p[2], ci);
+  } else {
+    for (int c = 0; c < 3; ++c) ci[c] = (int)floorf(p[c] * a.rs_invh);
+  }
+}
 // Bucket of neighbour q (0..26; 13 is the cell itself) of cell ci.
 template <class Real>
 __device__ __forceinline__ unsigned res_key(const KArgs<Real>& a, int mol, const int* ci, int q) {
@@ -255,138 +314,199 @@ __device__ __forceinline__ unsigned res_key(const KArgs<Real>& a, int mol, const
   return hash_block(mol, cc[0], cc[1], cc[2]) & a.rs_mask;
 }
 
-// Grid item `id` (a segment, or bead id - nseg16 of a wide one) to the front of
-// its cell's list; a head of an earlier rebuild (another epoch) is an empty list.
+// A grid item is a segment, or its first part when it spans two molecules (id:
+// the segment), the second part (id: nseg16 + its first slot), or a bead of a
+// wide segment (nseg16 + its slot).  Into the front of its cell's list; a head
+// of an earlier rebuild (another epoch) is an empty list.
 template <class Real>
 __device__ __forceinline__ void res_insert(const KArgs<Real>& a, int mol, const float* p, unsigned id, unsigned epoch) {
   int ci[3];
-  seg_cell(a, p[0], p[1], p[2], ci);
+  res_cell(a, p, ci);
   const unsigned long long old =
       atomicExch(a.rs_head + res_key(a, mol, ci, 13), ((unsigned long long)epoch << 32) | id);
   a.rs_next[id] = (unsigned)(old >> 32) == epoch ? (unsigned)old : RES_NONE;
 }
-
-// Lists of the `nb` (16 or 32) beads from slot g0 on, one lane per bead.
+// Sphere and slot range (first slot | (beads - 1) << ENT_J_BITS) of item id.
 template <class Real>
-__device__ __forceinline__ void res_list(const KArgs<Real>& a, int64_t g0, int nb, unsigned epoch, float4* win, int* gi,
-                                         float4* gc, int* list, int& cnt, int& total) {
-  const int lane = threadIdx.x & 31;
-  const int g = (int)g0 + lane;
-  const bool in = lane < nb && g < a.n;
-  float4 raw[2];
-  int word[2];
-  bool val[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int64_t j = g0 - 16 + lane + 32 * h;
-    val[h] = j >= 0 && j < a.n;
-    raw[h] = val[h] ? a.wpos[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    word[h] = val[h] ? ((a.topo[j] & F_STERIC) | CL_VALID) : 0;
+__device__ __forceinline__ int res_item(const KArgs<Real>& a, unsigned id, float4& sph) {
+  const unsigned nseg = (unsigned)a.nseg16;
+  if (id < nseg) {
+    sph = a.segc[id];
+    const int nb = a.n_mol > 1 ? a.rs_part[id] : min(SEG_W, (int)a.n - (int)(id * SEG_W));
+    return (int)(id * SEG_W) | ((nb - 1) << ENT_J_BITS);
   }
-  const int64_t sA = g0 / SEG_W;
-  const bool hasB = nb > 16 && sA + 1 < a.nseg16;
-  const float4 sc[2] = {a.segc[sA], hasB ? a.segc[sA + 1] : make_float4(0.0f, 0.0f, 0.0f, -1.0f)};
-  const float4 mp = in ? a.wpos[g] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  // molecule of each segment (staged slots 16 and 32) and its slot range
-  const int qmol[2] = {__shfl_sync(0xffffffffu, __float_as_int(raw[0].w), 16),
-                       __shfl_sync(0xffffffffu, __float_as_int(raw[1].w), 0)};
-  // the cell lists around both segments: each lane walks one cell of either (a
-  // bucket that a lower lane of the same segment also reads is dropped)
-  unsigned id[2] = {RES_NONE, RES_NONE};
-  unsigned key[2] = {RES_NONE, RES_NONE};
+  const unsigned j = id - nseg, s = j / SEG_W;
+  const float4 whole = a.segc[s], second = a.rs_sph1[s], p = a.wpos[j];
+  if (whole.w < 0.0f) {
+    sph = make_float4(p.x, p.y, p.z, 0.0f);
+    return (int)j;
+  }
+  sph = second;
+  return (int)j | ((min((int)((s + 1) * SEG_W), (int)a.n) - (int)j - 1) << ENT_J_BITS);
+}
+
+// Bead g of a wide segment (wrapped position mp) against the items of its own 27
+// cells; returns (cnt, total).  Out of line: wide segments are rare.
+template <class Real>
+__device__ __noinline__ int2 res_list_bead(const KArgs<Real>& a, int g, float4 mp, bool st_g, unsigned epoch, int* list,
+                                           int cnt, int total) {
+  const int s = g / SEG_W;
+  int ci[3];
+  const float p3[3] = {mp.x, mp.y, mp.z};
+  res_cell(a, p3, ci);
+  const int pmol = __float_as_int(mp.w);
+  const int plo = a.n_mol > 1 ? 2 * (int)a.mol_off[pmol] : 0, phi = a.n_mol > 1 ? 2 * (int)a.mol_off[pmol + 1] : (int)a.n;
+  const float4 pt = make_float4(mp.x, mp.y, mp.z, 0.0f);
+  const unsigned most = (unsigned)(a.nseg16 + a.n);   // items there are at most
+  // the buckets first, all heads in flight together; a bucket two cells share is walked once
+  unsigned keys[27], hd[27];
+#pragma unroll
+  for (int q = 0; q < 27; ++q) {
+    keys[q] = res_key(a, pmol, ci, q);
+    const unsigned long long e = a.rs_head[keys[q]];
+    hd[q] = (unsigned)(e >> 32) == epoch ? (unsigned)e : RES_NONE;
+  }
+#pragma unroll
+  for (int q = 1; q < 27; ++q)
+#pragma unroll
+    for (int o = 0; o < q; ++o)
+      if (keys[o] == keys[q]) hd[q] = RES_NONE;
+#pragma unroll 1
+  for (int q = 0; q < 27; ++q) {
+    unsigned walked = 0;
+    for (unsigned e = hd[q]; e != RES_NONE && walked <= most; e = a.rs_next[e], ++walked) {
+      float4 it;
+      const int ir = res_item(a, e, it);
+      const int j0 = ir & ENT_JMASK, js = j0 / SEG_W;
+      if (j0 < plo || j0 >= phi || (js <= s + 1 && js >= s - 1)) continue;
+      if (cl_spheres_meet(a, pt, it)) cl_item_pairs(a, g, mp, st_g, ir, list, cnt, total);
+    }
+  }
+  return make_int2(cnt, total);
+}
+
+// Cell lists around the lanes' parts sc of segments sA, sA + 1 (radius < 0:
+// none) of molecules qmol: first item of the cell each lane walks for either
+// (a bucket that a lower lane of the same part also reads is dropped), and the
+// slot ranges of the molecules.
+struct ResQuery {
+  unsigned id[2];
+  int slo[2], shi[2];
+};
+template <class Real>
+__device__ __forceinline__ void res_query(const KArgs<Real>& a, const float4* sc, const int* qmol, unsigned epoch, ResQuery& q) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
+    unsigned key = RES_NONE;
     if (lane < 27 && sc[h].w >= 0.0f) {
       int ci[3];
-      seg_cell(a, sc[h].x, sc[h].y, sc[h].z, ci);
-      key[h] = res_key(a, qmol[h], ci, lane);
+      const float p[3] = {sc[h].x, sc[h].y, sc[h].z};
+      res_cell(a, p, ci);
+      key = res_key(a, qmol[h], ci, lane);
     }
-    const unsigned same = __match_any_sync(0xffffffffu, key[h]);
-    if (key[h] != RES_NONE && __ffs(same) - 1 == lane) {
-      const unsigned long long e = a.rs_head[key[h]];
-      if ((unsigned)(e >> 32) == epoch) id[h] = (unsigned)e;
+    q.id[h] = RES_NONE;
+    const unsigned same = __match_any_sync(0xffffffffu, key);
+    if (key != RES_NONE && __ffs(same) - 1 == lane) {
+      const unsigned long long e = a.rs_head[key];
+      if ((unsigned)(e >> 32) == epoch) q.id[h] = (unsigned)e;
+    }
+    q.slo[h] = 0;
+    q.shi[h] = (int)a.n;
+    if (a.n_mol > 1 && sc[h].w >= 0.0f) {
+      q.slo[h] = 2 * (int)a.mol_off[qmol[h]];
+      q.shi[h] = 2 * (int)a.mol_off[qmol[h] + 1];
     }
   }
-  int64_t slo[2] = {0, 0}, shi[2] = {a.n, a.n};
-  if (a.n_mol > 1) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (h == 0 || hasB) {
-        slo[h] = 2 * a.mol_off[qmol[h]];
-        shi[h] = 2 * a.mol_off[qmol[h] + 1];
-      }
-  }
-  const bool fast = cl_stage(a, lane, raw, word, val, win);
-  bool st_g = false;
-  cl_window(a, g0, lane, in, fast, win, st_g, list, cnt, total);
-  __syncwarp();
+}
+// Pairs of the lanes' beads (`in`) with the items of those lists.
+template <class Real>
+__device__ __forceinline__ void res_walk(const KArgs<Real>& a, ResQuery& q, const float4* sc, int sA, int g, bool in,
+                                         bool st_g, float4 mp, float4* win, int* gi, float4* gc, int* list, int& cnt,
+                                         int& total) {
+  const int lane = threadIdx.x & 31;
   const unsigned most = (unsigned)(a.nseg16 + a.n);   // items there are at most
-  for (unsigned walked = 0; walked <= most && __any_sync(0xffffffffu, id[0] != RES_NONE || id[1] != RES_NONE); ++walked) {
-    const int hq = id[0] != RES_NONE ? 0 : 1;
-    const unsigned e = hq ? id[1] : id[0];
+  for (unsigned walked = 0; walked <= most && __any_sync(0xffffffffu, q.id[0] != RES_NONE || q.id[1] != RES_NONE); ++walked) {
+    const int hq = q.id[0] != RES_NONE ? 0 : 1;
+    const unsigned e = hq ? q.id[1] : q.id[0];
     bool acc = false;
     int ir = 0;
     float4 it = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (e != RES_NONE) {
       const unsigned nx = a.rs_next[e];
-      if (hq) id[1] = nx; else id[0] = nx;
-      if (e < (unsigned)a.nseg16) {
-        it = a.segc[e];
-        const int64_t b0 = (int64_t)e * SEG_W;
-        ir = (int)b0 | (((int)min((int64_t)SEG_W, a.n - b0) - 1) << ENT_J_BITS);
-      } else {
-        const float4 p = a.wpos[e - (unsigned)a.nseg16];
-        it = make_float4(p.x, p.y, p.z, 0.0f);
-        ir = (int)(e - (unsigned)a.nseg16);
-      }
-      const int64_t j0 = ir & ENT_JMASK, js = j0 / SEG_W, s = sA + hq;
-      const int64_t lo_h = hq ? slo[1] : slo[0], hi_h = hq ? shi[1] : shi[0];
+      ir = res_item(a, e, it);
+      if (hq) q.id[1] = nx; else q.id[0] = nx;
+      const int j0 = ir & ENT_JMASK, js = j0 / SEG_W, s = sA + hq;
+      const int lo_h = hq ? q.slo[1] : q.slo[0], hi_h = hq ? q.shi[1] : q.shi[0];
       if (j0 >= lo_h && j0 < hi_h && (js > s + 1 || js < s - 1)) acc = cl_spheres_meet(a, hq ? sc[1] : sc[0], it);
     }
     cl_items(a, lane, g, in, st_g, sc, mp, acc, hq, ir, it, win, gi, gc, list, cnt, total);
   }
-  // a wide segment: each of its beads queries its own 27 cells
+}
+// The second parts (slots n0 on) of segments that span two molecules.  Out of
+// line: they are rare.
+template <class Real>
+__device__ __noinline__ int2 res_list_second(const KArgs<Real>& a, int sA, float4 scA, float4 scB, int n0A, int n0B, int g,
+                                             bool in, bool st_g, float4 mp, unsigned epoch, float4* win, int* gi, float4* gc,
+                                             int* list, int cnt, int total) {
+  const float4 sc[2] = {scA, scB};
+  const int qmol[2] = {scA.w >= 0.0f ? __float_as_int(a.wpos[SEG_W * sA + n0A].w) : 0,
+                       scB.w >= 0.0f ? __float_as_int(a.wpos[SEG_W * (sA + 1) + n0B].w) : 0};
+  ResQuery q;
+  res_query(a, sc, qmol, epoch, q);
+  res_walk(a, q, sc, sA, g, in, st_g, mp, win, gi, gc, list, cnt, total);
+  return make_int2(cnt, total);
+}
+
+// Lists of the `nb` (16 or 32) beads from slot g0 on, one lane per bead.
+template <class Real>
+__device__ __forceinline__ void res_list(const KArgs<Real>& a, int g0, int nb, unsigned epoch, float4* win, int* gi,
+                                         float4* gc, int* list, int& cnt, int& total) {
+  const int lane = threadIdx.x & 31;
+  const int g = g0 + lane;
+  const bool in = lane < nb && g < (int)a.n;
+  float4 raw[2];
+  int word[2];
+  bool val[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    if (!(in && (lane >> 4) == h && (h == 0 || hasB) && sc[h].w < 0.0f)) continue;
-    const int64_t s = sA + h;
-    int ci[3];
-    seg_cell(a, mp.x, mp.y, mp.z, ci);
-    const int pmol = __float_as_int(mp.w);
-    const int64_t plo = a.n_mol > 1 ? 2 * a.mol_off[pmol] : 0, phi = a.n_mol > 1 ? 2 * a.mol_off[pmol + 1] : a.n;
-    const float4 pt = make_float4(mp.x, mp.y, mp.z, 0.0f);
-    // the buckets first, all heads in flight together; a bucket two cells share is walked once
-    unsigned keys[27], hd[27];
-#pragma unroll
-    for (int q = 0; q < 27; ++q) {
-      keys[q] = res_key(a, pmol, ci, q);
-      const unsigned long long e = a.rs_head[keys[q]];
-      hd[q] = (unsigned)(e >> 32) == epoch ? (unsigned)e : RES_NONE;
-    }
-#pragma unroll
-    for (int q = 1; q < 27; ++q)
-#pragma unroll
-      for (int o = 0; o < q; ++o)
-        if (keys[o] == keys[q]) hd[q] = RES_NONE;
-#pragma unroll 1
-    for (int q = 0; q < 27; ++q) {
-      unsigned walked = 0;
-      for (unsigned e = hd[q]; e != RES_NONE && walked <= most; e = a.rs_next[e], ++walked) {
-        const bool seg = e < (unsigned)a.nseg16;
-        const int64_t j0 = seg ? (int64_t)e * SEG_W : (int64_t)(e - (unsigned)a.nseg16), js = j0 / SEG_W;
-        if (j0 < plo || j0 >= phi || (js <= s + 1 && js >= s - 1)) continue;
-        float4 it;
-        int ir = (int)j0;
-        if (seg) {
-          it = a.segc[e];
-          ir |= ((int)min((int64_t)SEG_W, a.n - j0) - 1) << ENT_J_BITS;
-        } else {
-          const float4 p = a.wpos[j0];
-          it = make_float4(p.x, p.y, p.z, 0.0f);
-        }
-        if (cl_spheres_meet(a, pt, it)) cl_item_pairs(a, g, mp, st_g, ir, list, cnt, total);
-      }
-    }
+    const int j = g0 - 16 + lane + 32 * h;
+    val[h] = j >= 0 && j < (int)a.n;
+    raw[h] = val[h] ? a.wpos[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    word[h] = val[h] ? ((a.topo[j] & F_STERIC) | CL_VALID) : 0;
+  }
+  const int sA = g0 / SEG_W;
+  const bool hasB = nb > 16 && sA + 1 < (int)a.nseg16;
+  const float4 none = make_float4(0.0f, 0.0f, 0.0f, -1.0f);
+  const float4 sc[2] = {a.segc[sA], hasB ? a.segc[sA + 1] : none};
+  // slots of the first parts
+  const int n0A = a.n_mol > 1 ? a.rs_part[sA] : SEG_W, n0B = a.n_mol > 1 && hasB ? a.rs_part[sA + 1] : SEG_W;
+  const float4 mp = in ? a.wpos[g] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  // molecule of each segment's first slot (staged slots 16 and 32)
+  const int qmol[2] = {__shfl_sync(0xffffffffu, __float_as_int(raw[0].w), 16),
+                       __shfl_sync(0xffffffffu, __float_as_int(raw[1].w), 0)};
+  ResQuery q;
+  res_query(a, sc, qmol, epoch, q);
+  const bool fast = cl_stage(a, lane, raw, word, val, win);   // while the heads load
+  bool st_g = false;
+  cl_window(a, g0, lane, in, fast, win, st_g, list, cnt, total);
+  __syncwarp();
+  const bool second = (lane & 15) >= ((lane >> 4) ? n0B : n0A);   // of the segment's second molecule
+  res_walk(a, q, sc, sA, g, in && !second, st_g, mp, win, gi, gc, list, cnt, total);
+  const bool spA = sc[0].w >= 0.0f && n0A < min(SEG_W, (int)a.n - g0);
+  const bool spB = sc[1].w >= 0.0f && n0B < min(SEG_W, (int)a.n - g0 - SEG_W);
+  if (spA || spB) {
+    const int2 r = res_list_second(a, sA, spA ? a.rs_sph1[sA] : none, spB ? a.rs_sph1[sA + 1] : none, n0A, n0B, g,
+                                   in && second, st_g, mp, epoch, win, gi, gc, list, cnt, total);
+    cnt = r.x;
+    total = r.y;
+  }
+  // a wide segment: each of its beads queries its own 27 cells
+  const int lh = lane >> 4;
+  if (in && (lh == 0 || hasB) && (lh ? sc[1].w : sc[0].w) < 0.0f) {
+    const int2 r = res_list_bead(a, g, mp, st_g, epoch, list, cnt, total);
+    cnt = r.x;
+    total = r.y;
   }
   __syncwarp();
 }
@@ -413,6 +533,7 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   short* const jx = reinterpret_cast<short*>(sm + lay.jx);
   int* const xo = reinterpret_cast<int*>(sm + lay.xo);
   short* const xw = reinterpret_cast<short*>(sm + lay.xw);
+  Real* const ext = reinterpret_cast<Real*>(sm + lay.load);   // applied loads of last base pairs: [6][len]
   const int OC = lay.own;
   const unsigned ns = (unsigned)a.ns;
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nwarp = (int)(blockDim.x >> 5);
@@ -458,6 +579,12 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     Vd[0] = a.V[gu]; Vd[1] = a.V[ns + gu]; Vd[2] = a.V[2 * ns + gu];
     Om = V3<Real>{a.Om[gu], a.Om[ns + gu], a.Om[2 * ns + gu]};
     kr[0] = a.kref[gu]; kr[1] = a.kref[ns + gu]; kr[2] = a.kref[2 * ns + gu];
+    if (f & F_TOP) {
+      V3<Real> Fe, Tq;
+      read_load(a, f >> MOL_SHIFT, Fe, Tq);
+      ext[i] = Fe.x; ext[lay.len + i] = Fe.y; ext[2 * lay.len + i] = Fe.z;
+      ext[3 * lay.len + i] = Tq.x; ext[4 * lay.len + i] = Tq.y; ext[5 * lay.len + i] = Tq.z;
+    }
   }
   const int mol = f >> MOL_SHIFT;
   const bool frozen = (f & F_FROZEN) != 0;
@@ -592,13 +719,22 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   // owners next to junctions of circular molecules
   auto junction_chunk = [&](int c) {
     const int x = 32 * c + lane;
-    if (x < njo) {
-      const int o = xo[x], w = xw[x];
+    const bool on = x < njo;
+    ResJunc<Real> src{a, spos, flg, &s_to, cur, seq, s0, len, 0, 0, {}, {}};
+    int o = 0;
+    if (on) {
+      o = xo[x];
+      const int m = a.topo[o] >> MOL_SHIFT;
+      src.off = (int)a.mol_off[m];
+      src.N = (int)a.mol_off[m + 1] - src.off;
+      src.load(o);
+    }
+    __syncwarp();   // the lanes that waited for a record join the others
+    if (on) {
+      const int w = xw[x];
       const unsigned l = (unsigned)(o - s0);
       const bool home = w >= 2 && w < len + 2;
       int fo = (l < (unsigned)len ? flg[l] : a.topo[o]) | F_PREV | F_NEXT;   // both neighbours exist on a ring
-      const int m = fo >> MOL_SHIFT, off0 = (int)a.mol_off[m];
-      const ResJunc<Real> src{a, spos, flg, &s_to, cur, seq, s0, len, off0, (int)a.mol_off[m + 1] - off0};
       unsigned rm = 0u;
       if constexpr (EXT) {
         if (a.bubble) {
@@ -699,17 +835,31 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
         a.wpos[gu] = make_float4(pw[0], pw[1], pw[2], __int_as_float(mol));
         if constexpr (sizeof(Real) == 8) a.img[gu] = packed;
       }
-      float c3[3];
-      const float R = seg_sphere(a, mine, pw, c3);
+      // the segment's parts: one molecule, or two of them
       int mlo = mine ? mol : INT_MAX, mhi = mine ? mol : INT_MIN;
-      for (int o = 8; o > 0; o >>= 1) {
-        mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
-        mhi = max(mhi, __shfl_xor_sync(0xffffffffu, mhi, o, 16));
-      }
-      const bool wide = !(R <= a.sg_rcap) || mlo != mhi;
+      if (a.n_mol > 1)
+        for (int o = 8; o > 0; o >>= 1) {
+          mlo = min(mlo, __shfl_xor_sync(0xffffffffu, mlo, o, 16));
+          mhi = max(mhi, __shfl_xor_sync(0xffffffffu, mhi, o, 16));
+        }
+      const unsigned half = 0xffffu << (lane & 16);
+      const bool first = mine && mol == mlo, second = mine && mol == mhi && mhi != mlo;
+      const int n0 = __popc(__ballot_sync(0xffffffffu, first) & half);
+      const bool more = (__ballot_sync(0xffffffffu, mine && !first && !second) & half) != 0u;   // a third molecule
+      const bool two = (__ballot_sync(0xffffffffu, second) & half) != 0u;
+      float c3[3], d3[3] = {0.0f, 0.0f, 0.0f};
+      const float R = seg_sphere(a, first, 0, pw, c3);
+      float R1 = 0.0f;
+      if (__any_sync(0xffffffffu, two)) R1 = seg_sphere(a, second, n0 & 15, pw, d3);
+      const bool wide = more || !(R <= a.rs_rcap) || (two && !(R1 <= a.rs_rcap));
       if (mine && (lane & 15) == 0) {
         a.segc[g >> 4] = make_float4(c3[0], c3[1], c3[2], wide ? -1.0f : R);
+        a.rs_part[g >> 4] = n0;
         if (!wide) res_insert(a, mol, c3, (unsigned)(g >> 4), epoch);
+      }
+      if (two && second && !wide && (lane & 15) == n0) {
+        a.rs_sph1[g >> 4] = make_float4(d3[0], d3[1], d3[2], R1);
+        res_insert(a, mol, d3, (unsigned)a.nseg16 + gu, epoch);
       }
       if (mine && wide) res_insert(a, mol, pw, (unsigned)a.nseg16 + gu, epoch);
     }
@@ -751,17 +901,19 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
       if (mine && !frozen && !end) nucleotide_noise(a, local, step, mol, eb, ep);
     };
     if (!sync_warp && !end) {
-      // owners and list pairs, 32 at a time: the ends and the other owners to the
-      // last warps first, so that the first ones, whose threads also draw the
-      // noise, hold pairs
-      const int nin = (e1 - e0 + 31) >> 5, nco = 1 + nin + ((njo + 31) >> 5);
+      // owners and list pairs, 32 at a time: the ends, which wait for the
+      // neighbours, to the last warp alone, then owners to the last warps first,
+      // so that the first ones, whose threads also draw the noise, hold pairs
+      const int nj = (njo + 31) >> 5, nco = nj + ((e1 - e0 + 31) >> 5);
       const int ncp = npair <= lay.pairs ? (npair + 31) >> 5 : 0;
-      for (int c = nwork - 1 - warp; c < nco + ncp; c += nwork) {
-        if (c == 0) edge_chunk();
-        else if (c <= nin) owner(e0 + 32 * (c - 1) + lane, e0 + 32 * (c - 1) + lane < e1);
-        else if (c < nco) junction_chunk(c - 1 - nin);
-        else pair_chunk(c - nco);
-      }
+      const int nrest = nwork > 1 ? nwork - 1 : 1;
+      if (warp == nwork - 1) edge_chunk();
+      if (warp < nrest)
+        for (int c = nrest - 1 - warp; c < nco + ncp; c += nrest) {
+          if (c < nj) junction_chunk(c);
+          else if (c < nco) owner(e0 + 32 * (c - nj) + lane, e0 + 32 * (c - nj) + lane < e1);
+          else pair_chunk(c - nco);
+        }
     }
     if (it > 0) agree(before, [&] { if (sync_warp) draw_noise(); });
     if (!sync_warp || it == 0) draw_noise();
@@ -823,7 +975,9 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
           Fb += res_pair(a, s0, i, me, f, e, qj, fj);
         }
       }
-      if (f & F_TOP) add_load(a, mol, me, q, Fb, Fp);
+      if (f & F_TOP)
+        add_load(a, V3<Real>{ext[i], ext[lay.len + i], ext[2 * lay.len + i]},
+                 V3<Real>{ext[3 * lay.len + i], ext[4 * lay.len + i], ext[5 * lay.len + i]}, me, q, Fb, Fp);
       const V3<Real> F = Fb + Fp;
       const V3<Real> Tc = h * cross(um, Fp - Fb);
       V3<Real> un = um;
