@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -141,6 +142,49 @@ static void* dalloc(dsdna_ctx* c, size_t bytes) {
   return p;
 }
 
+// Pinned host slots of 64 bytes that kernels write results to, 64 to a page
+// shared by the contexts of the process (a page of its own takes 100 us to
+// allocate, a fifth of a small context's creation).  A page goes back when its
+// last slot does.
+struct HostPage {
+  char* mem = nullptr;
+  uint64_t used = 0;
+};
+static std::mutex g_pages_mutex;
+static std::vector<HostPage> g_pages;
+
+static double* host_slot() {
+  std::lock_guard<std::mutex> lock(g_pages_mutex);
+  HostPage* page = nullptr;
+  for (HostPage& p : g_pages)
+    if (~p.used) page = &p;
+  if (!page) {
+    HostPage p;
+    if (cudaHostAlloc((void**)&p.mem, 4096, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return nullptr;
+    g_pages.push_back(p);
+    page = &g_pages.back();
+  }
+  int k = 0;
+  while ((page->used >> k) & 1u) ++k;
+  page->used |= 1ull << k;
+  return (double*)(page->mem + 64 * k);
+}
+
+static void host_slot_free(double* slot) {
+  std::lock_guard<std::mutex> lock(g_pages_mutex);
+  for (size_t i = 0; i < g_pages.size(); ++i) {
+    HostPage& p = g_pages[i];
+    const ptrdiff_t at = (char*)slot - p.mem;
+    if (at < 0 || at >= 4096) continue;
+    p.used &= ~(1ull << (at / 64));
+    if (!p.used) {
+      cudaFreeHost(p.mem);
+      g_pages.erase(g_pages.begin() + (ptrdiff_t)i);
+    }
+    return;
+  }
+}
+
 static void free_all(dsdna_ctx* c) {
   for (auto& g : c->gexec)
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
@@ -149,7 +193,7 @@ static void free_all(dsdna_ctx* c) {
     else cudaFree(p);
   }
   c->bufs.clear();
-  if (c->obs_host) { cudaFreeHost(c->obs_host); c->obs_host = nullptr; }
+  if (c->obs_host) { host_slot_free(c->obs_host); c->obs_host = nullptr; }
 }
 
 // Philox4x32-10 (Salmon et al., SC'11) for the host-side initial velocities.
@@ -626,8 +670,8 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   ALLOC(obs_scratch, double, 3 * (size_t)(3 * (c->maxN + 4)) + (size_t)c->maxN + 4);   // curves + twist increments
   ALLOC(obs_part, double, obs_partials(c->maxN));
   ALLOC(obs_counter, unsigned, 1);
-  if (cudaHostAlloc((void**)&c->obs_host, 8 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
-      cudaHostGetDevicePointer((void**)&c->obs_out, c->obs_host, 0) != cudaSuccess)
+  c->obs_host = host_slot();
+  if (!c->obs_host || cudaHostGetDevicePointer((void**)&c->obs_out, c->obs_host, 0) != cudaSuccess)
     return bad(fail(c, DSDNA_ENOMEM, "host allocation failed: observables"));
   ALLOC(steps_left, int64_t, 1);
   ALLOC(iters, unsigned, 4);
@@ -713,11 +757,10 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
       cudaMemset(c->X, 0, (f64 ? 48 : 24) * ns) != cudaSuccess || cudaMemset(c->kref, 0, 12 * ns) != cudaSuccess ||
       cudaMemset(c->img, 0, 4 * ns) != cudaSuccess)
     return bad(fail(c, DSDNA_ECUDA, "initialisation"));
-  // sequence numbers start at 1: zeroed records match no step
-  const unsigned first_seq = 1;
+  // zeroed records match no step: sequence numbers start above zero
   if (c->resident && (cudaMemset(c->rs_head, 0, sizeof(unsigned long long) * ((size_t)c->rs_mask + 1)) != cudaSuccess ||
                       cudaMemset(c->rs_xch, 0, sizeof(uint4) * (f64 ? 4 : 2) * 2 * ns) != cudaSuccess ||
-                      cudaMemcpy(c->rs_seq, &first_seq, sizeof(first_seq), cudaMemcpyHostToDevice) != cudaSuccess))
+                      cudaMemset(c->rs_seq, 1, sizeof(unsigned)) != cudaSuccess))
     return bad(fail(c, DSDNA_ECUDA, "initialisation"));
   if (!f64 && (cudaMemset(c->Kw, 0, sizeof(int4) * 2 * ns) != cudaSuccess ||
                cudaMemset(c->U, 0, sizeof(float4) * 2 * ns) != cudaSuccess))

@@ -103,10 +103,45 @@ cudaError_t resident_launch(int mode, const KArgs<Real>& a, int grid, int T, siz
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   ResLayout lay = res_layout<Real>((int)(SEG_W * ((a.nseg16 + grid - 1) / grid)), a.n_junc > 0, T);
-  void* args[] = {const_cast<KArgs<Real>*>(&a), &lay};
+  ResOnce<false> once;
+  void* args[] = {const_cast<KArgs<Real>*>(&a), &lay, &once};
   const void* fn = (mode & MODE_EXT) ? (const void*)resident_kernel<Real, true> : (const void*)resident_kernel<Real, false>;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
+
+// One force evaluation (ONCE) of the configuration X, u in device memory.
+// Prepared per device by resident_once_prepare.
+#ifdef DSDNA_KERN_MIXED
+cudaError_t resident_once_prepare() {
+  const size_t most = res_layout<float>(res_max_len<float>(), 0, res_max_threads<float>()).bytes;
+  cudaError_t e = cudaFuncSetAttribute(resident_kernel<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(resident_kernel<float, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+cudaError_t resident_once(const KArgs<float>& a, int nsm, const int* off, int steric_phase, const double* X, const double* u,
+                          double* Fb, double* Fp, unsigned* err, cudaStream_t st) {
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nsm, 1023), a.nseg16));
+  const int len = SEG_W * (int)((a.nseg16 + grid - 1) / grid);
+  if (len > res_max_len<float>()) return cudaErrorInvalidConfiguration;
+  const int T = 32 * std::min(res_max_threads<float>() / 32, 2 * ((len + 31) / 32) + 2);
+  ResLayout lay = res_layout<float>(len, 0, T);
+  ResOnce<true> once{X, u, Fb, Fp, err, steric_phase, {}};
+  std::copy(off, off + a.n_mol + 1, once.off);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)T);
+  cfg.dynamicSmemBytes = lay.bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  void* args[] = {const_cast<KArgs<float>*>(&a), &lay, &once};
+  return cudaLaunchKernelExC(&cfg, a.bubble ? (const void*)resident_kernel<float, true, true>
+                                            : (const void*)resident_kernel<float, false, true>, args);
+}
+#endif
 
 // Kernel attributes of the rebuild kernels for the current device, set when a
 // context is created: the chain-window list build asks for the largest

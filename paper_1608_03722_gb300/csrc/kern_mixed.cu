@@ -1,4 +1,5 @@
 // kern_mixed.cu -- engine kernels with FP32 forces and FP64 position/velocity accumulation.
+#define DSDNA_KERN_MIXED 1   // the single force evaluation exists in mixed precision only
 #include "kern_launch.cuh"
 namespace dsdna {
 template cudaError_t engine_occupancy<float>(int, int, int*, size_t*);

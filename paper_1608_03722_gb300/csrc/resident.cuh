@@ -35,6 +35,7 @@
 // 1220 us, melting 16 x 1000 bp 1807 -> 749 us; 50 FP64 steps of 200 bp 3722
 // -> 1224 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
 #pragma once
+#include "../../include/dsdna.h"
 #include "chainlist.cuh"
 #include "engine_kernels.cuh"
 
@@ -511,12 +512,30 @@ __device__ __forceinline__ void res_list(const KArgs<Real>& a, int g0, int nb, u
   __syncwarp();
 }
 
+// Arguments of a single force evaluation (ONCE).
+template <bool ONCE>
+struct ResOnce {};
+template <>
+struct ResOnce<true> {
+  const double* X;              // [n][3] centres
+  const double* u;              // [n][3] orientations
+  double* Fb;                   // [n][3] bead and patch forces
+  double* Fp;
+  unsigned* err;                // error bits (host memory, mapped)
+  int steric_phase;
+  int off[DSDNA_NOALLOC_MAX_MOL + 1];   // base-pair offsets of the molecules
+};
+
 // ---------------------------------------------------------------- the kernel
 // Bound by latency: a step is the grid barrier, one pass of owners and pairs
 // out of shared memory and one pass of updates.
-template <class Real, bool EXT>
+// ONCE: one force evaluation of a configuration given in device memory instead
+// of steps (linear molecules, no loads): flags, mirror and lists are made from
+// it on the way, and the site forces go straight to the caller's arrays.
+template <class Real, bool EXT, bool ONCE = false>
 __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
-    resident_kernel(const __grid_constant__ KArgs<Real> a, const __grid_constant__ ResLayout lay) {
+    resident_kernel(const __grid_constant__ KArgs<Real> a, const __grid_constant__ ResLayout lay,
+                    const __grid_constant__ ResOnce<ONCE> once) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ unsigned s_fl[2], s_word, s_to;
   __shared__ int s_scan[33], s_nx, s_nj;
@@ -552,18 +571,40 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   const int g = s0 + i;
   const unsigned gu = (unsigned)(mine ? g : s0);
 
-  const int64_t step0 = *a.step;
-  int64_t budget = a.steps_left ? *a.steps_left : a.nsteps;
-  if (*a.err & B_ERRMASK) budget = 0;
-  const unsigned seq0 = *a.rs_seq;
-  unsigned epoch = (unsigned)*a.nrebuild;
+  const int64_t step0 = ONCE ? 0 : *a.step;
+  int64_t budget = ONCE ? 1 : (a.steps_left ? *a.steps_left : a.nsteps);
+  if (!ONCE && (*a.err & B_ERRMASK)) budget = 0;
+  const unsigned call = *a.rs_seq, seq0 = ONCE ? call + 1u : call;
+  unsigned epoch = ONCE ? call : (unsigned)*a.nrebuild;
   int cur = (int)(step0 & 1);
 
   // state into registers and shared memory
   double Xd[3] = {0, 0, 0}, Vd[3] = {0, 0, 0};
   V3<Real> Om{0, 0, 0};
   int kr[3] = {0, 0, 0}, packed = 0, f = 0;
-  if (mine) {
+  if constexpr (ONCE) {
+    if (blockIdx.x == 0)
+      for (int m = i; m <= a.n_mol; m += blockDim.x) const_cast<int64_t*>(a.mol_off)[m] = once.off[m];
+    if (mine) {
+      int lo = 0, hi = a.n_mol - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) / 2;
+        if (once.off[mid] <= g >> 1) lo = mid; else hi = mid - 1;
+      }
+      const int N = once.off[lo + 1] - once.off[lo], k = (g >> 1) - once.off[lo], q = (g & 1) ? N - 1 - k : k;
+      f = (q % 3 == once.steric_phase ? F_STERIC : 0) | (q > 0 ? F_PREV : 0) | (q < N - 1 ? F_NEXT : 0) | (lo << MOL_SHIFT);
+      double w[3];
+      for (int c = 0; c < 3; ++c) { Xd[c] = once.X[3 * gu + c]; w[c] = once.u[3 * gu + c]; }
+      const double l2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+      if (fabs(l2 - 1.0) > 1e-6) { const double l = sqrt(l2); w[0] /= l; w[1] /= l; w[2] /= l; }
+      const SPos<Real> me{fixs(Xd[0], a.fixS[0]), fixs(Xd[1], a.fixS[1]), fixs(Xd[2], a.fixS[2]),
+                          (Real)w[0], (Real)w[1], (Real)w[2]};
+      spos2[0][i] = me;
+      a.topo[gu] = f;
+      flg[i] = f;
+      rec_store(a, cur, gu, seq0, f, me);
+    }
+  } else if (mine) {
     SPos<Real> me;
     load_slot(a, cur, g, me);
     spos2[0][i] = me;
@@ -588,7 +629,7 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   }
   const int mol = f >> MOL_SHIFT;
   const bool frozen = (f & F_FROZEN) != 0;
-  const uint32_t local = mine ? (uint32_t)(g - 2 * (int)a.mol_off[mol]) : 0u;
+  const uint32_t local = mine && !ONCE ? (uint32_t)(g - 2 * (int)a.mol_off[mol]) : 0u;
   if (i == 0) { s_fl[0] = 0u; s_fl[1] = 0u; s_nx = 0; s_nj = 0; s_to = 0u; s_word = 0u; }
   __syncthreads();
   if constexpr (EXT) {
@@ -649,7 +690,7 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     const int p = off[i] + q;
     if (p < lay.pairs) { ent[p] = e; po[p] = (unsigned short)i; }
   };
-  {
+  if constexpr (!ONCE) {
     const int cnt = mine ? a.ncnt[gu] : 0;
     number_pairs(cnt);
     for (int q = 0; q < cnt; ++q) keep_entry(q, a.nbr[(unsigned)q * ns + gu]);
@@ -658,10 +699,10 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   // halo slot of this lane (edge_chunk), its static flags
   const int hl = lane < RES_HALO ? lane - RES_HALO : len + lane - RES_HALO, hs = s0 + hl;
   const bool halo = lane < 2 * RES_HALO && hs >= 0 && hs < (int)a.n;
-  const int hf = halo ? a.topo[hs] : 0;
+  int hf = !ONCE && halo ? a.topo[hs] : 0;
   __syncthreads();
 
-  unsigned errbits = 0, phase = 0, seq = seq0;
+  unsigned errbits = 0, phase = ONCE ? call : 0u, seq = seq0;
   SPos<Real>* spos = spos2[0];
   unsigned fl = 0;   // this thread's flags of the step
   // owners within `edge` slots of an end read the halo (five base pairs with the bubble rule)
@@ -887,6 +928,13 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   };
 
   int64_t it = 0;   // steps taken
+  if constexpr (ONCE) {
+    if (!rebuild(&s_fl[1])) {
+      budget = 0;
+      errbits = s_word;
+    }
+    if (halo) hf = a.topo[hs];
+  }
   for (;; ++it) {
     const bool end = it == budget;
     const int64_t step = step0 + it;
@@ -898,7 +946,7 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     V3<Real> eb{0, 0, 0}, ep{0, 0, 0};
     unsigned* const before = &s_fl[(it + 1) & 1];   // flags of the step before
     auto draw_noise = [&] {
-      if (mine && !frozen && !end) nucleotide_noise(a, local, step, mol, eb, ep);
+      if (!ONCE && mine && !frozen && !end) nucleotide_noise(a, local, step, mol, eb, ep);
     };
     if (!sync_warp && !end) {
       // owners and list pairs, 32 at a time: the ends, which wait for the
@@ -975,6 +1023,11 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
           Fb += res_pair(a, s0, i, me, f, e, qj, fj);
         }
       }
+      if constexpr (ONCE) {
+        double *ob = once.Fb + 3 * gu, *op = once.Fp + 3 * gu;
+        ob[0] = Fb.x; ob[1] = Fb.y; ob[2] = Fb.z;
+        op[0] = Fp.x; op[1] = Fp.y; op[2] = Fp.z;
+      } else {
       if (f & F_TOP)
         add_load(a, V3<Real>{ext[i], ext[lay.len + i], ext[2 * lay.len + i]},
                  V3<Real>{ext[3 * lay.len + i], ext[4 * lay.len + i], ext[5 * lay.len + i]}, me, q, Fb, Fp);
@@ -993,7 +1046,9 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
       rec_store(a, nxt, gu, seq0 + (unsigned)it + 1u, EXT ? flg[i] : 0, nw);
       snxt[i] = nw;
       if (moved(a, k0, k1, k2, un, kr)) fl |= B_STALE;
+      }
     }
+    if constexpr (ONCE) break;
     if constexpr (EXT) {
       if (a.bubble) {
         __syncwarp();
@@ -1010,6 +1065,13 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     if (lane == 0 && fl) atomicOr(&s_fl[it & 1], fl);
     fl = 0;
     __syncthreads();   // the next step's positions and this step's flags are complete
+  }
+  if constexpr (ONCE) {
+    if (i == 0 && s_to) fl |= B_ETIMEOUT;
+    fl = (__reduce_or_sync(0xffffffffu, fl) | errbits) & B_ERRMASK;
+    if (lane == 0 && fl) atomicOr_system(once.err, fl);
+    if (blockIdx.x == 0 && i == 0) *a.rs_seq = call + 1u;
+    return;
   }
   const int64_t done = it;
   // state back to memory: orientation and mirror into the buffer of the step

@@ -88,3 +88,36 @@ def test_rings_and_bubbles(prec, rule):
     V, Om = I.maxwell(u, rng)
     _both(n_bp, X, u, V, Om, ring=ring, precision=prec, skin=0.15, seed=7, dt=0.002, K2=1.0 if rule else 6.0,
           bubble_rule=rule, steps=400)
+
+
+@pytest.mark.parametrize("lengths", [[1], [8], [9, 1, 7], [1] * 9, [16, 16, 16], [1216, 1217], [8192], [300] * 27])
+@pytest.mark.parametrize("rule", [0, 1])
+def test_single_launch_forces(lengths, rule):
+    """dsdna_forces_noalloc in one launch: the forces of the context's separate
+    rebuild and force kernels bit for bit, at stretch edges, at its size limit
+    and with open base pairs."""
+    import ctypes as C
+    import torch
+    cfg = I.ragged_batch(lengths, seed=len(lengths), spread=0.02)
+    X = cfg.X.copy()
+    kw = dict(bubble_rule=rule)
+    if rule:
+        for k in range(0, len(X) // 2 - 5, 40):          # runs of four open pairs
+            for q in range(k, k + 4):
+                r = X[2 * q + 1] - X[2 * q]
+                X[2 * q + 1] += 0.5 * r / np.linalg.norm(r)
+        kw["R0"] = 3.0
+    p = D.dsdna_default_params(**kw)
+    ctx = D.Context(p, cfg.n_bp, X=X, u=cfg.u, V=cfg.V, Om=cfg.Om)
+    want = ctx.compute_forces()
+    ctx.close()
+    nb = cfg.n_bp.astype(np.int32)
+    d = [torch.tensor(a, dtype=torch.float64, device="cuda") for a in (X, cfg.u)]
+    F = [torch.full((len(X), 3), float("nan"), dtype=torch.float64, device="cuda") for _ in range(2)]
+    for _ in range(3):
+        rc = D.load().dsdna_forces_noalloc(C.byref(p), len(nb), nb.ctypes.data_as(C.POINTER(C.c_int)),
+                                           *[C.c_void_p(t.data_ptr()) for t in (*d, *F)],
+                                           C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+        for a, b in zip(F, want):
+            assert np.array_equal(a.cpu().numpy(), b)
