@@ -576,8 +576,8 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
              (c->p.rebuild_mode == 2 || (c->p.rebuild_mode == 0 && n <= DSDNA_FUSED_REBUILD_MAX_NT));
   // chain-window list build: a grid of 16-slot segments whose cells span two
   // of the widest segments kept whole plus the list radius; in a periodic box
-  // at least 3 cells per edge, in an open box hashed (at most half full with
-  // whole segments)
+  // at least 3 cells per edge, in an open box hashed (at most a quarter full
+  // with whole segments)
   c->sg_edge = (2.0 * DSDNA_SEG_RCAP + rmax) * 1.001 + 0.01;
   if (c->table == TABLE_LINEAR && c->p.list_build == 0) {
     bool fits = true;
@@ -593,7 +593,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
     }
   } else if (c->table == TABLE_HASH && c->p.list_build == 0) {
     unsigned Hs = 2048;
-    while ((int64_t)Hs < n / 8) Hs <<= 1;
+    while ((int64_t)Hs < n / 4) Hs <<= 1;   // a quarter full: 8 of 16 items a segment reads are its own
     c->chain = true;
     c->sg_mask = Hs - 1;
     c->sg_H = Hs + 2048;   // a last tile of empty entries: start[Hs] is a scanned entry

@@ -496,10 +496,8 @@ __global__ void __launch_bounds__(CL_WARPS * 32, 4) k_rebuild_list_chain(const K
         key[h] = seg_key(a, qmol[h], ci, lane);
       }
       if (!a.periodic) {
-        for (int o = 0; o < 27; ++o) {
-          const unsigned ko = __shfl_sync(0xffffffffu, key[h], o);
-          if (o < lane && ko == key[h]) key[h] = CL_NONE;
-        }
+        const unsigned same = __match_any_sync(0xffffffffu, key[h]);
+        if (__ffs(same) - 1 != lane) key[h] = CL_NONE;
       }
     }
     unsigned rb[2] = {0u, 0u}, re[2] = {0u, 0u};

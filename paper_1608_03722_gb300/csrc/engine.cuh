@@ -71,7 +71,7 @@ struct GridBar {
   unsigned gen;
   unsigned acc[3];
   unsigned pad[27];
-  unsigned res[3][32];   // words of the resident kernel's agreements, a 128-byte line each
+  unsigned res[3][32];   // barrier words, a 128-byte line each
 };
 
 template <class Real>
@@ -349,16 +349,22 @@ template <class Real> __device__ __forceinline__ V3<Real> uvec(const SPos<Real>&
 // Mirror coordinate: low 32 bits of round(x S) (ties away from zero).  One
 // FP64 multiply, then the rounding by integer operations on the bits of the
 // product (the FP64 pipe of GB300 runs at a small fraction of the integer
-// rate); exact for any |x S| below 2^63.
+// rate), exact for any |x S| below 2^63: with the 53-bit significand m and the
+// right shift sh, (m >> sh) plus the bit below, both by funnel shifts of its
+// words (13 instructions; 64-bit shifts and adds took 22).
 __device__ __forceinline__ int fixs(double x, double S) {
-  const long long b = __double_as_longlong(x * S);
-  const int sh = 1075 - (int)((b >> 52) & 0x7FF);          // right shift of the 53-bit significand
-  if (sh > 53) return 0;                                    // |x S| < 1/2 rounds to zero
-  if (sh < -40) return 0;                                   // an integer multiple of 2^32
-  const unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  const unsigned long long r = sh > 0 ? (m + (1ull << (sh - 1))) >> sh : m << (-sh);
-  const unsigned lo = (unsigned)r;
-  return b < 0 ? (int)(0u - lo) : (int)lo;
+  const double p = x * S;
+  const int hb = __double2hiint(p);
+  int sh = 1075 - ((hb >> 20) & 0x7FF);
+  unsigned hi = ((unsigned)hb & 0xFFFFFu) | 0x100000u, lo = (unsigned)__double2loint(p);
+  unsigned r;
+  if (sh > 0) {
+    if (sh > 32) { lo = hi; hi = 0u; sh -= 32; }
+    r = __funnelshift_rc(lo, hi, sh) + (__funnelshift_rc(lo, hi, sh - 1) & 1u);   // shifts past 32 give 0
+  } else {
+    r = sh < -31 ? 0u : lo << -sh;   // an integer already; a multiple of 2^32 from there on
+  }
+  return hb < 0 ? (int)(0u - r) : (int)r;
 }
 
 // FP64 -> FP32 (round to nearest even) and FP32 -> FP64 (exact) by integer
@@ -375,12 +381,22 @@ __device__ __forceinline__ float d2f_bits(double x) {
   const unsigned long long r = (t + 0x0FFFFFFFull + ((t >> 29) & 1ull)) >> 29;
   return __uint_as_float((unsigned)r | sign);
 }
+// The same on the two words: fewer instructions (list rebuild 210 -> 205 us at
+// 1 Mbp), but the step kernel, which waits on a conversion where the rebuild
+// issues, takes 112.4 us per step with the one above and 113.4 with this one.
+__device__ __forceinline__ float d2f_words(double x) {
+  const unsigned hb = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned sign = hb & 0x80000000u, a = hb & 0x7FFFFFFFu;
+  if (a < 0x38100000u) return __uint_as_float(sign);
+  const unsigned r = __funnelshift_l(lo, a - 0x38000000u, 3);   // rebias the exponent 1023 -> 127, drop 29 bits
+  const unsigned up = ((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (r & 1u)) >> 29;
+  return __uint_as_float((r + up) | sign);
+}
 __device__ __forceinline__ double f2d_bits(float f) {
   const unsigned u = __float_as_uint(f);
-  const unsigned a = u & 0x7FFFFFFFu;
-  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-  if (a < 0x00800000u) return __longlong_as_double((long long)sign);
-  return __longlong_as_double((long long)((((unsigned long long)a << 29) + 0x3800000000000000ull) | sign));
+  const unsigned a = u & 0x7FFFFFFFu, sign = u & 0x80000000u;
+  if (a < 0x00800000u) return __hiloint2double((int)sign, 0);
+  return __hiloint2double((int)(((a >> 3) + 0x38000000u) | sign), (int)(a << 29));
 }
 
 // bead offset -h u on the fixed-point grid (rebuild trigger only); Sf: grid units per nm
@@ -514,36 +530,34 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   return v;
 }
 
-// Grid-wide barrier of a cooperative launch that also ORs every block's flag
-// word.  The wait is bounded by a clock budget; on expiry the block reports
-// B_ETIMEOUT and the caller leaves the kernel.
-__device__ __forceinline__ unsigned grid_sync(GridBar* bar, unsigned nblocks,
-                                              unsigned local, unsigned long long budget, unsigned* s_word) {
+// Grid-wide barrier number `phase` of a cooperative launch (the launch clears
+// *bar) that also ORs every block's flag word.  Blocks arrive with one release
+// add on word phase mod 3 of bar->res -- arrivals in bits 0-15, blocks with
+// flags above them, whose flags are ORed into bar->acc first -- and poll that
+// word; block 0 clears the word of the barrier before, two barriers ahead of
+// its next use.  The wait is bounded by a clock budget; on expiry the block
+// reports B_ETIMEOUT and the caller leaves the kernel.  An atomic count, a
+// generation word with back-off and a flag word read after it took 0.8 us
+// longer per 1 Mbp step (112.5 -> 111.6 us).
+__device__ __forceinline__ unsigned grid_sync(GridBar* bar, unsigned nblocks, unsigned& phase, unsigned local,
+                                              unsigned long long budget, unsigned* s_word) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned g = ld_acquire(&bar->gen);
-    atomicOr(&bar->acc[g % 3], local);
-    __threadfence();
-    const unsigned arrived = atomicAdd(&bar->count, 1u);
-    unsigned res = 0;
-    if (arrived == nblocks - 1) {
-      atomicExch(&bar->count, 0u);
-      atomicExch(&bar->acc[(g + 1) % 3], 0u);
-      __threadfence();
-      atomicAdd(&bar->gen, 1u);
-    } else {
-      const unsigned long long t0 = clock64();
-      unsigned ns = 32;
-      while (ld_acquire(&bar->gen) == g) {
-        __nanosleep(ns);
-        if (ns < 256) ns <<= 1;
-        if ((unsigned long long)(clock64() - t0) > budget) { res = B_ETIMEOUT; break; }
-      }
+    const unsigned k = phase % 3;
+    if (local) atomicOr(&bar->acc[k], local);
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar->res[k]), "r"(local ? 65537u : 1u) : "memory");
+    const unsigned long long t0 = clock64();
+    unsigned v, res = 0;
+    while (((v = ld_acquire(bar->res[k])) & 65535u) != nblocks)
+      if ((unsigned long long)(clock64() - t0) > budget) { res = B_ETIMEOUT; break; }
+    if (v >> 16) res |= ld_acquire(&bar->acc[k]);   // final: every block ORed its flags before it arrived
+    if (blockIdx.x == 0) {
+      bar->res[(k + 2) % 3][0] = 0u;
+      bar->acc[(k + 2) % 3] = 0u;
     }
-    __threadfence();
-    res |= ld_acquire(&bar->acc[g % 3]);   // final once gen moved on; a load, not a serialised atomic
     *s_word = res;
   }
+  ++phase;
   __syncthreads();
   return *s_word;
 }

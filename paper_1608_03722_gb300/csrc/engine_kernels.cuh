@@ -881,27 +881,27 @@ __device__ void strip_pass(const KArgs<Real>& a, const SegSmem<Real>& sm, int64_
 // the barriers.  The list phase keeps each lane's buffer in the warp's
 // shared ring, which the next step restages.  Linear and hashed tables.
 template <class Real>
-__device__ unsigned fused_rebuild(const KArgs<Real>& a, const SegSmem<Real>& sm, int cur, unsigned* s_word,
-                                  unsigned* s_red) {
+__device__ unsigned fused_rebuild(const KArgs<Real>& a, const SegSmem<Real>& sm, int cur, unsigned& phase,
+                                  unsigned* s_word, unsigned* s_red) {
   static_assert(seg_warp_bytes<Real>() >= sizeof(int) * 32 * LIST_CAP, "list buffers must fit in a warp's ring");
   unsigned fl = 0;
   rebuild_bin(a, cur, fl);
-  unsigned r = grid_sync(a.bar, gridDim.x, fl, a.spin_budget, s_word);
+  unsigned r = grid_sync(a.bar, gridDim.x, phase, fl, a.spin_budget, s_word);
   if (r & B_ERRMASK) return r;
   rebuild_scan_a(a, s_red);
-  r = grid_sync(a.bar, gridDim.x, 0u, a.spin_budget, s_word);
+  r = grid_sync(a.bar, gridDim.x, phase, 0u, a.spin_budget, s_word);
   if (r & B_ERRMASK) return r;
   rebuild_scan_b(a, s_red);
-  r = grid_sync(a.bar, gridDim.x, 0u, a.spin_budget, s_word);
+  r = grid_sync(a.bar, gridDim.x, phase, 0u, a.spin_budget, s_word);
   if (r & B_ERRMASK) return r;
   rebuild_scatter(a);
-  r = grid_sync(a.bar, gridDim.x, 0u, a.spin_budget, s_word);
+  r = grid_sync(a.bar, gridDim.x, phase, 0u, a.spin_budget, s_word);
   if (r & B_ERRMASK) return r;
   fl = 0;
   int* list = reinterpret_cast<int*>(sm.pos) + (threadIdx.x & 31) * LIST_CAP;
   if (a.table == TABLE_LINEAR) rebuild_list_lanes<Real>(a, fl, list);
   else rebuild_list_lanes_hash<Real>(a, fl, list);
-  r = grid_sync(a.bar, gridDim.x, fl, a.spin_budget, s_word);
+  r = grid_sync(a.bar, gridDim.x, phase, fl, a.spin_budget, s_word);
   if (blockIdx.x == 0 && threadIdx.x == 0 && !(r & B_ERRMASK)) *a.nrebuild += 1;
   return r;
 }
@@ -933,7 +933,7 @@ __global__ void __launch_bounds__(engine_max_threads<Real>(), 1) engine_kernel(c
   if (MODE == MODE_STEP && (*a.err & B_ERRMASK)) budget = 0;
   int need = 0;
   int64_t done = 0;
-  unsigned errbits = 0;
+  unsigned errbits = 0, phase = 0;
   for (int64_t it = 0; it < budget; ++it) {
     const int64_t step = step0 + it;
     const int cur = (int)(step & 1);
@@ -941,7 +941,7 @@ __global__ void __launch_bounds__(engine_max_threads<Real>(), 1) engine_kernel(c
     __syncthreads();
     unsigned fl = 0;
     if (EXT && a.n_junc) {   // circular molecules: junction owners first, then a grid barrier
-      const unsigned r = grid_sync(a.bar, gridDim.x, junction_pass<Real, MODE>(a, cur), a.spin_budget, &s_word);
+      const unsigned r = grid_sync(a.bar, gridDim.x, phase, junction_pass<Real, MODE>(a, cur), a.spin_budget, &s_word);
       if (r & B_ERRMASK) { errbits = r; break; }
     }
     const int64_t wpb = blockDim.x >> 5;
@@ -955,13 +955,13 @@ __global__ void __launch_bounds__(engine_max_threads<Real>(), 1) engine_kernel(c
       errbits = s_fl;
       break;
     }
-    const unsigned r = grid_sync(a.bar, gridDim.x, s_fl, a.spin_budget, &s_word);
+    const unsigned r = grid_sync(a.bar, gridDim.x, phase, s_fl, a.spin_budget, &s_word);
     if (r & B_ERRMASK) { errbits = r; break; }
     ++done;
     if (r & B_STALE) {
       if constexpr (FUSED) {
         __shared__ unsigned s_red[32];
-        const unsigned rr = fused_rebuild(a, sm, (int)((step + 1) & 1), &s_word, s_red);
+        const unsigned rr = fused_rebuild(a, sm, (int)((step + 1) & 1), phase, &s_word, s_red);
         if (rr & B_ERRMASK) { errbits = rr; break; }
         continue;
       } else {

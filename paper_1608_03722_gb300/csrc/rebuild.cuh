@@ -68,9 +68,9 @@ __device__ __forceinline__ void bead_position_f(const KArgs<Real>& a, int cur, i
   const float h = (float)a.c.h;
   if constexpr (sizeof(Real) == 4) {
     const float4 u = a.U[(size_t)cur * a.ns + g];
-    b[0] = d2f_bits(a.X[g]) - h * u.x;
-    b[1] = d2f_bits(a.X[a.ns + g]) - h * u.y;
-    b[2] = d2f_bits(a.X[2 * a.ns + g]) - h * u.z;
+    b[0] = d2f_words(a.X[g]) - h * u.x;
+    b[1] = d2f_words(a.X[a.ns + g]) - h * u.y;
+    b[2] = d2f_words(a.X[2 * a.ns + g]) - h * u.z;
   } else {
     const double* X = a.X + (size_t)cur * 3 * a.ns;
     const double* u = a.ud + (size_t)cur * 3 * a.ns;

@@ -848,9 +848,9 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
         const SPos<Real> me = spos[i];
         float b[3];
         if constexpr (sizeof(Real) == 4) {
-          b[0] = d2f_bits(Xd[0]) - hf * me.ux;
-          b[1] = d2f_bits(Xd[1]) - hf * me.uy;
-          b[2] = d2f_bits(Xd[2]) - hf * me.uz;
+          b[0] = d2f_words(Xd[0]) - hf * me.ux;
+          b[1] = d2f_words(Xd[1]) - hf * me.uy;
+          b[2] = d2f_words(Xd[2]) - hf * me.uz;
           kr[0] = me.kx + bead_off(hf * me.ux, a.fixSf[0]);
           kr[1] = me.ky + bead_off(hf * me.uy, a.fixSf[1]);
           kr[2] = me.kz + bead_off(hf * me.uz, a.fixSf[2]);
