@@ -951,6 +951,19 @@ static int map_err(dsdna_ctx* c, unsigned bits) {
   return fail(c, DSDNA_ECUDA, "unknown device error");
 }
 
+// The error word to the context's pinned slot, queued with a call's results so
+// that one wait completes both.
+static int queue_error_word(dsdna_ctx* c) {
+  CK(cudaMemcpyAsync(c->obs_host + 7, c->err, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st), "read error word");
+  return DSDNA_OK;
+}
+static int queued_error(dsdna_ctx* c) {
+  CK(cudaStreamSynchronize(c->st), "synchronize");
+  unsigned bits = 0;
+  std::memcpy(&bits, c->obs_host + 7, sizeof(bits));
+  return map_err(c, bits);
+}
+
 static int sync_check(dsdna_ctx* c) {
   CK(cudaStreamSynchronize(c->st), "synchronize");
   unsigned bits = 0;
@@ -1064,16 +1077,19 @@ extern "C" int dsdna_energy_virial(dsdna_ctx* c, int mol, double energy[DSDNA_NT
   CK(cudaMemsetAsync(c->eout, 0, sizeof(double) * EOUT_STRIDE * c->n_mol, c->st), "clear energies");
   int rc = launch(c, MODE_ENERGY, 0);
   if (rc) return rc;
-  rc = sync_check(c);
-  if (rc) return rc;
-  std::vector<double> e((size_t)c->n_mol * EOUT_STRIDE);
-  CK(cudaMemcpy(e.data(), c->eout, sizeof(double) * e.size(), cudaMemcpyDeviceToHost), "read energies");
   const int m0 = mol < 0 ? 0 : mol, m1 = mol < 0 ? c->n_mol : mol + 1;
+  std::vector<double> e((size_t)(m1 - m0) * EOUT_STRIDE);
+  rc = queue_error_word(c);
+  if (rc) return rc;
+  CK(cudaMemcpyAsync(e.data(), c->eout + (size_t)m0 * EOUT_STRIDE, sizeof(double) * e.size(), cudaMemcpyDeviceToHost, c->st),
+     "read energies");
+  rc = queued_error(c);
+  if (rc) return rc;
   for (int k = 0; k < DSDNA_NTERMS; ++k) if (energy) energy[k] = 0.0;
   for (int k = 0; k < 6; ++k) if (virial) virial[k] = 0.0;
   for (int m = m0; m < m1; ++m) {
-    for (int k = 0; k < DSDNA_NTERMS; ++k) if (energy) energy[k] += e[(size_t)m * EOUT_STRIDE + k];
-    for (int k = 0; k < 6; ++k) if (virial) virial[k] += e[(size_t)m * EOUT_STRIDE + NTERMS + k];
+    for (int k = 0; k < DSDNA_NTERMS; ++k) if (energy) energy[k] += e[(size_t)(m - m0) * EOUT_STRIDE + k];
+    for (int k = 0; k < 6; ++k) if (virial) virial[k] += e[(size_t)(m - m0) * EOUT_STRIDE + NTERMS + k];
   }
   return DSDNA_OK;
 }
@@ -1220,16 +1236,13 @@ extern "C" int dsdna_compute_forces(dsdna_ctx* c, double* Fb, double* Fp) {
   if (c->poisoned) return fail(c, DSDNA_ESTATE, "context poisoned by an earlier error");
   int rc = launch(c, MODE_FORCES, 0);
   if (rc) return rc;
-  rc = sync_check(c);
+  rc = queue_error_word(c);
   if (rc) return rc;
-  std::vector<double> h((size_t)c->n * 6);
-  CK(cudaMemcpy(h.data(), c->fout, sizeof(double) * h.size(), cudaMemcpyDeviceToHost), "read forces");
-  for (int64_t i = 0; i < c->n; ++i)
-    for (int q = 0; q < 3; ++q) {
-      if (Fb) Fb[3 * i + q] = h[6 * i + q];
-      if (Fp) Fp[3 * i + q] = h[6 * i + 3 + q];
-    }
-  return DSDNA_OK;
+  // the kernel wrote both arrays as the caller wants them: straight into place
+  const size_t bytes = sizeof(double) * 3 * (size_t)c->n;
+  if (Fb) CK(cudaMemcpyAsync(Fb, c->fout, bytes, cudaMemcpyDeviceToHost, c->st), "read forces");
+  if (Fp) CK(cudaMemcpyAsync(Fp, c->fout + 3 * c->n, bytes, cudaMemcpyDeviceToHost, c->st), "read forces");
+  return queued_error(c);
 }
 
 extern "C" int dsdna_neighbor_pairs(dsdna_ctx* c, int64_t cap, int64_t* pi, int64_t* pj, int64_t* count) {

@@ -185,7 +185,7 @@ struct KArgs {
   int* rebuild;
   unsigned long long* nrebuild;
   // outputs
-  double* fout;    // MODE_FORCES: [n][6]
+  double* fout;    // MODE_FORCES: [2][n][3] bead, then patch forces
   double* eout;    // MODE_ENERGY: [n_mol][16]
   // step loop in a CUDA graph (conditional WHILE/IF nodes)
   int64_t* steps_left;              // steps still to run in this graph launch (null: run nsteps)

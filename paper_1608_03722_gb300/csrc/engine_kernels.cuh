@@ -772,8 +772,9 @@ __device__ __forceinline__ void nucleotide_pass(const KArgs<Real>& a, const SegS
       add_load(a, Fe, Tq, me, sm.pos[ring(g ^ 1)], Fb, Fp);
     }
     if constexpr (MODE == MODE_FORCES) {
-      double* o = a.fout + 6 * g;
-      o[0] = Fb.x; o[1] = Fb.y; o[2] = Fb.z; o[3] = Fp.x; o[4] = Fp.y; o[5] = Fp.z;
+      double *ob = a.fout + 3 * g, *op = ob + 3 * a.n;
+      ob[0] = Fb.x; ob[1] = Fb.y; ob[2] = Fb.z;
+      op[0] = Fp.x; op[1] = Fp.y; op[2] = Fp.z;
     } else {
       // rigid body (Sec. 2): force and torque about the centre
       const V3<Real> F = Fb + Fp;

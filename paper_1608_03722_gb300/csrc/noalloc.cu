@@ -174,15 +174,6 @@ __global__ void k_noalloc_prep(const double* X, const double* u, int64_t n, int6
   U[g] = make_float4((float)u0, (float)u1, (float)u2, 0.0f);
 }
 
-__global__ void k_noalloc_split(const double* fout, int64_t n, double* Fb, double* Fp) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n) return;
-  for (int c = 0; c < 3; ++c) {
-    Fb[3 * g + c] = fout[6 * g + c];
-    Fp[3 * g + c] = fout[6 * g + 3 + c];
-  }
-}
-
 }  // namespace
 
 extern "C" int dsdna_forces_noalloc(const dsdna_params* p, int n_mol, const int* n_bp, const double* X, const double* u,
@@ -346,8 +337,9 @@ extern "C" int dsdna_forces_noalloc(const dsdna_params* p, int n_mol, const int*
   // the bubble rule runs in the kernel instance that has it (same launch bounds, so the same grid fits)
   if (e == cudaSuccess) e = engine_launch<float>(MODE_FORCES | (ext ? MODE_EXT : 0), a, grid, NA_T, s->smem, st);
   if (e != cudaSuccess) return na_fail(DSDNA_ECUDA, cudaGetErrorString(e));
-  k_noalloc_split<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.fout, n, F_bead, F_patch);
-  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(F_bead, a.fout, 24 * (size_t)n, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(F_patch, a.fout + 3 * n, 24 * (size_t)n, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess) e = cudaGetLastError();
   unsigned bits = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&bits, ctrl, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
