@@ -320,7 +320,8 @@ int dsdna_get_bubble_mask(dsdna_ctx* ctx, int mol, unsigned char* mask);
 int dsdna_set_bubble_mask(dsdna_ctx* ctx, int mol, const unsigned char* mask);
 
 /* Conservative site forces (bead, patch) on every nucleotide at the current
- * state, including the applied loads, as FP64 host arrays [3*n_nt] each. */
+ * state, including the applied loads, as FP64 host arrays [3*n_nt] each.
+ * After a device-side error their contents are undefined. */
 int dsdna_compute_forces(dsdna_ctx* ctx, double* F_bead, double* F_patch);
 
 /* Build the neighbour list at the current state and return its pairs
@@ -378,13 +379,14 @@ int dsdna_autotune(const dsdna_params* base, const dsdna_system* sys, const dsdn
  * Scratch memory: one fixed device array of about 5 MB (cell table,
  * neighbour list, position mirrors), reserved on every GPU that loads the
  * library until the process exits.  The first call on a device looks up that
- * array's device address (cudaGetSymbolAddress) with the device current.  No
- * call can be captured into a CUDA graph: each copies the molecule table
- * from host memory and waits for its stream.  Every call reuses the same
- * array and starts by clearing what must begin at zero; calls that overlap on
- * the GPU (other streams, other host threads) race on it and must be
- * serialised by the caller.  Returns DSDNA_OK or a negative dsdna_status
- * (EFENE for a broken backbone bond, EOVERFLOW for more than 32 neighbours). */
+ * array's device address (cudaGetSymbolAddress) with the device current, and
+ * the first call of the process maps a page of the library's own static memory
+ * for the GPUs (cudaHostRegister), where the kernel reports errors.  No call
+ * can be captured into a CUDA graph: each waits for its stream.  Every call
+ * reuses the same array, so calls that overlap on the GPU (other streams,
+ * other host threads) race on it and must be serialised by the caller.
+ * Returns DSDNA_OK or a negative dsdna_status (EFENE for a broken backbone
+ * bond, EOVERFLOW for more than 32 neighbours). */
 #define DSDNA_NOALLOC_MAX_NT 16384
 #define DSDNA_NOALLOC_MAX_MOL 256
 int dsdna_forces_noalloc(const dsdna_params* params, int n_mol, const int* n_bp, const double* X, const double* u,

@@ -88,12 +88,17 @@ struct DeviceSetup {
   int grid = 0;
   size_t smem = 0;
   int nsm = 0;
-  unsigned* err = nullptr;         // pinned host word the single-launch path reports errors in
+  unsigned* err = nullptr;         // host word the single-launch path reports errors in
   unsigned* err_dev = nullptr;
   bool dirty = false;              // its last call failed: the barrier words start over
 };
 constexpr int NA_MAX_DEV = 64;
 DeviceSetup g_setup[NA_MAX_DEV];
+// The devices' error words, 64 bytes each, in a page of the library's own that
+// the first call maps for the GPUs (the call allocates nothing).
+alignas(4096) unsigned g_err_page[4096 / sizeof(unsigned)];
+bool g_err_mapped = false;
+static_assert(64 * NA_MAX_DEV <= sizeof(g_err_page), "one word per device");
 std::mutex g_setup_mutex;
 
 // error codes only: this entry point keeps no message state
@@ -125,9 +130,13 @@ int setup_device(int dev, DeviceSetup** out) {
     s.grid = std::min(bps * nsm, NA_MAX_GRID);
     s.nsm = nsm;
     if (resident_once_prepare() != cudaSuccess) return na_fail(DSDNA_ECUDA, "attributes of the force kernel");
-    if (!s.err && (cudaHostAlloc((void**)&s.err, 64, cudaHostAllocMapped) != cudaSuccess ||
-                   cudaHostGetDevicePointer((void**)&s.err_dev, s.err, 0) != cudaSuccess))
-      return na_fail(DSDNA_ECUDA, "error word");
+    if (!g_err_mapped) {
+      if (cudaHostRegister(g_err_page, sizeof(g_err_page), cudaHostRegisterMapped | cudaHostRegisterPortable) != cudaSuccess)
+        return na_fail(DSDNA_ECUDA, "error word");
+      g_err_mapped = true;
+    }
+    s.err = g_err_page + 16 * dev;
+    if (cudaHostGetDevicePointer((void**)&s.err_dev, s.err, 0) != cudaSuccess) return na_fail(DSDNA_ECUDA, "error word");
     s.base = static_cast<unsigned char*>(p);
     s.ready = true;
   }
