@@ -238,6 +238,36 @@ __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
 __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
 __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+// Quotient and root of the interaction terms.  In FP64 without branches: the
+// library's tests for special operands end a basic block each, and a term's
+// chain of FP64 latencies (a warp or two per SM in small systems) could not
+// overlap the next term's.  The hardware's 20-bit reciprocal (root) y is refined
+// by one third-order step and the result corrected by its exact remainder, as
+// in Markstein, IA-64 and Elementary Functions (2000), ch. 8 and 9: rounded to
+// nearest like the operators they stand for, but for about one operand in a
+// million.  Operands are separations and their products: normal numbers (a zero
+// divisor gives NaN, the root of zero is zero).  20 FP64 steps with a state
+// download: 200 bp 28 -> 26.5 us per step, 6000 bp 33.2 -> 31.3, 12,000 bp 44.5 ->
+// 42.3; errors against the 64-bit evaluation alike to the third digit.  rsqrt
+// written the same way gained nothing more.
+__device__ __forceinline__ float div_(float a, float b) { return a / b; }
+__device__ __forceinline__ double div_(double a, double b) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  const double e = fma(-b, y, 1.0);
+  y = fma(y, fma(e, e, e), y);
+  const double q = a * y;
+  return fma(fma(-b, q, a), y, q);
+}
+__device__ __forceinline__ float root_(float x) { return sqrtf(x); }
+__device__ __forceinline__ double root_(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = 0.5 * y, s0 = x * y, e = fma(-s0, h, 0.5);
+  const double s = fma(s0, fma(1.5 * e, e, e), s0);
+  const double r = fma(fma(-s, s, x), h, s);
+  return x > 0.0 ? r : x;
+}
 __device__ __forceinline__ float log_(float x) { return logf(x); }
 __device__ __forceinline__ double log_(double x) { return log(x); }
 __device__ __forceinline__ float exp_(float x) { return expf(x); }
@@ -432,13 +462,13 @@ template <class Real>
 __device__ __forceinline__ V3<Real> t_fene(const Coef<Real>& c, V3<Real> d, unsigned& fl, Real* E) {
   Real r2 = dot(d, d);
   if (r2 >= c.R02) { fl |= B_EFENE; r2 = (Real)0.98 * c.R02; }
-  const Real q = (Real)1 - r2 / c.R02;
-  Real fr = -c.K1 / q;
+  const Real q = (Real)1 - div_(r2, c.R02);
+  Real fr = div_(-c.K1, q);
   Real e = (Real)0, ew = (Real)0;
   if (E) e = (Real)-0.5 * c.K1 * c.R02 * log_(q);
   if (r2 < c.rcbb2) {
-    const Real s2 = c.sbb2 / r2, s6 = s2 * s2 * s2;
-    fr += (Real)24 * c.eps_bb * s6 * ((Real)2 * s6 - (Real)1) / r2;
+    const Real s2 = div_(c.sbb2, r2), s6 = s2 * s2 * s2;
+    fr += div_((Real)24 * c.eps_bb * s6 * ((Real)2 * s6 - (Real)1), r2);
     if (E) ew = (Real)4 * c.eps_bb * (s6 * s6 - s6 + (Real)0.25);
   }
   if (E) { E[0] += e; E[1] += ew; }
@@ -448,11 +478,11 @@ __device__ __forceinline__ V3<Real> t_fene(const Coef<Real>& c, V3<Real> d, unsi
 // App. A Eq. 13: d = p_next - p_this.
 template <class Real>
 __device__ __forceinline__ V3<Real> t_morse(const Coef<Real>& c, V3<Real> d, Real* E) {
-  const Real r = sqrt_(dot(d, d));
+  const Real r = root_(dot(d, d));
   const Real x = exp_(-c.lam * (r - c.r0m));
   if (E) E[5] += c.K4 * ((Real)1 - x) * ((Real)1 - x);
   // force on the second site: -dU/dr * d / r
-  return ((Real)-2 * c.K4 * c.lam * x * ((Real)1 - x) / r) * d;
+  return div_((Real)-2 * c.K4 * c.lam * x * ((Real)1 - x), r) * d;
 }
 
 // App. A Eq. 12 on A-E-F-B (positions relative to anything).  phi with the
@@ -463,7 +493,7 @@ __device__ __forceinline__ void t_dihedral(const Coef<Real>& c, V3<Real> A, V3<R
   const V3<Real> b1 = Ep - A, b2 = Fp - Ep, b3 = B - Fp;
   const V3<Real> n1 = cross(b1, b2), n2 = cross(b2, b3);
   const Real n1s = dot(n1, n1), n2s = dot(n2, n2), b2s = dot(b2, b2);
-  const Real lb2 = sqrt_(b2s);
+  const Real lb2 = root_(b2s);
   const Real y = lb2 * dot(b1, n2), x = dot(n1, n2);
   // sin(phi - d) and cos(phi - d) from (x, y) without the angle itself
   const Real inv = rsqrt_(x * x + y * y);
@@ -471,9 +501,9 @@ __device__ __forceinline__ void t_dihedral(const Coef<Real>& c, V3<Real> A, V3<R
   const Real s_pd = sp * c.cosd - cp * c.sind;   // sin(phi - d)
   if (E) E[4] += c.K3 * ((Real)1 + (cp * c.cosd + sp * c.sind));
   const Real dU = -c.K3 * s_pd;                  // dU/dphi
-  fA = (dU * lb2 / n1s) * n1;                    // -dU * (-|b2|/|n1|^2 n1)
-  fB = (-dU * lb2 / n2s) * n2;                   // -dU * (|b2|/|n2|^2 n2)
-  const Real p = dot(b1, b2) / b2s, q = dot(b3, b2) / b2s;
+  fA = div_(dU * lb2, n1s) * n1;                    // -dU * (-|b2|/|n1|^2 n1)
+  fB = div_(-dU * lb2, n2s) * n2;                   // -dU * (|b2|/|n2|^2 n2)
+  const Real p = div_(dot(b1, b2), b2s), q = div_(dot(b3, b2), b2s);
   fE = ((Real)-1 - p) * fA + q * fB;
   fF = p * fA - ((Real)1 + q) * fB;
 }
@@ -487,10 +517,10 @@ __device__ __forceinline__ void t_planar(const Coef<Real>& c, V3<Real> v1, V3<Re
   Real cs = dot(e1, e2);
   cs = cs > (Real)1 ? (Real)1 : (cs < (Real)-1 ? (Real)-1 : cs);
   const Real al = acos_(cs);
-  Real sn = sqrt_((Real)1 - cs * cs);
+  Real sn = root_((Real)1 - cs * cs);
   if (sn < (Real)1e-6) sn = (Real)1e-6;
   if (E) E[6] += (Real)0.5 * c.K5 * (al - c.alpha0) * (al - c.alpha0);
-  const Real k = c.K5 * (al - c.alpha0) / sn;    // dU/dalpha / sin(alpha)
+  const Real k = div_(c.K5 * (al - c.alpha0), sn);    // dU/dalpha / sin(alpha)
   f1 = (k * i1) * (e2 - cs * e1);
   f2 = (k * i2) * (e1 - cs * e2);
 }
@@ -512,9 +542,9 @@ template <class Real>
 __device__ __forceinline__ V3<Real> t_wca(const Coef<Real>& c, V3<Real> d, Real s2sig, Real rc2, Real* e) {
   const Real r2 = dot(d, d);
   if (r2 >= rc2) { *e = (Real)0; return V3<Real>{0, 0, 0}; }
-  const Real s2 = s2sig / r2, s6 = s2 * s2 * s2;
+  const Real s2 = div_(s2sig, r2), s6 = s2 * s2 * s2;
   *e = (Real)4 * c.eps * (s6 * s6 - s6 + (Real)0.25);
-  return ((Real)-24 * c.eps * s6 * ((Real)2 * s6 - (Real)1) / r2) * d;
+  return div_((Real)-24 * c.eps * s6 * ((Real)2 * s6 - (Real)1), r2) * d;
 }
 
 template <class Real>
