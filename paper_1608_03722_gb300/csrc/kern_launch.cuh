@@ -66,7 +66,14 @@ cudaError_t engine_launch(int mode, const KArgs<Real>& a, int grid, int T, size_
 // Launch shape of the resident kernel: blocks, threads and shared memory for n
 // slots (0 blocks: a stretch would be longer than a CTA holds).  One stretch of
 // whole segments per SM; warps for all owners and pairs of the stretch at once
-// (about two warps per 32 slots), at least one thread per slot.
+// (about two warps per 32 slots), at least one thread per slot.  In FP64, where
+// a second chunk in the same warp is another chain of FP64 latencies, four warps
+// per tile (20 steps of 1216 bp 563 -> 539 us, of four rings of 300 bp 833 -> 781;
+// the most a CTA holds from two tiles on).  Rings evaluate the owners next to
+// their junctions besides: three warps per tile up to three tiles (100 steps of
+// one ring of 500 bp 744 -> 661 us, 20 rings of 300 bp 930 -> 871), but at five
+// tiles the wider barriers cost more (12 rings of 1000 bp 840 -> 880); linear
+// molecules in mixed precision gain nothing (1216 bp 574 -> 583).
 template <class Real>
 cudaError_t resident_shape(int64_t n, int rings, bool ext, int nsm, int* grid, int* T, size_t* smem) {
   const int64_t nu = (n + SEG_W - 1) / SEG_W;
@@ -77,7 +84,8 @@ cudaError_t resident_shape(int64_t n, int rings, bool ext, int nsm, int* grid, i
     return cudaSuccess;
   }
   const int tiles = (int)(len + 31) / 32;
-  *T = 32 * std::min(res_max_threads<Real>() / 32, 2 * tiles + 2);
+  const int warps = sizeof(Real) == 8 ? 4 * tiles + 4 : rings && tiles <= 3 ? 3 * tiles + 3 : 2 * tiles + 2;
+  *T = 32 * std::min(res_max_threads<Real>() / 32, warps);
   *smem = res_layout<Real>((int)len, rings, *T).bytes;
   const void* fn = ext ? (const void*)resident_kernel<Real, true> : (const void*)resident_kernel<Real, false>;
   // the attribute is per kernel, shared by every context: the largest any may use
