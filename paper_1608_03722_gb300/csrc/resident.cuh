@@ -32,8 +32,13 @@
 // same order, so trajectories agree bit for bit.  100 steps and one state
 // download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1953 ->
 // 682 us, periodic walk of 30 kbp 2232 -> 1104 us, 64 rings of 500 bp 3435 ->
-// 1220 us, melting 16 x 1000 bp 1807 -> 749 us; 50 FP64 steps of 200 bp 3722
-// -> 1224 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
+// 1129 us, melting 16 x 1000 bp 1807 -> 734 us; 50 FP64 steps of 200 bp 3722
+// -> 1158 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
+//
+// A 200 bp FP64 step is 42,000 cycles: 27,000 for one pass of an owner's terms
+// (a chain of FP64 latencies), 3500 to gather forces, 9400 to update.  Dealing
+// the FP64 work in groups of few lanes over all schedulers was slower (24 -> 38
+// us): the pipe is shared by the SM and timed by warp instructions.
 #pragma once
 #include "../../include/dsdna.h"
 #include "chainlist.cuh"
@@ -955,9 +960,15 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
       const int nj = (njo + 31) >> 5, nco = nj + ((e1 - e0 + 31) >> 5);
       const int ncp = npair <= lay.pairs ? (npair + 31) >> 5 : 0;
       const int nrest = nwork > 1 ? nwork - 1 : 1;
+      // a warp with a junction chunk, which waits for other stretches too, gets
+      // no other chunk while these are at most half of the warps: with a share of
+      // the others it was last by 2000 of a step's 13,000 cycles (100 steps of 64
+      // rings of 500 bp 1185 -> 1129 us).  Up to three tiles there are warps for
+      // all chunks at once (kern_launch.cuh) and none is kept free (1% slower).
+      const int jw = lay.len > 96 && 2 * nj <= nrest ? nj : 0, w0 = nrest - 1 - warp;
       if (warp == nwork - 1) edge_chunk();
       if (warp < nrest)
-        for (int c = nrest - 1 - warp; c < nco + ncp; c += nrest) {
+        for (int c = w0; c < (w0 < jw ? nj : nco + ncp); c += w0 < jw ? nj : nrest - jw) {
           if (c < nj) junction_chunk(c);
           else if (c < nco) owner(e0 + 32 * (c - nj) + lane, e0 + 32 * (c - nj) + lane < e1);
           else pair_chunk(c - nco);
