@@ -31,9 +31,9 @@
 // All forces, sums and updates are those of engine_kernel, term by term in the
 // same order, so trajectories agree bit for bit.  100 steps and one state
 // download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1953 ->
-// 682 us, periodic walk of 30 kbp 2232 -> 1104 us, 64 rings of 500 bp 3435 ->
-// 1129 us, melting 16 x 1000 bp 1807 -> 734 us; 50 FP64 steps of 200 bp 3722
-// -> 1158 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
+// 669 us, periodic walk of 30 kbp 2232 -> 1107 us, 64 rings of 500 bp 3435 ->
+// 1146 us, melting 16 x 1000 bp 1807 -> 730 us; 50 FP64 steps of 200 bp 3722
+// -> 1154 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
 //
 // A 200 bp FP64 step is 42,000 cycles: 27,000 for one pass of an owner's terms
 // (a chain of FP64 latencies), 3500 to gather forces, 9400 to update.  Dealing
