@@ -121,3 +121,15 @@ def test_single_launch_forces(lengths, rule):
         assert rc == 0
         for a, b in zip(F, want):
             assert np.array_equal(a.cpu().numpy(), b)
+
+
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("rings,n_bp", [(30, 300), (250, 36), (40, 191)])
+def test_rings_in_long_stretches(prec, rings, n_bp):
+    """Stretches of more than 96 slots (FP64: up to 128), where junction owners have warps of their own: one or
+    more junctions per stretch, molecules that end inside a segment."""
+    parts = [I.ring_helix(n_bp, round(n_bp / 10), center=(0, 0, 0.5 * n_bp * m)) for m in range(rings)]
+    rng = np.random.default_rng(9)
+    X, u = I.perturb(np.concatenate([p[0] for p in parts]), np.concatenate([p[1] for p in parts]), rng, dx=0.005, dtheta=0.01)
+    V, Om = I.maxwell(u, rng)
+    _both([n_bp] * rings, X, u, V, Om, ring=[1] * rings, precision=prec, skin=0.15, seed=4, dt=0.002, steps=80)
