@@ -243,30 +243,37 @@ __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
 // chain of FP64 latencies (a warp or two per SM in small systems) could not
 // overlap the next term's.  The hardware's 20-bit reciprocal (root) y is refined
 // by one third-order step and the result corrected by its exact remainder, as
-// in Markstein, IA-64 and Elementary Functions (2000), ch. 8 and 9: rounded to
-// nearest like the operators they stand for, but for about one operand in a
-// million.  Operands are separations and their products: normal numbers (a zero
-// divisor gives NaN, the root of zero is zero).  20 FP64 steps with a state
-// download: 200 bp 28 -> 26.5 us per step, 6000 bp 33.2 -> 31.3, 12,000 bp 44.5 ->
-// 42.3; errors against the 64-bit evaluation alike to the third digit.  rsqrt
+// in Markstein, IA-64 and Elementary Functions (2000), ch. 8 and 9.  The root's
+// correction needs its factor 1 / 2 sqrt(x) refined too: with the 20-bit one a
+// root in ten million was a last bit off.  Equal to the operators bit for bit
+// (1e8 operands of the terms' ranges and next to ties; zeros, infinities and NaN
+// too), but subnormal operands and results are not corrected; special operands
+// go by selects on the words, beside the FP64 pipe.  20 FP64 steps with a state
+// download, operators -> these: 200 bp 557 -> 552 us, 6000 bp 654 -> 635, 12,000
+// bp 890 -> 856, 19,000 bp 1317 -> 1260, 32 rings of 500 bp 1344 -> 1284.  rsqrt
 // written the same way gained nothing more.
 __device__ __forceinline__ float div_(float a, float b) { return a / b; }
 __device__ __forceinline__ double div_(double a, double b) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  const double e = fma(-b, y, 1.0);
-  y = fma(y, fma(e, e, e), y);
-  const double q = a * y;
-  return fma(fma(-b, q, a), y, q);
+  double y0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(b));
+  const double e = fma(-b, y0, 1.0), y1 = fma(y0, fma(e, e, e), y0);
+  const int hb = __double2hiint(b), lb = __double2loint(b);
+  const bool ok = (unsigned)((hb & 0x7fffffff) - 0x00100000) < 0x7fc00000u;   // b and 1/b normal
+  // 1/b of an all-ones significand is a hair above the middle of two numbers: the upper one
+  const int up = (lb & (hb | (int)0xfff00000)) == -1 ? 1 : 0;
+  const double y = __hiloint2double(__double2hiint(ok ? y1 : y0), ok ? __double2loint(y1) + up : 0);
+  const double q = a * y, r = fma(fma(-b, q, a), y, q);
+  return ok && (unsigned)((__double2hiint(q) & 0x7fffffff) - 0x00100000) < 0x7fe00000u ? r : q;
 }
 __device__ __forceinline__ float root_(float x) { return sqrtf(x); }
 __device__ __forceinline__ double root_(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double h = 0.5 * y, s0 = x * y, e = fma(-s0, h, 0.5);
-  const double s = fma(s0, fma(1.5 * e, e, e), s0);
-  const double r = fma(fma(-s, s, x), h, s);
-  return x > 0.0 ? r : x;
+  const double h = 0.5 * y, s0 = x * y, e = fma(-s0, h, 0.5), p = fma(1.5 * e, e, e);
+  const double s = fma(s0, p, s0), h1 = fma(h, p, h);
+  const double r = fma(fma(-s, s, x), h1, s);
+  const int hi = __double2hiint(x);
+  return (hi & 0x7ff00000) == 0 || hi == 0x7ff00000 ? x : r;   // zero, infinity (a negative x gives NaN)
 }
 __device__ __forceinline__ float log_(float x) { return logf(x); }
 __device__ __forceinline__ double log_(double x) { return log(x); }
