@@ -6,6 +6,7 @@
 #include "engine_kernels.cuh"
 #include "rebuild.cuh"
 #include "chainlist.cuh"
+#include "once_calls.h"
 #include "resident.cuh"
 
 namespace dsdna {
@@ -126,14 +127,15 @@ cudaError_t resident_once_prepare() {
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(resident_kernel<float, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
-cudaError_t resident_once(const KArgs<float>& a, int nsm, const int* off, int steric_phase, const double* X, const double* u,
-                          double* Fb, double* Fp, unsigned* err, cudaStream_t st) {
+static_assert(ONCE_CALLS < RES_SEQ, "tags of calls between two clears differ");
+cudaError_t resident_once(const KArgs<float>& a, int nsm, const int* off, int steric_phase, unsigned call, const double* X,
+                          const double* u, double* Fb, double* Fp, unsigned* err, cudaStream_t st) {
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nsm, 1023), a.nseg16));
   const int len = SEG_W * (int)((a.nseg16 + grid - 1) / grid);
   if (len > res_max_len<float>()) return cudaErrorInvalidConfiguration;
   const int T = 32 * std::min(res_max_threads<float>() / 32, 2 * ((len + 31) / 32) + 2);
   ResLayout lay = res_layout<float>(len, 0, T);
-  ResOnce<true> once{X, u, Fb, Fp, err, steric_phase, {}};
+  ResOnce<true> once{X, u, Fb, Fp, err, steric_phase, call, {}};
   std::copy(off, off + a.n_mol + 1, once.off);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);

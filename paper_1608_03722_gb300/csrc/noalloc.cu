@@ -17,6 +17,7 @@
 
 #include "../../include/dsdna.h"
 #include "engine.cuh"
+#include "once_calls.h"
 
 namespace dsdna {
 template <class Real> cudaError_t engine_occupancy(int mode, int T, int* blocks_per_sm, size_t* smem);
@@ -24,8 +25,8 @@ template <class Real> cudaError_t engine_launch(int mode, const KArgs<Real>& a, 
 template <class Real> cudaError_t rebuild_launch(const KArgs<Real>& a, int scan_grid, cudaStream_t st);
 __attribute__((visibility("hidden"))) void fill_coef_mixed(const dsdna_params& p, Coef<float>& c);
 cudaError_t resident_once_prepare();
-cudaError_t resident_once(const KArgs<float>& a, int nsm, const int* off, int steric_phase, const double* X, const double* u,
-                          double* Fb, double* Fp, unsigned* err, cudaStream_t st);
+cudaError_t resident_once(const KArgs<float>& a, int nsm, const int* off, int steric_phase, unsigned call, const double* X,
+                          const double* u, double* Fb, double* Fp, unsigned* err, cudaStream_t st);
 }  // namespace dsdna
 
 using namespace dsdna;
@@ -69,8 +70,7 @@ constexpr size_t O_SEGC = O_NEXT + al((NA_SEG + NA_MAX_NT) * sizeof(unsigned));
 constexpr size_t O_PART = O_SEGC + al(NA_SEG * sizeof(float4));
 constexpr size_t O_SPH1 = O_PART + al(NA_SEG * sizeof(int));
 constexpr size_t O_XCH = O_SPH1 + al(NA_SEG * sizeof(float4));
-constexpr size_t O_CALL = O_XCH + al(2 * NA_MAX_NT * sizeof(uint4));   // calls made
-constexpr size_t O_RBAR = O_CALL + 256;                                  // its barrier words
+constexpr size_t O_RBAR = O_XCH + al(2 * NA_MAX_NT * sizeof(uint4));   // its barrier words
 constexpr size_t NA_BYTES = O_RBAR + al(sizeof(GridBar));
 static_assert(NA_MAX_NT / 8 <= NA_BUCKETS, "one bucket per eight nucleotides");
 
@@ -90,7 +90,8 @@ struct DeviceSetup {
   int nsm = 0;
   unsigned* err = nullptr;         // host word the single-launch path reports errors in
   unsigned* err_dev = nullptr;
-  bool dirty = false;              // its last call failed: the barrier words start over
+  OnceCalls calls;
+  bool dirty = false;              // its last call failed: the device words start over
 };
 constexpr int NA_MAX_DEV = 64;
 DeviceSetup g_setup[NA_MAX_DEV];
@@ -316,14 +317,19 @@ extern "C" int dsdna_forces_noalloc(const dsdna_params* p, int n_mol, const int*
     a.rs_rcap = periodic ? (float)DSDNA_SEG_RCAP : (float)DSDNA_RES_RCAP;
     a.rs_invh = (float)(1.0 / ((2.0 * DSDNA_RES_RCAP + std::sqrt((double)a.c.rl_max2)) * 1.001 + 0.01));
     a.rs_xch = reinterpret_cast<uint4*>(b + O_XCH);
-    a.rs_seq = reinterpret_cast<unsigned*>(b + O_CALL);
     a.bar = reinterpret_cast<GridBar*>(b + O_RBAR);
     int off[NA_MAX_MOL + 1];
     for (int m = 0; m <= n_mol; ++m) off[m] = (int)mol_off[m];
     cudaError_t e = cudaSuccess;
-    if (s->dirty) e = cudaMemsetAsync(a.bar, 0, sizeof(GridBar), st);
+    bool clear = false;
+    const unsigned call = s->calls.take(s->dirty, &clear);
+    if (clear) {
+      e = cudaMemsetAsync(a.bar, 0, sizeof(GridBar), st);
+      if (e == cudaSuccess) e = cudaMemsetAsync(a.rs_head, 0, NA_BUCKETS * sizeof(unsigned long long), st);
+      if (e == cudaSuccess) e = cudaMemsetAsync(a.rs_xch, 0, 2 * NA_MAX_NT * sizeof(uint4), st);
+    }
     *s->err = 0u;
-    if (e == cudaSuccess) e = resident_once(a, s->nsm, off, p->steric_phase, X, u, F_bead, F_patch, s->err_dev, st);
+    if (e == cudaSuccess) e = resident_once(a, s->nsm, off, p->steric_phase, call, X, u, F_bead, F_patch, s->err_dev, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     s->dirty = e != cudaSuccess || *s->err != 0u;
     if (e != cudaSuccess) return na_fail(DSDNA_ECUDA, cudaGetErrorString(e));

@@ -528,6 +528,7 @@ struct ResOnce<true> {
   double* Fp;
   unsigned* err;                // error bits (host memory, mapped)
   int steric_phase;
+  unsigned call;                // number of the call (once_calls.h)
   int off[DSDNA_NOALLOC_MAX_MOL + 1];   // base-pair offsets of the molecules
 };
 
@@ -579,8 +580,14 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   const int64_t step0 = ONCE ? 0 : *a.step;
   int64_t budget = ONCE ? 1 : (a.steps_left ? *a.steps_left : a.nsteps);
   if (!ONCE && (*a.err & B_ERRMASK)) budget = 0;
-  const unsigned call = *a.rs_seq, seq0 = ONCE ? call + 1u : call;
-  unsigned epoch = ONCE ? call : (unsigned)*a.nrebuild;
+  unsigned seq0, phase = 0u, epoch;
+  if constexpr (ONCE) {
+    phase = epoch = once.call;
+    seq0 = once.call + 1u;
+  } else {
+    seq0 = *a.rs_seq;
+    epoch = (unsigned)*a.nrebuild;
+  }
   int cur = (int)(step0 & 1);
 
   // state into registers and shared memory
@@ -707,7 +714,7 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   int hf = !ONCE && halo ? a.topo[hs] : 0;
   __syncthreads();
 
-  unsigned errbits = 0, phase = ONCE ? call : 0u, seq = seq0;
+  unsigned errbits = 0, seq = seq0;
   SPos<Real>* spos = spos2[0];
   unsigned fl = 0;   // this thread's flags of the step
   // owners within `edge` slots of an end read the halo (five base pairs with the bubble rule)
@@ -1081,7 +1088,6 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     if (i == 0 && s_to) fl |= B_ETIMEOUT;
     fl = (__reduce_or_sync(0xffffffffu, fl) | errbits) & B_ERRMASK;
     if (lane == 0 && fl) atomicOr_system(once.err, fl);
-    if (blockIdx.x == 0 && i == 0) *a.rs_seq = call + 1u;
     return;
   }
   const int64_t done = it;
