@@ -157,7 +157,7 @@ struct KArgs {
   float sg_rcap;     // widest segment kept whole in the grid
   float sg_reach;    // largest list radius plus a margin (sphere test)
   // resident kernel: hash of segment-grid cells to linked lists of grid items
-  unsigned long long* rs_head;   // [rs_mask + 1] epoch of the rebuild << 32 | first item
+  unsigned long long* rs_head;   // [rs_mask + 1] rebuild number and first item (cell_heads.h)
   unsigned* rs_next;             // [nseg16 + n] next item of the list
   unsigned rs_mask;
   int* rs_part;                  // [nseg16] slots of each segment's first part (16 in one molecule)

@@ -80,6 +80,7 @@ cudaError_t resident_shape(int64_t n, int rings, bool ext, int nsm, int* grid, i
   const int64_t nu = (n + SEG_W - 1) / SEG_W;
   *grid = (int)std::max<int64_t>(1, std::min<int64_t>(nsm, nu));
   const int64_t len = SEG_W * ((nu + *grid - 1) / *grid);
+  static_assert((int64_t)res_max_len<Real>() * 1023 * 17 / 16 < (1 << RES_ID_BITS), "item numbers fit the list heads");
   if (nsm < 1 || nsm > 1023 || len > res_max_len<Real>()) {
     *grid = 0;
     return cudaSuccess;

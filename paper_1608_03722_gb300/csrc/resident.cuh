@@ -41,6 +41,7 @@
 // us): the pipe is shared by the SM and timed by warp instructions.
 #pragma once
 #include "../../include/dsdna.h"
+#include "cell_heads.h"
 #include "chainlist.cuh"
 #include "engine_kernels.cuh"
 
@@ -296,8 +297,6 @@ __device__ __forceinline__ V3<Real> res_pair(const KArgs<Real>& a, int s0, int b
 }
 
 // ---------------------------------------------------------------- list build
-constexpr unsigned RES_NONE = 0xffffffffu;
-
 // The segment grid of the resident kernel: cells of the wide kernel's segment
 // grid in a periodic box; in an open box wider ones that keep segments of up to
 // DSDNA_RES_RCAP whole (a molten stretch spreads its 16 slots over 2 nm and
@@ -325,12 +324,12 @@ __device__ __forceinline__ unsigned res_key(const KArgs<Real>& a, int mol, const
 // wide segment (nseg16 + its slot).  Into the front of its cell's list; a head
 // of an earlier rebuild (another epoch) is an empty list.
 template <class Real>
-__device__ __forceinline__ void res_insert(const KArgs<Real>& a, int mol, const float* p, unsigned id, unsigned epoch) {
+__device__ __forceinline__ void res_insert(const KArgs<Real>& a, int mol, const float* p, unsigned id, unsigned long long epoch) {
   int ci[3];
   res_cell(a, p, ci);
   const unsigned long long old =
-      atomicExch(a.rs_head + res_key(a, mol, ci, 13), ((unsigned long long)epoch << 32) | id);
-  a.rs_next[id] = (unsigned)(old >> 32) == epoch ? (unsigned)old : RES_NONE;
+      atomicExch(a.rs_head + res_key(a, mol, ci, 13), res_head(epoch, id));
+  a.rs_next[id] = res_first(old, epoch);
 }
 // Sphere and slot range (first slot | (beads - 1) << ENT_J_BITS) of item id.
 template <class Real>
@@ -354,7 +353,7 @@ __device__ __forceinline__ int res_item(const KArgs<Real>& a, unsigned id, float
 // Bead g of a wide segment (wrapped position mp) against the items of its own 27
 // cells; returns (cnt, total).  Out of line: wide segments are rare.
 template <class Real>
-__device__ __noinline__ int2 res_list_bead(const KArgs<Real>& a, int g, float4 mp, bool st_g, unsigned epoch, int* list,
+__device__ __noinline__ int2 res_list_bead(const KArgs<Real>& a, int g, float4 mp, bool st_g, unsigned long long epoch, int* list,
                                            int cnt, int total) {
   const int s = g / SEG_W;
   int ci[3];
@@ -369,8 +368,7 @@ __device__ __noinline__ int2 res_list_bead(const KArgs<Real>& a, int g, float4 m
 #pragma unroll
   for (int q = 0; q < 27; ++q) {
     keys[q] = res_key(a, pmol, ci, q);
-    const unsigned long long e = a.rs_head[keys[q]];
-    hd[q] = (unsigned)(e >> 32) == epoch ? (unsigned)e : RES_NONE;
+    hd[q] = res_first(a.rs_head[keys[q]], epoch);
   }
 #pragma unroll
   for (int q = 1; q < 27; ++q)
@@ -400,7 +398,8 @@ struct ResQuery {
   int slo[2], shi[2];
 };
 template <class Real>
-__device__ __forceinline__ void res_query(const KArgs<Real>& a, const float4* sc, const int* qmol, unsigned epoch, ResQuery& q) {
+__device__ __forceinline__ void res_query(const KArgs<Real>& a, const float4* sc, const int* qmol, unsigned long long epoch,
+                                          ResQuery& q) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -413,10 +412,7 @@ __device__ __forceinline__ void res_query(const KArgs<Real>& a, const float4* sc
     }
     q.id[h] = RES_NONE;
     const unsigned same = __match_any_sync(0xffffffffu, key);
-    if (key != RES_NONE && __ffs(same) - 1 == lane) {
-      const unsigned long long e = a.rs_head[key];
-      if ((unsigned)(e >> 32) == epoch) q.id[h] = (unsigned)e;
-    }
+    if (key != RES_NONE && __ffs(same) - 1 == lane) q.id[h] = res_first(a.rs_head[key], epoch);
     q.slo[h] = 0;
     q.shi[h] = (int)a.n;
     if (a.n_mol > 1 && sc[h].w >= 0.0f) {
@@ -453,8 +449,8 @@ __device__ __forceinline__ void res_walk(const KArgs<Real>& a, ResQuery& q, cons
 // line: they are rare.
 template <class Real>
 __device__ __noinline__ int2 res_list_second(const KArgs<Real>& a, int sA, float4 scA, float4 scB, int n0A, int n0B, int g,
-                                             bool in, bool st_g, float4 mp, unsigned epoch, float4* win, int* gi, float4* gc,
-                                             int* list, int cnt, int total) {
+                                             bool in, bool st_g, float4 mp, unsigned long long epoch, float4* win, int* gi,
+                                             float4* gc, int* list, int cnt, int total) {
   const float4 sc[2] = {scA, scB};
   const int qmol[2] = {scA.w >= 0.0f ? __float_as_int(a.wpos[SEG_W * sA + n0A].w) : 0,
                        scB.w >= 0.0f ? __float_as_int(a.wpos[SEG_W * (sA + 1) + n0B].w) : 0};
@@ -466,7 +462,7 @@ __device__ __noinline__ int2 res_list_second(const KArgs<Real>& a, int sA, float
 
 // Lists of the `nb` (16 or 32) beads from slot g0 on, one lane per bead.
 template <class Real>
-__device__ __forceinline__ void res_list(const KArgs<Real>& a, int g0, int nb, unsigned epoch, float4* win, int* gi,
+__device__ __forceinline__ void res_list(const KArgs<Real>& a, int g0, int nb, unsigned long long epoch, float4* win, int* gi,
                                          float4* gc, int* list, int& cnt, int& total) {
   const int lane = threadIdx.x & 31;
   const int g = g0 + lane;
@@ -580,13 +576,15 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
   const int64_t step0 = ONCE ? 0 : *a.step;
   int64_t budget = ONCE ? 1 : (a.steps_left ? *a.steps_left : a.nsteps);
   if (!ONCE && (*a.err & B_ERRMASK)) budget = 0;
-  unsigned seq0, phase = 0u, epoch;
+  unsigned seq0, phase = 0u;
+  unsigned long long epoch;
   if constexpr (ONCE) {
-    phase = epoch = once.call;
+    phase = once.call;
+    epoch = once.call;
     seq0 = once.call + 1u;
   } else {
     seq0 = *a.rs_seq;
-    epoch = (unsigned)*a.nrebuild;
+    epoch = *a.nrebuild;
   }
   int cur = (int)(step0 & 1);
 
