@@ -320,8 +320,8 @@ int dsdna_get_bubble_mask(dsdna_ctx* ctx, int mol, unsigned char* mask);
 int dsdna_set_bubble_mask(dsdna_ctx* ctx, int mol, const unsigned char* mask);
 
 /* Conservative site forces (bead, patch) on every nucleotide at the current
- * state, including the applied loads, as FP64 host arrays [3*n_nt] each.
- * After a device-side error their contents are undefined. */
+ * state, including the applied loads, as FP64 host arrays [3*n_nt] each,
+ * left as they were after a device-side error. */
 int dsdna_compute_forces(dsdna_ctx* ctx, double* F_bead, double* F_patch);
 
 /* Build the neighbour list at the current state and return its pairs

@@ -1238,11 +1238,16 @@ extern "C" int dsdna_compute_forces(dsdna_ctx* c, double* Fb, double* Fp) {
   if (rc) return rc;
   rc = queue_error_word(c);
   if (rc) return rc;
-  // the kernel wrote both arrays as the caller wants them: straight into place
+  // after an error the caller's arrays stay as they were: the word is read
+  // before the copies, which go straight into place (the kernel wrote both
+  // arrays as the caller wants them)
+  rc = queued_error(c);
+  if (rc) return rc;
   const size_t bytes = sizeof(double) * 3 * (size_t)c->n;
   if (Fb) CK(cudaMemcpyAsync(Fb, c->fout, bytes, cudaMemcpyDeviceToHost, c->st), "read forces");
   if (Fp) CK(cudaMemcpyAsync(Fp, c->fout + 3 * c->n, bytes, cudaMemcpyDeviceToHost, c->st), "read forces");
-  return queued_error(c);
+  CK(cudaStreamSynchronize(c->st), "synchronize");
+  return DSDNA_OK;
 }
 
 extern "C" int dsdna_neighbor_pairs(dsdna_ctx* c, int64_t cap, int64_t* pi, int64_t* pj, int64_t* count) {
