@@ -204,7 +204,10 @@ typedef struct dsdna_system {
   const int* circular;   /* [n_mol] or NULL (all linear) */
 } dsdna_system;
 
-/* Device allocator used for every buffer of a context.  NULL: cudaMalloc/cudaFree. */
+/* Device allocator used for every buffer of a context or network.  NULL:
+ * cudaMalloc/cudaFree.  Blocks may have any alignment (one that does not start on
+ * a 16-byte boundary is released and asked for again with 15 bytes more); alloc
+ * returns NULL when out of memory. */
 typedef struct dsdna_allocator {
   void* (*alloc)(size_t bytes, void* user);
   void (*release)(void* ptr, void* user);

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/dsdna.h"
+#include "alloc.h"
 #include "engine.cuh"
 #include "obs.h"
 
@@ -49,7 +50,7 @@ struct dsdna_ctx {
   int64_t n = 0;
   int64_t ns = 0;                // row stride of the [component][slot] arrays (n rounded up to 32)
   int maxN = 0;
-  std::vector<void*> bufs;
+  std::vector<void*> bufs;       // as the allocator gave them
   int64_t bytes = 0;
   // device buffers
   double* X = nullptr; double* V = nullptr; void* Om = nullptr;
@@ -132,13 +133,15 @@ static int cuda_fail(dsdna_ctx* c, cudaError_t e, const char* what) {
 static void* dalloc(dsdna_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 16;
   bytes = (bytes + 255) & ~(size_t)255;
-  void* p = nullptr;
+  void *p = nullptr, *raw = nullptr;
   if (c->have_alloc) {
-    p = c->alloc.alloc(bytes, c->alloc.user);
+    p = alloc16(c->alloc, bytes, &raw);
   } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
     p = nullptr;
+  } else {
+    raw = p;
   }
-  if (p) { c->bufs.push_back(p); c->bytes += (int64_t)bytes; }
+  if (p) { c->bufs.push_back(raw); c->bytes += (int64_t)bytes; }
   return p;
 }
 

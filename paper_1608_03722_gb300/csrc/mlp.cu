@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "../../include/dsdna.h"
+#include "alloc.h"
 
 namespace {
 
@@ -504,16 +505,17 @@ struct dsdna_mlp {
   cudaStream_t st = nullptr;
   dsdna_allocator alloc{};
   bool have_alloc = false;
-  std::vector<void*> bufs;
+  std::vector<void*> bufs;   // as the allocator gave them
   int64_t adam_t = 0;
 };
 
 static void* mlp_alloc(dsdna_mlp* m, size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
-  void* p = nullptr;
-  if (m->have_alloc) p = m->alloc.alloc(bytes, m->alloc.user);
+  void *p = nullptr, *raw = nullptr;
+  if (m->have_alloc) p = dsdna::alloc16(m->alloc, bytes, &raw);
   else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
-  if (p) m->bufs.push_back(p);
+  else raw = p;
+  if (p) m->bufs.push_back(raw);
   return p;
 }
 
