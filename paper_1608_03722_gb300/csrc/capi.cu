@@ -11,13 +11,13 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <string>
 #include <vector>
 
 #include "../../include/dsdna.h"
 #include "alloc.h"
 #include "engine.cuh"
+#include "host_slots.h"
 #include "obs.h"
 
 namespace dsdna {
@@ -145,48 +145,14 @@ static void* dalloc(dsdna_ctx* c, size_t bytes) {
   return p;
 }
 
-// Pinned host slots of 64 bytes that kernels write results to, 64 to a page
-// shared by the contexts of the process (a page of its own takes 100 us to
-// allocate, a fifth of a small context's creation).  A page goes back when its
-// last slot does.
-struct HostPage {
-  char* mem = nullptr;
-  uint64_t used = 0;
-};
-static std::mutex g_pages_mutex;
-static std::vector<HostPage> g_pages;
-
-static double* host_slot() {
-  std::lock_guard<std::mutex> lock(g_pages_mutex);
-  HostPage* page = nullptr;
-  for (HostPage& p : g_pages)
-    if (~p.used) page = &p;
-  if (!page) {
-    HostPage p;
-    if (cudaHostAlloc((void**)&p.mem, 4096, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return nullptr;
-    g_pages.push_back(p);
-    page = &g_pages.back();
-  }
-  int k = 0;
-  while ((page->used >> k) & 1u) ++k;
-  page->used |= 1ull << k;
-  return (double*)(page->mem + 64 * k);
+// Pinned host slots that kernels write results to (a page for every context
+// takes 100 us to allocate, a fifth of a small context's creation).
+static void* pinned_page() {
+  void* p = nullptr;
+  return cudaHostAlloc(&p, 4096, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess ? p : nullptr;
 }
-
-static void host_slot_free(double* slot) {
-  std::lock_guard<std::mutex> lock(g_pages_mutex);
-  for (size_t i = 0; i < g_pages.size(); ++i) {
-    HostPage& p = g_pages[i];
-    const ptrdiff_t at = (char*)slot - p.mem;
-    if (at < 0 || at >= 4096) continue;
-    p.used &= ~(1ull << (at / 64));
-    if (!p.used) {
-      cudaFreeHost(p.mem);
-      g_pages.erase(g_pages.begin() + (ptrdiff_t)i);
-    }
-    return;
-  }
-}
+static void pinned_page_free(void* p) { cudaFreeHost(p); }
+static HostSlots& pinned_slots() { return host_slots<pinned_page, pinned_page_free>(); }
 
 static void free_all(dsdna_ctx* c) {
   for (auto& g : c->gexec)
@@ -196,7 +162,7 @@ static void free_all(dsdna_ctx* c) {
     else cudaFree(p);
   }
   c->bufs.clear();
-  if (c->obs_host) { host_slot_free(c->obs_host); c->obs_host = nullptr; }
+  if (c->obs_host) { pinned_slots().give(c->obs_host); c->obs_host = nullptr; }
 }
 
 // Philox4x32-10 (Salmon et al., SC'11) for the host-side initial velocities.
@@ -673,7 +639,7 @@ extern "C" int dsdna_create(const dsdna_params* params, const dsdna_system* sys,
   ALLOC(obs_scratch, double, 3 * (size_t)(3 * (c->maxN + 4)) + (size_t)c->maxN + 4);   // curves + twist increments
   ALLOC(obs_part, double, obs_partials(c->maxN));
   ALLOC(obs_counter, unsigned, 1);
-  c->obs_host = host_slot();
+  c->obs_host = pinned_slots().take();
   if (!c->obs_host || cudaHostGetDevicePointer((void**)&c->obs_out, c->obs_host, 0) != cudaSuccess)
     return bad(fail(c, DSDNA_ENOMEM, "host allocation failed: observables"));
   ALLOC(steps_left, int64_t, 1);
