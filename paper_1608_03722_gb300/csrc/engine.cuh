@@ -572,17 +572,26 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
 // add on word phase mod 3 of bar->res -- arrivals in bits 0-15, blocks with
 // flags above them, whose flags are ORed into bar->acc first -- and poll that
 // word; block 0 clears the word of the barrier before, two barriers ahead of
-// its next use.  The wait is bounded by a clock budget; on expiry the block
+// its next use.  `local`: the block's flags (thread 0), with EACH those of each
+// thread (in the junction and rebuild phases only: at every barrier it cost 2% of
+// a mid-size step).  The wait is bounded by a clock budget; on expiry the block
 // reports B_ETIMEOUT and the caller leaves the kernel.  An atomic count, a
-// generation word with back-off and a flag word read after it took 0.8 us
-// longer per 1 Mbp step (112.5 -> 111.6 us).
+// generation word with back-off and a flag word read after it took 0.8 us longer
+// per 1 Mbp step (112.5 -> 111.6 us).
+template <bool EACH = false>
 __device__ __forceinline__ unsigned grid_sync(GridBar* bar, unsigned nblocks, unsigned& phase, unsigned local,
                                               unsigned long long budget, unsigned* s_word) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned k = phase % 3;
+  const unsigned k = phase % 3;
+  bool any = local != 0u;
+  if constexpr (EACH) {
     if (local) atomicOr(&bar->acc[k], local);
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar->res[k]), "r"(local ? 65537u : 1u) : "memory");
+    any = __syncthreads_or((int)local) != 0;
+  } else {
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    if (!EACH && local) atomicOr(&bar->acc[k], local);
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar->res[k]), "r"(any ? 65537u : 1u) : "memory");
     const unsigned long long t0 = clock64();
     unsigned v, res = 0;
     while (((v = ld_acquire(bar->res[k])) & 65535u) != nblocks)

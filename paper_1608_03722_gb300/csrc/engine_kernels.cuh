@@ -887,7 +887,7 @@ __device__ unsigned fused_rebuild(const KArgs<Real>& a, const SegSmem<Real>& sm,
   static_assert(seg_warp_bytes<Real>() >= sizeof(int) * 32 * LIST_CAP, "list buffers must fit in a warp's ring");
   unsigned fl = 0;
   rebuild_bin(a, cur, fl);
-  unsigned r = grid_sync(a.bar, gridDim.x, phase, fl, a.spin_budget, s_word);
+  unsigned r = grid_sync<true>(a.bar, gridDim.x, phase, fl, a.spin_budget, s_word);
   if (r & B_ERRMASK) return r;
   rebuild_scan_a(a, s_red);
   r = grid_sync(a.bar, gridDim.x, phase, 0u, a.spin_budget, s_word);
@@ -902,7 +902,7 @@ __device__ unsigned fused_rebuild(const KArgs<Real>& a, const SegSmem<Real>& sm,
   int* list = reinterpret_cast<int*>(sm.pos) + (threadIdx.x & 31) * LIST_CAP;
   if (a.table == TABLE_LINEAR) rebuild_list_lanes<Real>(a, fl, list);
   else rebuild_list_lanes_hash<Real>(a, fl, list);
-  r = grid_sync(a.bar, gridDim.x, phase, fl, a.spin_budget, s_word);
+  r = grid_sync<true>(a.bar, gridDim.x, phase, fl, a.spin_budget, s_word);
   if (blockIdx.x == 0 && threadIdx.x == 0 && !(r & B_ERRMASK)) *a.nrebuild += 1;
   return r;
 }
@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(engine_max_threads<Real>(), 1) engine_kernel(c
     __syncthreads();
     unsigned fl = 0;
     if (EXT && a.n_junc) {   // circular molecules: junction owners first, then a grid barrier
-      const unsigned r = grid_sync(a.bar, gridDim.x, phase, junction_pass<Real, MODE>(a, cur), a.spin_budget, &s_word);
+      const unsigned r = grid_sync<true>(a.bar, gridDim.x, phase, junction_pass<Real, MODE>(a, cur), a.spin_budget, &s_word);
       if (r & B_ERRMASK) { errbits = r; break; }
     }
     const int64_t wpb = blockDim.x >> 5;
