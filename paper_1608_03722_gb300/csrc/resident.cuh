@@ -845,6 +845,29 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
       if (lane == 0) s_word = res_agree(a, phase);
     }
   };
+  // A list beyond its capacity is agreed on one step after its build, and that
+  // step, without the pairs left out, is not kept: positions and velocities at
+  // the build wait in the list buffer (free until the next build; the lanes'
+  // words side by side), orientations in the other position buffer.  Written to
+  // memory instead, they had to arrive before the next agreement: 10 kbp 652 ->
+  // 664 us per 100 steps, here 660.
+  int* const kept = reinterpret_cast<int*>(sm + lay.list) + warp * 32 * LIST_CAP + lane;
+  auto keep_state = [&](bool back) {
+    int w = 0;
+    auto word = [&](int& x) {
+      if (back) x = kept[32 * w]; else kept[32 * w] = x;
+      ++w;
+    };
+    auto real = [&](auto& x) {
+      int p[sizeof(x) / 4];
+      memcpy(p, &x, sizeof(x));
+      for (unsigned q = 0; q < sizeof(x) / 4; ++q) word(p[q]);
+      memcpy(&x, p, sizeof(x));
+    };
+    static_assert(LIST_CAP >= 18, "the words of a state fit its lane's share of the list buffer");
+    for (int c = 0; c < 3; ++c) { real(Xd[c]); real(Vd[c]); }
+    real(Om.x); real(Om.y); real(Om.z);
+  };
   // bin the beads, thread the segments into the hash, wait for all, build the
   // CTA's own lists
   auto rebuild = [&](unsigned* flags) {
@@ -932,6 +955,10 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     }
     number_pairs(mine ? cnt : 0);
     for (int q = 0; q < cnt; ++q) keep_entry(q, list[q]);
+    if constexpr (!ONCE) {
+      __syncwarp();   // the lanes' lists are read
+      keep_state(false);
+    }
     if (blockIdx.x == 0 && i == 0) *a.nrebuild += 1;
     __syncthreads();
     return true;
@@ -984,7 +1011,15 @@ __global__ void __launch_bounds__(res_max_threads<Real>(), 1)
     __syncthreads();
     if (it > 0) {
       const unsigned r = s_word;
-      if (r & B_ERRMASK) { errbits = r; --it; break; }   // the last step was not taken
+      if (r & B_ERRMASK) {   // the last step was not taken
+        errbits = r;
+        --it;
+        if (r & B_EOVF) {
+          keep_state(true);
+          spos = snxt;
+        }
+        break;
+      }
       if (r & B_STALE) {
         if (!rebuild(before)) { errbits = s_word; break; }
         if (!end) {   // the pair forces once more, from the new lists
