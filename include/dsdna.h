@@ -334,7 +334,8 @@ int dsdna_neighbor_pairs(dsdna_ctx* ctx, int64_t cap, int64_t* pi, int64_t* pj, 
 
 int dsdna_get_info(const dsdna_ctx* ctx, dsdna_info* info);
 
-/* Step counter (number of steps queued so far). */
+/* Step counter: steps queued so far; once an error is reported, or replaced by
+ * a new state, the steps taken without one. */
 int64_t dsdna_step_counter(const dsdna_ctx* ctx);
 
 /* Text of the last error of ctx (or of the last failed create when ctx is NULL). */

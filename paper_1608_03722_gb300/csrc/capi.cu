@@ -909,9 +909,18 @@ static int step_host_loop(dsdna_ctx* c, int64_t nsteps) {
   return DSDNA_OK;
 }
 
+// The steps the device has taken: after an error fewer than were queued.  Every
+// copy of the state in or out goes by their parity.
+static int read_step(dsdna_ctx* c) {
+  CK(cudaMemcpy(&c->step, c->step_d, sizeof(c->step), cudaMemcpyDeviceToHost), "read step");
+  return DSDNA_OK;
+}
+
 static int map_err(dsdna_ctx* c, unsigned bits) {
   if (!bits) return DSDNA_OK;
   c->poisoned = true;
+  const int rc = read_step(c);
+  if (rc) return rc;
   if (bits & B_EFENE) return fail(c, DSDNA_EFENE, "backbone bond reached R0 (FENE diverges)");
   if (bits & B_ENAN) return fail(c, DSDNA_ENAN, "non-finite velocity");
   if (bits & B_EOVF) return fail(c, DSDNA_EOVERFLOW, "neighbour list capacity exceeded");
@@ -1129,6 +1138,30 @@ extern "C" int dsdna_profiles(dsdna_ctx* c, int mol, double* centre, double* twi
   return DSDNA_OK;
 }
 
+// After an error in a step of the strip kernel positions and velocities in place
+// are those after it, and what is kept twice (orientations and the mirror; in
+// FP64 positions) stands in the other buffer: into the one of the steps taken.
+static int settle_state(dsdna_ctx* c) {
+  unsigned bits = 0;
+  CK(cudaMemcpy(&bits, c->err, sizeof(bits), cudaMemcpyDeviceToHost), "read error word");
+  if (!(bits & B_AHEAD)) return DSDNA_OK;
+  const size_t ns = (size_t)c->ns, to = (size_t)(c->step & 1), from = to ^ 1;
+  auto copy = [&](void* p, size_t bytes) {   // a buffer of `bytes` to its twin
+    return cudaMemcpyAsync((char*)p + to * bytes, (char*)p + from * bytes, bytes, cudaMemcpyDeviceToDevice, c->st);
+  };
+  if (c->fp64()) {
+    CK(copy(c->X, 3 * sizeof(double) * ns), "settle state");
+    CK(copy(c->ud, 3 * sizeof(double) * ns), "settle state");
+  } else {
+    CK(copy(c->Kw, sizeof(int4) * ns), "settle state");
+    CK(copy(c->U, sizeof(float4) * ns), "settle state");
+  }
+  bits &= ~B_AHEAD;
+  CK(cudaMemcpyAsync(c->err, &bits, sizeof(bits), cudaMemcpyHostToDevice, c->st), "settle state");
+  CK(cudaStreamSynchronize(c->st), "settle state");
+  return DSDNA_OK;
+}
+
 extern "C" int dsdna_get_state(dsdna_ctx* c, int mol, double* X, double* V, double* u, double* Om) {
   if (!c) return DSDNA_EINVAL;
   if (mol < -1 || mol >= c->n_mol) return fail(c, DSDNA_EINVAL, "molecule index out of range");
@@ -1136,6 +1169,8 @@ extern "C" int dsdna_get_state(dsdna_ctx* c, int mol, double* X, double* V, doub
     // Post-mortem read: the engine stopped at the step that raised the error,
     // so the state shows it; the error itself stays in last_error.
     CK(cudaStreamSynchronize(c->st), "synchronize");
+    const int rc = settle_state(c);
+    if (rc) return rc;
   } else {
     int rc = sync_check(c);
     if (rc) return rc;
@@ -1162,6 +1197,9 @@ extern "C" int dsdna_set_state(dsdna_ctx* c, int mol, const double* X, const dou
   if (e != cudaSuccess) return cuda_fail(c, e, "set_state sync");
   c->poisoned = false;
   c->errmsg.clear();
+  int rc = read_step(c);   // an error may not have been seen yet
+  if (!rc) rc = settle_state(c);
+  if (rc) return rc;
   CK(cudaMemsetAsync(c->err, 0, 16, c->st), "clear errors");
   const int one = 1;
   CK(cudaMemcpyAsync(c->rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, c->st), "request rebuild");

@@ -44,6 +44,7 @@ enum : int { TABLE_HASH = 0, TABLE_MORTON = 1, TABLE_LINEAR = 2 };
 enum : unsigned {
   B_STALE = 1u, B_EFENE = 2u, B_ENAN = 4u, B_EOVF = 8u, B_ETIMEOUT = 16u, B_EIMG = 32u
 };
+constexpr unsigned B_AHEAD = 0x80000000u;   // in a.err: the state in memory is that after the step that failed, which is not counted
 constexpr unsigned B_ERRMASK = B_EFENE | B_ENAN | B_EOVF | B_ETIMEOUT | B_EIMG;
 enum : int { MODE_STEP = 0, MODE_FORCES = 1, MODE_ENERGY = 2 };
 constexpr int MODE_EXT = 4;   // launch flag: kernel instance with circular molecules / bubble rule

@@ -957,7 +957,7 @@ __global__ void __launch_bounds__(engine_max_threads<Real>(), 1) engine_kernel(c
       break;
     }
     const unsigned r = grid_sync(a.bar, gridDim.x, phase, s_fl, a.spin_budget, &s_word);
-    if (r & B_ERRMASK) { errbits = r; break; }
+    if (r & B_ERRMASK) { errbits = r | B_AHEAD; break; }
     ++done;
     if (r & B_STALE) {
       if constexpr (FUSED) {
@@ -972,7 +972,7 @@ __global__ void __launch_bounds__(engine_max_threads<Real>(), 1) engine_kernel(c
     }
   }
   if (threadIdx.x == 0) {
-    if (errbits & B_ERRMASK) atomicOr(a.err, errbits & B_ERRMASK);
+    if (errbits & B_ERRMASK) atomicOr(a.err, errbits & (B_ERRMASK | B_AHEAD));
     if (blockIdx.x == 0 && MODE == MODE_STEP) {
       *a.step = step0 + done;
       if (need) *a.rebuild = 1;
