@@ -4,11 +4,13 @@
 // Some callers cannot call cudaMalloc: processes whose device memory is
 // entirely reserved by another pool allocator, and tight loops that cannot
 // afford the device-wide synchronisation that cudaMalloc/cudaFree imply.
-// dsdna_forces_noalloc gives them the force pass of the engine (the same
-// persistent kernel in its forces mode: cell hash, neighbour list, bonded and
-// pair forces) with all of its scratch memory in one file-scope device array
-// of fixed size.  That array is reserved on every GPU that loads the library
-// and stays there until the process exits.
+// dsdna_forces_noalloc gives them the engine's forces with all of its scratch
+// memory in one file-scope device array of fixed size, reserved on every GPU
+// that loads the library until the process exits.  Open boxes, and periodic ones
+// of at least 3 segment-grid cells per edge, take one launch of the resident
+// kernel (chain-window lists, forces straight to the caller's arrays); smaller
+// periodic boxes the separate rebuild kernels (cell walk) and the strip kernel's
+// forces mode.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -295,7 +297,7 @@ extern "C" int dsdna_forces_noalloc(const dsdna_params* p, int n_mol, const int*
   // One launch where the chain-window lists apply (open box, or a periodic box
   // of at least 3 segment-grid cells per edge): the resident kernel stages the
   // configuration, builds the lists and writes the forces: 33 us for 5 x 1339
-  // bp, against 97 us as copies, clears, staging, five rebuild kernels, forces
+  // bp (the kernel 23), against 97 us as copies, clears, staging, five rebuild kernels, forces
   // and a split (which small periodic boxes still take).
   const double rmax = cellh / 1.0001, sg_edge = (2.0 * DSDNA_SEG_RCAP + rmax) * 1.001 + 0.01;
   bool chain = true;

@@ -31,14 +31,15 @@
 // All forces, sums and updates are those of engine_kernel, term by term in the
 // same order, so trajectories agree bit for bit.  100 steps and one state
 // download, strip kernel with in-kernel rebuild -> this kernel: 10 kbp 1953 ->
-// 669 us, periodic walk of 30 kbp 2232 -> 1107 us, 64 rings of 500 bp 3435 ->
-// 1146 us, melting 16 x 1000 bp 1807 -> 730 us; 50 FP64 steps of 200 bp 3722
-// -> 1154 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
+// 677 us, periodic walk of 30 kbp 2232 -> 1117 us, 64 rings of 500 bp 3435 ->
+// 1151 us, melting 16 x 1000 bp 1807 -> 739 us; 50 FP64 steps of 200 bp 3722
+// -> 1188 us (a warp per SM instead of eight sharing one SM's FP64 pipe).
 //
-// A 200 bp FP64 step is 42,000 cycles: 27,000 for one pass of an owner's terms
-// (a chain of FP64 latencies), 3500 to gather forces, 9400 to update.  Dealing
-// the FP64 work in groups of few lanes over all schedulers was slower (24 -> 38
-// us): the pipe is shared by the SM and timed by warp instructions.
+// Cycles of a step by clock stamps on every CTA (profiles/resident_kernel.md):
+// 10 kbp 6800 (3800 until all forces and the agreement are there, 2850 to gather
+// and update) and 20,000 per rebuild; 200 bp in FP64 40,900 (27,500 for one pass
+// of the owners' terms, 13,400 to gather and update).  Dealing the FP64 work in
+// groups of few lanes over all schedulers was slower (24 -> 38 us).
 #pragma once
 #include "../../include/dsdna.h"
 #include "cell_heads.h"
